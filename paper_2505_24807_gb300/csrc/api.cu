@@ -85,6 +85,7 @@ void invalidate_mixed(DevMol& m) {
   m.CTf_hi.release();
   m.CTf_lo.release();
   m.CTf.release();
+  m.mg_orb.reset();
 }
 
 }  // namespace

@@ -89,6 +89,7 @@ struct DevMol {
   DevBuf<double> eps;     // n orbital energies
   DevBuf<float> CTf_hi, CTf_lo;  // TF32-pair operand copies of CT for the tensor-core path
   DevBuf<float> CTf;             // float32 copy of CT for the float32 SIMT products
+  std::shared_ptr<void> mg_orb;  // residue operands of the orbitals for the float64 products (products.cu)
   DevBuf<double> dip;            // MO dipole integrals <i|r_x|a>, 3 x nocc x nvir (lazily)
   DevBuf<int> gb_rows, gb_cols;  // atom-aligned G tiles (first AO, count, first atom, end atom)
   int gb_nrows = 0, gb_ncols = 0;
@@ -118,6 +119,7 @@ struct Ctx {
   DevBuf<float> fs0, fs1, fs2;
   Profiler prof;
   DevBuf<int> tc_err;   // error word of the tensor-core kernels' bounded waits
+  std::shared_ptr<void> mg_work;    // scratch of the residue products (modgemm.h)
   std::shared_ptr<void> dav_cache;  // Davidson workspace kept between solves (davidson.cu)
   std::shared_ptr<void> batch_cache;  // lock-step batched solver's arenas (batch.cu)
   // batched solves: worker contexts (own stream and scratch), reused across calls

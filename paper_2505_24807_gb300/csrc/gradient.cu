@@ -524,6 +524,7 @@ void parameter_gradient(Ctx& c, DevMol& m, int root, double* grad_host, int* cg_
     XS_CHECK_LAUNCH();
     rz = rz_new;
   }
+  check_device_error(c);
   if (it >= 500) throw Error(XS_ENOCONV, "adjoint (A+B) Z = L solve did not converge");
   if (cg_iterations) *cg_iterations = it;
   // relaxed difference density P = Delta - sym(C_occ Z C_vir^T)

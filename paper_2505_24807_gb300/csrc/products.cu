@@ -6,8 +6,14 @@
 // For TDHF one G build gives G+ and G- and two back-transforms give (A+B)X and
 // (A-B)X.  The two transforms contract the smaller of nocc and nvir against
 // n^2 last.  Batches of vectors share each GEMM (the vectors are stacked into
-// one tall operand where the shared factor is on the right).
+// one tall operand where the shared factor is on the right).  In float64 the
+// transforms of all but small molecules are residue products on the tensor
+// cores (modgemm.h; rule and figures at mg_applies), the others run on the
+// float64 pipe.
+#include <algorithm>
+
 #include "kernels.h"
+#include "modgemm.h"
 #include "products.h"
 #include "tc.h"
 
@@ -47,6 +53,110 @@ void backtransform(cudaStream_t s, int n, int o, int v, int nvec, const T* CT, c
   }
 }
 
+// Residue operands of the orbitals (modgemm.h), made on first use and kept with
+// the molecule until its orbitals change, like the mixed path's TF32 pairs:
+// C_occ (n x o) and C_vir (n x v) of the P build, C_vir^T (v x n) and C_occ^T
+// (o x n) of the back-transform.
+struct MgOrbitals {
+  MgPlanes s_occ, s_vir, s_virT, s_occT;
+  MgOperand occ, vir, virT, occT;
+};
+
+// bytes of residue planes (operands and result) that one context holds at most
+// beyond a single vector's; larger batches run in chunks
+constexpr double kMgBytes = 1.5e9;
+
+// Where the residue products run: from 160 AOs up, and from 96 AOs up when the
+// batch gives them work.  Four products cost the residue path 105-115 us in
+// kernels whatever their size (16 launches) and the float64 pipe 55 us at 62
+// AOs, so the line is where they meet; kernel time of the four products of A X,
+// pipe -> residues: 62 AOs, 20 vectors 61 -> 125 us; 134 AOs, 8 vectors (54 MFLOP)
+// 116 -> 128, 16 vectors (108 MFLOP) 170 -> 158; 178 AOs, 1 vector 118 -> 122,
+// 4 vectors 131 -> 127; 222 AOs, 1 vector 133 -> 123; 579 AOs, 20 vectors
+// 9932 -> 807 us.
+bool mg_applies(const DevMol& m, int nvec) {
+  const double n = m.n, o = m.o, v = m.v;
+  if (m.v > m.o || m.n < 96 || m.n > kMgMaxK) return false;
+  return m.n >= 160 || 4.0 * nvec * (n * o * v + n * n * v) >= 8e7;
+}
+
+// operands and scratch for the residue products of `chunk` vectors, or null
+// where they do not fit the device (the float64-pipe path serves those)
+MgOrbitals* mg_prepare(Ctx& c, DevMol& m, int chunk) {
+  const int n = m.n, o = m.o, v = m.v;
+  cudaStream_t s = c.stream;
+  try {
+    if (!c.mg_work) c.mg_work = std::make_shared<MgWork>();
+    MgWork& w = *static_cast<MgWork*>(c.mg_work.get());
+    w.a.planes.ensure(mg_plane_count(n, v, chunk));
+    w.a.exps.ensure((size_t)chunk * n);
+    w.b.planes.ensure(std::max(mg_plane_count(n, n, chunk), mg_plane_count(v, o, chunk)));
+    w.b.exps.ensure((size_t)chunk * n);
+    w.res.ensure((size_t)kModuli * chunk * n * mg_ldn(n));
+    if (!c.tc_err.get()) {
+      c.tc_err.alloc(1);
+      XS_CUDA(cudaMemsetAsync(c.tc_err.get(), 0, sizeof(int), s));
+    }
+    if (!m.mg_orb) {
+      auto q = std::make_shared<MgOrbitals>();
+      const double* occ = m.CT.get();
+      const double* vir = occ + (size_t)o * n;
+      // C[mu][p] = CT[p][mu]: rows along mu are contiguous, K strided
+      q->occ = MgOperand{occ, 1, n, 0, n, o, 1};
+      q->vir = MgOperand{vir, 1, n, 0, n, v, 1};
+      q->virT = MgOperand{vir, n, 1, 0, v, n, 1};
+      q->occT = MgOperand{occ, n, 1, 0, o, n, 1};
+      mg_split(s, 0, q->occ, q->s_occ);
+      mg_split(s, 1, q->vir, q->s_vir);
+      mg_split(s, 0, q->virT, q->s_virT);
+      mg_split(s, 0, q->occT, q->s_occT);
+      m.mg_orb = q;
+    }
+    return static_cast<MgOrbitals*>(m.mg_orb.get());
+  } catch (const Error& e) {
+    if (e.status != XS_ENOMEM) throw;
+    cudaGetLastError();
+    c.mg_work.reset();
+    return nullptr;
+  }
+}
+
+// R (nvec x n x n) = C_occ X C_vir^T by residue products: W = C_occ X (n x v,
+// right operand X^T), then R = W C_vir^T
+void mg_pbuild(Ctx& c, const DevMol& m, const MgOrbitals& q, int nvec, const double* X, double* R, double* tmp) {
+  cudaStream_t s = c.stream;
+  MgWork& w = *static_cast<MgWork*>(c.mg_work.get());
+  const int n = m.n, o = m.o, v = m.v;
+  MgOperand x{X, 1, v, (long long)o * v, v, o, nvec};
+  mg_split(s, 1, x, w.b);
+  MgOut out;
+  out.C = tmp; out.ldc = v; out.sC = (long long)n * v;
+  mg_product(s, q.occ, x, nvec, out, w, c.tc_err.get());
+  MgOperand t{tmp, v, 1, (long long)n * v, n, v, nvec};
+  mg_split(s, 0, t, w.a);
+  out.C = R; out.ldc = n; out.sC = (long long)n * n;
+  mg_product(s, t, q.vir, nvec, out, w, c.tc_err.get());
+}
+
+// Y (nvec x o x v) = C_occ^T G C_vir + (eps_a - eps_i) X by residue products:
+// S^T = C_vir^T G^T (v x n), Y = C_occ^T S
+void mg_backtransform(Ctx& c, const DevMol& m, const MgOrbitals& q, int nvec, const double* G, const double* X,
+                      double* Y, double* tmp) {
+  cudaStream_t s = c.stream;
+  MgWork& w = *static_cast<MgWork*>(c.mg_work.get());
+  const int n = m.n, o = m.o, v = m.v;
+  MgOperand g{G, n, 1, (long long)n * n, n, n, nvec};
+  mg_split(s, 1, g, w.b);
+  MgOut out;
+  out.C = tmp; out.ldc = n; out.sC = (long long)v * n;
+  mg_product(s, q.virT, g, nvec, out, w, c.tc_err.get());
+  MgOperand t{tmp, n, 1, (long long)v * n, v, n, nvec};
+  mg_split(s, 1, t, w.b);
+  out.C = Y; out.ldc = v; out.sC = (long long)o * v;
+  out.X = X; out.eps = m.eps.get(); out.o = o;
+  mg_product(s, q.occT, t, nvec, out, w, c.tc_err.get());
+}
+
 }  // namespace
 
 int product_batch(const DevMol& m) {
@@ -58,13 +168,19 @@ int product_batch(const DevMol& m) {
   return nb;
 }
 
-void products_fp64(Ctx& c, const DevMol& m, int method, int nvec, const double* X, double* Y1, double* Y2,
-                   bool triplet) {
+void products_fp64(Ctx& c, DevMol& m, int method, int nvec, const double* X, double* Y1, double* Y2, bool triplet) {
   cudaStream_t s = c.stream;
   const int n = m.n, o = m.o, v = m.v;
   const long long ov = (long long)o * v, nn = (long long)n * n;
   const int nb = product_batch(m);
-  const int chunk = nvec < nb ? nvec : nb;
+  int chunk = nvec < nb ? nvec : nb;
+  MgOrbitals* q = nullptr;
+  if (mg_applies(m, nvec)) {
+    const double per = 2.0 * kModuli * n * (2.0 * mg_kp(n) + mg_kp(v));
+    const int mc = std::max(1, std::min(chunk, static_cast<int>(kMgBytes / per)));
+    q = mg_prepare(c, m, mc);
+    if (q) chunk = mc;
+  }
   c.ws1.ensure((size_t)chunk * nn);                         // R
   c.ws2.ensure((size_t)chunk * nn);                         // G or G+
   c.ws3.ensure((size_t)chunk * nn);                         // G-
@@ -72,6 +188,15 @@ void products_fp64(Ctx& c, const DevMol& m, int method, int nvec, const double* 
   for (int k0 = 0; k0 < nvec; k0 += chunk) {
     const int k = (nvec - k0) < chunk ? (nvec - k0) : chunk;
     const double* Xk = X + k0 * ov;
+    if (q) {
+      const bool rpa = method != XS_CIS;
+      mg_pbuild(c, m, *q, k, Xk, c.ws1.get(), c.ws4.get());
+      gbuild<double>(s, m, c.d_par.get(), gmode(rpa, triplet), k, c.ws1.get(), c.ws2.get(),
+                     rpa ? c.ws3.get() : nullptr, c.ws0);
+      mg_backtransform(c, m, *q, k, c.ws2.get(), Xk, Y1 + k0 * ov, c.ws4.get());
+      if (rpa) mg_backtransform(c, m, *q, k, c.ws3.get(), Xk, Y2 + k0 * ov, c.ws4.get());
+      continue;
+    }
     pbuild<double>(s, n, o, v, k, m.CT.get(), Xk, c.ws1.get(), c.ws4.get());
     if (method == XS_CIS) {
       gbuild<double>(s, m, c.d_par.get(), gmode(false, triplet), k, c.ws1.get(), c.ws2.get(), nullptr, c.ws0);

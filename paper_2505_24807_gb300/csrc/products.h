@@ -16,7 +16,7 @@ constexpr int kPrecF32 = 2;
 // digit split of the Davidson subspace needs it).
 void products(Ctx& c, DevMol& m, int method, int precision, int nvec, const double* X, double* Y1, double* Y2,
               bool triplet = false, unsigned int* mx1 = nullptr, unsigned int* mx2 = nullptr);
-void products_fp64(Ctx& c, const DevMol& m, int method, int nvec, const double* X, double* Y1, double* Y2,
+void products_fp64(Ctx& c, DevMol& m, int method, int nvec, const double* X, double* Y1, double* Y2,
                    bool triplet = false);
 // G_CIS(R) of nvec AO matrices (float64 device arrays)
 void gmatrix(Ctx& c, const DevMol& m, int precision, int nvec, const double* R, double* G);
