@@ -273,18 +273,13 @@ int xs_apply(xs_ctx* ctx, int mol, int kind, int nvec, const double* in, double*
     } else if (kind == XS_KIND_A || kind == XS_KIND_APB || kind == XS_KIND_AMB || kind == XS_KIND_A_TRIPLET ||
                kind == XS_KIND_APB_TRIPLET) {
       const bool triplet = kind == XS_KIND_A_TRIPLET || kind == XS_KIND_APB_TRIPLET;
-      DevBuf<double> X((size_t)nvec * ov), Y1((size_t)nvec * ov), Y2;
+      DevBuf<double> X((size_t)nvec * ov), Y((size_t)nvec * ov);
       copy_any(s, X.get(), in, sizeof(double) * nvec * ov);
-      if (kind == XS_KIND_A || kind == XS_KIND_A_TRIPLET) {
-        xs::products(c, m, XS_CIS, precision, nvec, X.get(), Y1.get(), nullptr, triplet);
-        xs::check_device_error(c);
-        copy_any(s, out, Y1.get(), sizeof(double) * nvec * ov);
-      } else {
-        Y2.alloc((size_t)nvec * ov);
-        xs::products(c, m, XS_TDHF, precision, nvec, X.get(), Y1.get(), Y2.get(), triplet);
-        xs::check_device_error(c);
-        copy_any(s, out, (kind == XS_KIND_AMB ? Y2 : Y1).get(), sizeof(double) * nvec * ov);
-      }
+      const bool cis = kind == XS_KIND_A || kind == XS_KIND_A_TRIPLET, minus = kind == XS_KIND_AMB;
+      xs::products(c, m, cis ? XS_CIS : XS_TDHF, precision, nvec, X.get(), minus ? nullptr : Y.get(),
+                   minus ? Y.get() : nullptr, triplet);
+      xs::check_device_error(c);
+      copy_any(s, out, Y.get(), sizeof(double) * nvec * ov);
     } else {
       throw Error(XS_EINVAL, "unknown product kind");
     }

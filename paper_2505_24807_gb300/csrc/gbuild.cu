@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(256, 4) gtile_kernel(int n, int np, int nvec, 
           if (kRpa) gm = -(K1ab - K1ba);
         } else {
           const int pab = (nA == 4) ? pidx(a, b) : 0;
-          const T J = J1 + J2[(long long)(PA + pab) * nvec + v];
+          const T J = J1 + (J2 ? J2[(long long)(PA + pab) * nvec + v] : T(0));
           if (!kRpa) {
             g = T(2) * J - K1ab;
           } else {
@@ -233,16 +233,18 @@ __global__ void __launch_bounds__(256, 4) gtile_kernel(int n, int np, int nvec, 
         const long long at = (long long)v * n * out.ldo + (long long)mu * out.ldo + lam;
         float h, l;
         tf32_pair(static_cast<float>(g), h, l);
-        out.Gh[at] = h;
-        out.Gl[at] = l;
-        if (kRpa) {
+        if (!kRpa || out.Gh) {
+          out.Gh[at] = h;
+          out.Gl[at] = l;
+        }
+        if (kRpa && out.Gmh) {
           tf32_pair(static_cast<float>(gm), h, l);
           out.Gmh[at] = h;
           out.Gml[at] = l;
         }
       } else {
-        out.G[v * nn + at_r] = g;
-        if (kRpa) out.Gm[v * nn + at_r] = gm;
+        if (!kRpa || out.G) out.G[v * nn + at_r] = g;
+        if (kRpa && out.Gm) out.Gm[v * nn + at_r] = gm;
       }
     }
     if (v0 + GV < nvec) {
@@ -281,7 +283,6 @@ void launch_tiles(cudaStream_t s, const DevMol& m, const double* d_par, GMode mo
 }
 
 inline bool has_coulomb(GMode mode) { return mode == G_CIS || mode == G_RPA; }
-inline bool has_minus(GMode mode) { return mode == G_RPA || mode == G_RPA_T; }
 
 // zero columns [n, ldo) of rows x ldo matrices (batch stride rows * ldo)
 __global__ void zero_pad_cols_kernel(int rows, int n, int ldo, int nvec, float* a, float* b) {
@@ -307,7 +308,8 @@ void gbuild(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, in
   const T* W = nullptr;
   if constexpr (sizeof(T) == 8) W = reinterpret_cast<const T*>(m.W.get());
   else W = reinterpret_cast<const T*>(m.Wf.get());
-  if (has_coulomb(mode)) {
+  const bool coulomb = has_coulomb(mode) && G;   // G- has no Coulomb part
+  if (coulomb) {
     dim3 block(8, 32);
     dim3 grid((m.L.natoms + 31) / 32);
     if constexpr (sizeof(T) == 4) {
@@ -327,13 +329,13 @@ void gbuild(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, in
     }
   }
   // algorithmic traffic: read R, write G (and G-), read the pair integrals once
-  const double outs = has_minus(mode) ? 2.0 : 1.0;
+  const double outs = (G ? 1.0 : 0.0) + (Gm ? 1.0 : 0.0);
   ProfScope ps(s, sizeof(T) == 8 ? "gbuild_assemble_f64" : "gbuild_assemble_f32",
                sizeof(T) * ((double)nvec * n * n * (1.0 + outs) + (double)np * np), 0.0);
   if constexpr (sizeof(T) == 4)
-    gpair_build(s, m, d_par, mode, nvec, W, J2, nvec, R, G, Gm);
+    gpair_build(s, m, d_par, mode, nvec, W, coulomb ? J2 : nullptr, nvec, R, G, Gm);
   else
-    launch_tiles<T, false>(s, m, d_par, mode, nvec, W, J2, R, GOut<T>{G, Gm, nullptr, nullptr, nullptr, nullptr, 0});
+    launch_tiles<T, false>(s, m, d_par, mode, nvec, W, coulomb ? J2 : nullptr, R, GOut<T>{G, Gm, nullptr, nullptr, nullptr, nullptr, 0});
 }
 
 void gbuild_split(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const float* R,
@@ -345,7 +347,8 @@ void gbuild_split(cudaStream_t s, const DevMol& m, const double* d_par, GMode mo
   float* rT = ws.get();
   float* J2 = ws.get() + (size_t)np * nvec;
   const float* W = m.Wf.get();
-  if (has_coulomb(mode)) {
+  const bool coulomb = has_coulomb(mode) && Gh;
+  if (coulomb) {
     dim3 block(8, 32);
     dim3 grid((m.L.natoms + 31) / 32);
     pack_diag_kernel<float, false><<<grid, block, 0, s>>>(m.L.natoms, n, np, nvec, m.atom_ao_off.get(),
@@ -356,14 +359,14 @@ void gbuild_split(cudaStream_t s, const DevMol& m, const double* d_par, GMode mo
   }
   if (ldo > n) {
     const long long cnt = (long long)nvec * n * (ldo - n);
-    zero_pad_cols_kernel<<<grid1(cnt, 256), 256, 0, s>>>(n, n, ldo, nvec, Gh, Gl);
-    if (has_minus(mode)) zero_pad_cols_kernel<<<grid1(cnt, 256), 256, 0, s>>>(n, n, ldo, nvec, Gmh, Gml);
+    if (Gh) zero_pad_cols_kernel<<<grid1(cnt, 256), 256, 0, s>>>(n, n, ldo, nvec, Gh, Gl);
+    if (Gmh) zero_pad_cols_kernel<<<grid1(cnt, 256), 256, 0, s>>>(n, n, ldo, nvec, Gmh, Gml);
     XS_CHECK_LAUNCH();
   }
   // algorithmic traffic: read R, write the G (and G-) TF32 pairs, read the pair integrals once
-  const double outs = has_minus(mode) ? 2.0 : 1.0;
+  const double outs = (Gh ? 1.0 : 0.0) + (Gmh ? 1.0 : 0.0);
   ProfScope ps(s, "gbuild_assemble_f32", 4.0 * ((double)nvec * n * n * (1.0 + 2.0 * outs) + (double)np * np), 0.0);
-  gpair_build_split(s, m, d_par, mode, nvec, W, J2, nvec, R, Gh, Gl, Gmh, Gml, ldo);
+  gpair_build_split(s, m, d_par, mode, nvec, W, coulomb ? J2 : nullptr, nvec, R, Gh, Gl, Gmh, Gml, ldo);
 }
 
 template <typename T>

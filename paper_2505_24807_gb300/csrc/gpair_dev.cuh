@@ -26,6 +26,7 @@ __device__ __forceinline__ void tf32_split(float x, float& hi, float& lo) {
   lo = __uint_as_float((__float_as_uint(x - hi) + 0x1000u) & 0xFFFFE000u);
 }
 
+// G+ or G- of the TDHF modes may be null: that output is not stored
 struct PairOut {
   float *G, *Gm;                 // plain outputs (row stride n)
   float *Gh, *Gl, *Gmh, *Gml;    // TF32 pairs (row stride ldo)
@@ -38,17 +39,19 @@ __device__ __forceinline__ void put(const PairOut& o, int n, long long vb, int r
     const long long at = vb * o.ldo + (long long)row * o.ldo + col;
     float h, l;
     tf32_split(g, h, l);
-    o.Gh[at] = h;
-    o.Gl[at] = l;
-    if (RPA) {
+    if (!RPA || o.Gh) {
+      o.Gh[at] = h;
+      o.Gl[at] = l;
+    }
+    if (RPA && o.Gmh) {
       tf32_split(gm, h, l);
       o.Gmh[at] = h;
       o.Gml[at] = l;
     }
   } else {
     const long long at = vb * n + (long long)row * n + col;
-    o.G[at] = g;
-    if (RPA) o.Gm[at] = gm;
+    if (!RPA || o.G) o.G[at] = g;
+    if (RPA && o.Gm) o.Gm[at] = gm;
   }
 }
 
@@ -186,8 +189,10 @@ __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, co
         g[lam] = kRpa ? -(Kij[mu][lam] + Kji[lam][mu]) : -Kij[mu][lam];
         q[lam] = -(Kij[mu][lam] - Kji[lam][mu]);
       }
-      put_row<SPLIT>(G0 + vb + out_ij, G1 + vb + out_ij, G1 ? G1 + vb + out_ij : nullptr, ldo, mu, 0, nJ, vout_ij, g);
-      if (kRpa) put_row<SPLIT>(M0 + vb + out_ij, M1 ? M1 + vb + out_ij : nullptr, M1 ? M1 + vb + out_ij : nullptr,
+      if (!kRpa || G0)
+        put_row<SPLIT>(G0 + vb + out_ij, G1 ? G1 + vb + out_ij : nullptr, G1 ? G1 + vb + out_ij : nullptr, ldo, mu, 0,
+                       nJ, vout_ij, g);
+      if (kRpa && M0) put_row<SPLIT>(M0 + vb + out_ij, M1 ? M1 + vb + out_ij : nullptr, M1 ? M1 + vb + out_ij : nullptr,
                                ldo, mu, 0, nJ, vout_ij, q);
     }
 #pragma unroll
@@ -199,9 +204,10 @@ __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, co
         g[mu] = kRpa ? -(Kij[mu][lam] + Kji[lam][mu]) : -Kji[lam][mu];
         q[mu] = Kij[mu][lam] - Kji[lam][mu];
       }
-      put_row<SPLIT>(G0 + vb + out_ji, G1 ? G1 + vb + out_ji : nullptr, G1 ? G1 + vb + out_ji : nullptr, ldo, lam, 0,
-                     nI, vout_ji, g);
-      if (kRpa) put_row<SPLIT>(M0 + vb + out_ji, M1 ? M1 + vb + out_ji : nullptr, M1 ? M1 + vb + out_ji : nullptr,
+      if (!kRpa || G0)
+        put_row<SPLIT>(G0 + vb + out_ji, G1 ? G1 + vb + out_ji : nullptr, G1 ? G1 + vb + out_ji : nullptr, ldo, lam, 0,
+                       nI, vout_ji, g);
+      if (kRpa && M0) put_row<SPLIT>(M0 + vb + out_ji, M1 ? M1 + vb + out_ji : nullptr, M1 ? M1 + vb + out_ji : nullptr,
                                ldo, lam, 0, nI, vout_ji, q);
     }
     if (v + 1 < nvec) {
@@ -248,7 +254,7 @@ __device__ __forceinline__ void diag_block(int n, int np, int nvec, int4 I, cons
             g = kRpa ? -(K1ab + K1ba) : -K1ab;
             if (kRpa) gm = -(K1ab - K1ba);
           } else {
-            const float J = J1 + J2[(long long)(I.z + pidx(a, b)) * ldj + v];
+            const float J = J1 + (J2 ? J2[(long long)(I.z + pidx(a, b)) * ldj + v] : 0.0f);
             if (!kRpa) {
               g = 2.0f * J - K1ab;
             } else {
@@ -286,7 +292,7 @@ __device__ __forceinline__ void diag_block(int n, int np, int nvec, int4 I, cons
           if (kTriplet) {
             g = kRpa ? -2.0f * k1 : -k1;
           } else {
-            const float J = k1 + J2[(long long)(I.z + i) * ldj + v];
+            const float J = k1 + (J2 ? J2[(long long)(I.z + i) * ldj + v] : 0.0f);
             g = kRpa ? 4.0f * J - 2.0f * k1 : 2.0f * J - k1;
           }
         } else {

@@ -453,7 +453,7 @@ void parameter_gradient(Ctx& c, DevMol& m, int root, double* grad_host, int* cg_
   const double* Y2 = rpa ? m.Wv.get() + (size_t)root * ov : nullptr;
   DevBuf<double> R(nn), R2(rpa ? nn : 1), Q(nn), GR(nn), Dl(nn), GD(nn), Dh(nn), tmp((size_t)n * std::max(o, v)),
       Gvv((size_t)v * v), Goo((size_t)o * o), T((size_t)std::max(o, v) * std::max(o, v)), L(ov), Z(ov), r(ov), zv(ov),
-      p(ov), Ap(ov), Am(ov), RZ(nn), P(nn), pk((size_t)3 * m.np), grad((size_t)XS_NELEM * XS_NPARAM), part;
+      p(ov), Ap(ov), RZ(nn), P(nn), pk((size_t)3 * m.np), grad((size_t)XS_NELEM * XS_NPARAM), part;
   DevBuf<double> ws;
   auto transition = [&](const double* Y, double* out) {   // C_occ Y C_vir^T
     gemm<double>(s, true, false, n, v, o, 1.0, CTocc, n, 0, Y, v, 0, 0.0, tmp.get(), v, 0, 1);
@@ -497,7 +497,7 @@ void parameter_gradient(Ctx& c, DevMol& m, int root, double* grad_host, int* cg_
   const int gb = static_cast<int>((ov + 255) / 256);
   diag_solve_kernel<<<gb, 256, 0, s>>>(o, v, m.eps.get(), L.get(), Z.get());
   XS_CHECK_LAUNCH();
-  products(c, m, XS_TDHF, XS_FP64, 1, Z.get(), Ap.get(), Am.get(), false);
+  products(c, m, XS_TDHF, XS_FP64, 1, Z.get(), Ap.get(), nullptr, false);
   XS_CUDA(cudaMemcpyAsync(r.get(), L.get(), sizeof(double) * ov, cudaMemcpyDeviceToDevice, s));
   axpby_kernel<<<gb, 256, 0, s>>>(ov, -1.0, Ap.get(), 1.0, r.get());
   XS_CHECK_LAUNCH();
@@ -510,7 +510,7 @@ void parameter_gradient(Ctx& c, DevMol& m, int root, double* grad_host, int* cg_
   for (; it < 500; ++it) {
     const double rn = std::sqrt(dot(s, ov, r.get(), r.get(), part));
     if (!(rn > 1e-11 * bnorm)) break;
-    products(c, m, XS_TDHF, XS_FP64, 1, p.get(), Ap.get(), Am.get(), false);
+    products(c, m, XS_TDHF, XS_FP64, 1, p.get(), Ap.get(), nullptr, false);
     const double pAp = dot(s, ov, p.get(), Ap.get(), part);
     if (!(pAp > 0.0)) throw Error(XS_EUNSTABLE, "A + B is not positive definite: unstable reference");
     const double alpha = rz / pAp;

@@ -40,13 +40,15 @@ inline GMode gmode(bool rpa, bool triplet) {
 }
 // nvec AO matrices R (n x n each, row-major, consecutive) -> G (CIS/Fock:
 // 2J(R) - K(R)) or G+ = 4J(Rs) - 2K(Rs) and G- = -2K(Ra) (RPA).
-// Gm is unused for G_CIS.  ws: scratch of at least 2 * np * nvec.
+// Gm is unused for G_CIS; in the TDHF modes either output may be null (not
+// formed).  ws: scratch of at least 2 * np * nvec.
 template <typename T>
 void gbuild(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const T* R,
             T* G, T* Gm, DevBuf<T>& ws);
 // Float32 G build whose output is the TF32 pair (hi, lo) of G (and G- for
 // TDHF) with row stride ldo >= n (batch stride n * ldo, columns n..ldo-1
 // zeroed): the back-transform's tensor-core operand without a separate split.
+// In the TDHF modes either pair may be null.
 void gbuild_split(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const float* R,
                   float* Gh, float* Gl, float* Gmh, float* Gml, int ldo, DevBuf<float>& ws);
 // Atom-aligned tiling of G used by gbuild (rows: one heavy atom or up to 4

@@ -182,8 +182,15 @@ void products_fp64(Ctx& c, DevMol& m, int method, int nvec, const double* X, dou
     if (q) chunk = mc;
   }
   c.ws1.ensure((size_t)chunk * nn);                         // R
-  c.ws2.ensure((size_t)chunk * nn);                         // G or G+
-  c.ws3.ensure((size_t)chunk * nn);                         // G-
+  double *G = nullptr, *Gm = nullptr;                       // G or G+, G-
+  if (Y1) {
+    c.ws2.ensure((size_t)chunk * nn);
+    G = c.ws2.get();
+  }
+  if (method != XS_CIS && Y2) {
+    c.ws3.ensure((size_t)chunk * nn);
+    Gm = c.ws3.get();
+  }
   c.ws4.ensure((size_t)chunk * n * (o > v ? o : v));        // transform scratch
   for (int k0 = 0; k0 < nvec; k0 += chunk) {
     const int k = (nvec - k0) < chunk ? (nvec - k0) : chunk;
@@ -191,22 +198,19 @@ void products_fp64(Ctx& c, DevMol& m, int method, int nvec, const double* X, dou
     if (q) {
       const bool rpa = method != XS_CIS;
       mg_pbuild(c, m, *q, k, Xk, c.ws1.get(), c.ws4.get());
-      gbuild<double>(s, m, c.d_par.get(), gmode(rpa, triplet), k, c.ws1.get(), c.ws2.get(),
-                     rpa ? c.ws3.get() : nullptr, c.ws0);
-      mg_backtransform(c, m, *q, k, c.ws2.get(), Xk, Y1 + k0 * ov, c.ws4.get());
-      if (rpa) mg_backtransform(c, m, *q, k, c.ws3.get(), Xk, Y2 + k0 * ov, c.ws4.get());
+      gbuild<double>(s, m, c.d_par.get(), gmode(rpa, triplet), k, c.ws1.get(), G, Gm, c.ws0);
+      if (Y1) mg_backtransform(c, m, *q, k, G, Xk, Y1 + k0 * ov, c.ws4.get());
+      if (Gm) mg_backtransform(c, m, *q, k, Gm, Xk, Y2 + k0 * ov, c.ws4.get());
       continue;
     }
     pbuild<double>(s, n, o, v, k, m.CT.get(), Xk, c.ws1.get(), c.ws4.get());
-    if (method == XS_CIS) {
-      gbuild<double>(s, m, c.d_par.get(), gmode(false, triplet), k, c.ws1.get(), c.ws2.get(), nullptr, c.ws0);
-      backtransform<double>(s, n, o, v, k, m.CT.get(), c.ws2.get(), Y1 + k0 * ov, c.ws4.get());
+    gbuild<double>(s, m, c.d_par.get(), gmode(method != XS_CIS, triplet), k, c.ws1.get(), G, Gm, c.ws0);
+    if (Y1) {
+      backtransform<double>(s, n, o, v, k, m.CT.get(), G, Y1 + k0 * ov, c.ws4.get());
       add_diag_term<double>(s, k, o, v, m.eps.get(), Xk, Y1 + k0 * ov);
-    } else {
-      gbuild<double>(s, m, c.d_par.get(), gmode(true, triplet), k, c.ws1.get(), c.ws2.get(), c.ws3.get(), c.ws0);
-      backtransform<double>(s, n, o, v, k, m.CT.get(), c.ws2.get(), Y1 + k0 * ov, c.ws4.get());
-      add_diag_term<double>(s, k, o, v, m.eps.get(), Xk, Y1 + k0 * ov);
-      backtransform<double>(s, n, o, v, k, m.CT.get(), c.ws3.get(), Y2 + k0 * ov, c.ws4.get());
+    }
+    if (Gm) {
+      backtransform<double>(s, n, o, v, k, m.CT.get(), Gm, Y2 + k0 * ov, c.ws4.get());
       add_diag_term<double>(s, k, o, v, m.eps.get(), Xk, Y2 + k0 * ov);
     }
   }
@@ -243,8 +247,9 @@ void products_f32(Ctx& c, DevMol& m, int method, int nvec, const double* X, doub
     convert_d2f(s, k * ov, Xk, Xf);
     pbuild<float>(s, n, o, v, k, m.CTf.get(), Xf, R, tmp);
     const bool rpa = method != XS_CIS;
-    gbuild<float>(s, m, c.d_par.get(), gmode(rpa, triplet), k, R, G, rpa ? Gm : nullptr, c.fs1);
+    gbuild<float>(s, m, c.d_par.get(), gmode(rpa, triplet), k, R, Y1 ? G : nullptr, rpa && Y2 ? Gm : nullptr, c.fs1);
     for (int pass = 0; pass < (rpa ? 2 : 1); ++pass) {
+      if (!(pass == 0 ? Y1 : Y2)) continue;
       double* Y = (pass == 0 ? Y1 : Y2) + k0 * ov;
       backtransform<float>(s, n, o, v, k, m.CTf.get(), pass == 0 ? G : Gm, Yf, tmp);
       convert_f2d(s, k * ov, Yf, Y);

@@ -8,8 +8,9 @@ namespace xs {
 // internal precision code: float32 SIMT products (polish step of mixed solves)
 constexpr int kPrecF32 = 2;
 
-// Y1 = A X (CIS) or Y1 = (A+B) X, Y2 = (A-B) X (TDHF) for nvec vectors
-// X (nvec x nocc x nvir, float64, device).  precision: XS_FP64 or XS_MIXED.
+// Y1 = A X (CIS) or Y1 = (A+B) X, Y2 = (A-B) X (TDHF; either may be null: that
+// product's share of the G build and its back-transform are left out) for nvec
+// vectors X (nvec x nocc x nvir, float64, device).  precision: XS_FP64 or XS_MIXED.
 // triplet: the spin-adapted triplet matrices (no Coulomb terms in G).
 // mx1, mx2 (XS_MIXED only, else ignored): per output vector abs_hi of its
 // largest |y| (common.cuh), formed by the epilogue that writes Y1 / Y2 (the

@@ -69,18 +69,23 @@ void products_mixed(Ctx& c, DevMol& m, int method, int nvec, const double* X, do
   const size_t sU = up((size_t)chunk * n * (vfirst ? vp : op)), sR = up((size_t)chunk * nn);
   const size_t sG = up((size_t)chunk * n * np_), sS = up((size_t)chunk * v * np_);
   const bool rpa = method != XS_CIS;
-  c.fs0.ensure(2 * sX + 2 * sU + sR + (rpa ? 4 : 2) * sG + 2 * sS);
+  const bool plus = Y1 != nullptr, minus = rpa && Y2;   // products asked for
+  c.fs0.ensure(2 * sX + 2 * sU + sR + ((plus ? 2 : 0) + (minus ? 2 : 0)) * sG + 2 * sS);
   float* p = c.fs0.get();
   float* Xh = p; p += sX;
   float* Xl = p; p += sX;
   float* Uh = p; p += sU;
   float* Ul = p; p += sU;
   float* R = p; p += sR;
-  float* Gh = p; p += sG;     // TF32 pair of G (CIS) or G+ (TDHF)
-  float* Gl = p; p += sG;
+  float* Gh = nullptr;        // TF32 pair of G (CIS) or G+ (TDHF)
+  float* Gl = nullptr;
   float* Gmh = nullptr;       // TF32 pair of G- (TDHF)
   float* Gml = nullptr;
-  if (rpa) {
+  if (plus) {
+    Gh = p; p += sG;
+    Gl = p; p += sG;
+  }
+  if (minus) {
     Gmh = p; p += sG;
     Gml = p; p += sG;
   }
@@ -92,7 +97,7 @@ void products_mixed(Ctx& c, DevMol& m, int method, int nvec, const double* X, do
     XS_CUDA(cudaMemsetAsync(err.get(), 0, sizeof(int), s));
   }
   if (mx1) XS_CUDA(cudaMemsetAsync(mx1, 0, sizeof(unsigned int) * nvec, s));
-  if (mx2 && rpa) XS_CUDA(cudaMemsetAsync(mx2, 0, sizeof(unsigned int) * nvec, s));
+  if (mx2 && minus) XS_CUDA(cudaMemsetAsync(mx2, 0, sizeof(unsigned int) * nvec, s));
 
   for (int k0 = 0; k0 < nvec; k0 += chunk) {
     const int k = (nvec - k0) < chunk ? (nvec - k0) : chunk;
@@ -135,6 +140,7 @@ void products_mixed(Ctx& c, DevMol& m, int method, int nvec, const double* X, do
     for (int pass = 0; pass < (rpa ? 2 : 1); ++pass) {
       const float* Gph = pass == 0 ? Gh : Gmh;
       const float* Gpl = pass == 0 ? Gl : Gml;
+      if (!Gph) continue;
       double* Yout = (pass == 0 ? Y1 : Y2) + k0 * ov;
       unsigned int* mxo = pass == 0 ? mx1 : mx2;
       {  // S^T = C_vir^T G^T : M = v, N = n, K = n
