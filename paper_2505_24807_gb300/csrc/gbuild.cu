@@ -182,7 +182,7 @@ __global__ void __launch_bounds__(256, 4) gtile_kernel(int n, int np, int nvec, 
           if (kRpa) gm = -(K1ab - K1ba);
         } else {
           const int pab = (nA == 4) ? pidx(a, b) : 0;
-          const T J = J1 + (J2 ? J2[(long long)(PA + pab) * nvec + v] : T(0));
+          const T J = J1 + J2[(long long)(PA + pab) * nvec + v];
           if (!kRpa) {
             g = T(2) * J - K1ab;
           } else {
@@ -308,7 +308,7 @@ void gbuild(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, in
   const T* W = nullptr;
   if constexpr (sizeof(T) == 8) W = reinterpret_cast<const T*>(m.W.get());
   else W = reinterpret_cast<const T*>(m.Wf.get());
-  const bool coulomb = has_coulomb(mode) && G;   // G- has no Coulomb part
+  const bool coulomb = has_coulomb(mode) && G;   // G- has no Coulomb part (J2 is then not formed, G not stored)
   if (coulomb) {
     dim3 block(8, 32);
     dim3 grid((m.L.natoms + 31) / 32);
@@ -333,9 +333,9 @@ void gbuild(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, in
   ProfScope ps(s, sizeof(T) == 8 ? "gbuild_assemble_f64" : "gbuild_assemble_f32",
                sizeof(T) * ((double)nvec * n * n * (1.0 + outs) + (double)np * np), 0.0);
   if constexpr (sizeof(T) == 4)
-    gpair_build(s, m, d_par, mode, nvec, W, coulomb ? J2 : nullptr, nvec, R, G, Gm);
+    gpair_build(s, m, d_par, mode, nvec, W, J2, nvec, R, G, Gm);
   else
-    launch_tiles<T, false>(s, m, d_par, mode, nvec, W, coulomb ? J2 : nullptr, R, GOut<T>{G, Gm, nullptr, nullptr, nullptr, nullptr, 0});
+    launch_tiles<T, false>(s, m, d_par, mode, nvec, W, J2, R, GOut<T>{G, Gm, nullptr, nullptr, nullptr, nullptr, 0});
 }
 
 void gbuild_split(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const float* R,
@@ -366,7 +366,7 @@ void gbuild_split(cudaStream_t s, const DevMol& m, const double* d_par, GMode mo
   // algorithmic traffic: read R, write the G (and G-) TF32 pairs, read the pair integrals once
   const double outs = (Gh ? 1.0 : 0.0) + (Gmh ? 1.0 : 0.0);
   ProfScope ps(s, "gbuild_assemble_f32", 4.0 * ((double)nvec * n * n * (1.0 + 2.0 * outs) + (double)np * np), 0.0);
-  gpair_build_split(s, m, d_par, mode, nvec, W, coulomb ? J2 : nullptr, nvec, R, Gh, Gl, Gmh, Gml, ldo);
+  gpair_build_split(s, m, d_par, mode, nvec, W, J2, nvec, R, Gh, Gl, Gmh, Gml, ldo);
 }
 
 template <typename T>

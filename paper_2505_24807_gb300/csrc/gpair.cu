@@ -33,7 +33,7 @@ namespace {
 
 constexpr int kPairThreads = 256;
 
-template <GMode MODE, bool SPLIT>
+template <GMode MODE, bool SPLIT, int OUT>
 __global__ void __launch_bounds__(kPairThreads, 2) gpair_kernel(int n, int np, int nvec, int npairs,
                                                                 const int2* __restrict__ pairs,
                                                                 const int4* __restrict__ sa,
@@ -44,42 +44,39 @@ __global__ void __launch_bounds__(kPairThreads, 2) gpair_kernel(int n, int np, i
   extern __shared__ float wsm[];   // 100 integrals per thread
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= npairs) return;
-  gpair_one<MODE, SPLIT>(n, np, nvec, pairs[t], sa, par, W, J2, ldj, R, o, wsm + threadIdx.x * 100);
+  gpair_one<MODE, SPLIT, OUT>(n, np, nvec, pairs[t], sa, par, W, J2, ldj, R, o, wsm + threadIdx.x * 100);
+}
+
+template <GMode MODE, bool SPLIT, int OUT>
+void launch_mode(cudaStream_t s, const DevMol& m, const double* d_par, int nvec, const float* W, const float* J2,
+                 int ldj, const float* R, const PairOut& o) {
+  const size_t smem = sizeof(float) * 100 * kPairThreads;
+  static const bool attr = [] {
+    XS_CUDA(cudaFuncSetAttribute(gpair_kernel<MODE, SPLIT, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 static_cast<int>(sizeof(float) * 100 * kPairThreads)));
+    return true;
+  }();
+  (void)attr;
+  const int npairs = m.gp_npairs;
+  gpair_kernel<MODE, SPLIT, OUT><<<(npairs + kPairThreads - 1) / kPairThreads, kPairThreads, smem, s>>>(
+      m.n, m.np, nvec, npairs, reinterpret_cast<const int2*>(m.gp_pairs.get()),
+      reinterpret_cast<const int4*>(m.gp_sa.get()), d_par, W, J2, ldj, R, o);
+  XS_CHECK_LAUNCH();
 }
 
 template <bool SPLIT>
 void launch_pairs(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const float* W,
                   const float* J2, int ldj, const float* R, const PairOut& o) {
-  const int np2 = m.gp_npairs;
-  const int2* pairs = reinterpret_cast<const int2*>(m.gp_pairs.get());
-  const int4* sa = reinterpret_cast<const int4*>(m.gp_sa.get());
-  const dim3 grid((np2 + kPairThreads - 1) / kPairThreads);
-  const size_t smem = sizeof(float) * 100 * kPairThreads;
-  static const bool attr = [] {
-    for (const void* f : {reinterpret_cast<const void*>(gpair_kernel<G_CIS, SPLIT>),
-                          reinterpret_cast<const void*>(gpair_kernel<G_RPA, SPLIT>),
-                          reinterpret_cast<const void*>(gpair_kernel<G_CIS_T, SPLIT>),
-                          reinterpret_cast<const void*>(gpair_kernel<G_RPA_T, SPLIT>)})
-      XS_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   static_cast<int>(sizeof(float) * 100 * kPairThreads)));
-    return true;
-  }();
-  (void)attr;
-  switch (mode) {
-    case G_CIS:
-      gpair_kernel<G_CIS, SPLIT><<<grid, kPairThreads, smem, s>>>(m.n, m.np, nvec, np2, pairs, sa, d_par, W, J2, ldj, R, o);
-      break;
-    case G_RPA:
-      gpair_kernel<G_RPA, SPLIT><<<grid, kPairThreads, smem, s>>>(m.n, m.np, nvec, np2, pairs, sa, d_par, W, J2, ldj, R, o);
-      break;
-    case G_CIS_T:
-      gpair_kernel<G_CIS_T, SPLIT><<<grid, kPairThreads, smem, s>>>(m.n, m.np, nvec, np2, pairs, sa, d_par, W, J2, ldj, R, o);
-      break;
-    default:
-      gpair_kernel<G_RPA_T, SPLIT><<<grid, kPairThreads, smem, s>>>(m.n, m.np, nvec, np2, pairs, sa, d_par, W, J2, ldj, R, o);
-      break;
-  }
-  XS_CHECK_LAUNCH();
+  const bool plus = SPLIT ? o.Gh != nullptr : o.G != nullptr, minus = SPLIT ? o.Gmh != nullptr : o.Gm != nullptr;
+#define XS_PAIRS(MODE, OUT) launch_mode<MODE, SPLIT, OUT>(s, m, d_par, nvec, W, J2, ldj, R, o)
+  if (mode == G_CIS) XS_PAIRS(G_CIS, kOutPlus);
+  else if (mode == G_CIS_T) XS_PAIRS(G_CIS_T, kOutPlus);
+  else if (mode == G_RPA && plus && minus) XS_PAIRS(G_RPA, kOutBoth);
+  else if (mode == G_RPA && plus) XS_PAIRS(G_RPA, kOutPlus);
+  else if (mode == G_RPA_T && plus && minus) XS_PAIRS(G_RPA_T, kOutBoth);
+  else if (mode == G_RPA_T && plus) XS_PAIRS(G_RPA_T, kOutPlus);
+  else XS_PAIRS(G_RPA_T, kOutMinus);   // G- = -K(R) + K(R^T) has no Coulomb part
+#undef XS_PAIRS
 }
 
 // Two-centre Coulomb of the diagonal blocks, J2 = W r (np x nvec, row

@@ -26,32 +26,34 @@ __device__ __forceinline__ void tf32_split(float x, float& hi, float& lo) {
   lo = __uint_as_float((__float_as_uint(x - hi) + 0x1000u) & 0xFFFFE000u);
 }
 
-// G+ or G- of the TDHF modes may be null: that output is not stored
+// Outputs of the TDHF modes to store (template parameter OUT): G+, G- or both
+constexpr int kOutPlus = 1, kOutMinus = 2, kOutBoth = 3;
+
 struct PairOut {
   float *G, *Gm;                 // plain outputs (row stride n)
   float *Gh, *Gl, *Gmh, *Gml;    // TF32 pairs (row stride ldo)
   int ldo;
 };
 
-template <bool SPLIT, bool RPA>
+template <bool SPLIT, bool RPA, int OUT>
 __device__ __forceinline__ void put(const PairOut& o, int n, long long vb, int row, int col, float g, float gm) {
   if (SPLIT) {
     const long long at = vb * o.ldo + (long long)row * o.ldo + col;
     float h, l;
-    tf32_split(g, h, l);
-    if (!RPA || o.Gh) {
+    if (!RPA || (OUT & kOutPlus)) {
+      tf32_split(g, h, l);
       o.Gh[at] = h;
       o.Gl[at] = l;
     }
-    if (RPA && o.Gmh) {
+    if (RPA && (OUT & kOutMinus)) {
       tf32_split(gm, h, l);
       o.Gmh[at] = h;
       o.Gml[at] = l;
     }
   } else {
     const long long at = vb * n + (long long)row * n + col;
-    if (!RPA || o.G) o.G[at] = g;
-    if (RPA && o.Gm) o.Gm[at] = gm;
+    if (!RPA || (OUT & kOutPlus)) o.G[at] = g;
+    if (RPA && (OUT & kOutMinus)) o.Gm[at] = gm;
   }
 }
 
@@ -138,10 +140,11 @@ __device__ __forceinline__ void put_row(float* A, float* B, float* unused, long 
   }
 }
 
-template <GMode MODE, bool SPLIT, bool HI, bool HJ>
+template <GMode MODE, bool SPLIT, int OUT, bool HI, bool HJ>
 __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, const float* __restrict__ R,
                                              const PairOut& o, const float* ws, int ldw) {
   constexpr bool kRpa = MODE == G_RPA || MODE == G_RPA_T;
+  constexpr bool kPlus = !kRpa || (OUT & kOutPlus), kMinus = kRpa && (OUT & kOutMinus);
   const int nI = sa_nao(I), nJ = sa_nao(J);
   const int ldo = SPLIT ? o.ldo : n;
   // 16-byte row segments: the block starts on a multiple of 4 AOs, is 4 wide
@@ -189,10 +192,8 @@ __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, co
         g[lam] = kRpa ? -(Kij[mu][lam] + Kji[lam][mu]) : -Kij[mu][lam];
         q[lam] = -(Kij[mu][lam] - Kji[lam][mu]);
       }
-      if (!kRpa || G0)
-        put_row<SPLIT>(G0 + vb + out_ij, G1 ? G1 + vb + out_ij : nullptr, G1 ? G1 + vb + out_ij : nullptr, ldo, mu, 0,
-                       nJ, vout_ij, g);
-      if (kRpa && M0) put_row<SPLIT>(M0 + vb + out_ij, M1 ? M1 + vb + out_ij : nullptr, M1 ? M1 + vb + out_ij : nullptr,
+      if (kPlus) put_row<SPLIT>(G0 + vb + out_ij, G1 + vb + out_ij, G1 ? G1 + vb + out_ij : nullptr, ldo, mu, 0, nJ, vout_ij, g);
+      if (kMinus) put_row<SPLIT>(M0 + vb + out_ij, M1 ? M1 + vb + out_ij : nullptr, M1 ? M1 + vb + out_ij : nullptr,
                                ldo, mu, 0, nJ, vout_ij, q);
     }
 #pragma unroll
@@ -204,10 +205,9 @@ __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, co
         g[mu] = kRpa ? -(Kij[mu][lam] + Kji[lam][mu]) : -Kji[lam][mu];
         q[mu] = Kij[mu][lam] - Kji[lam][mu];
       }
-      if (!kRpa || G0)
-        put_row<SPLIT>(G0 + vb + out_ji, G1 ? G1 + vb + out_ji : nullptr, G1 ? G1 + vb + out_ji : nullptr, ldo, lam, 0,
-                       nI, vout_ji, g);
-      if (kRpa && M0) put_row<SPLIT>(M0 + vb + out_ji, M1 ? M1 + vb + out_ji : nullptr, M1 ? M1 + vb + out_ji : nullptr,
+      if (kPlus) put_row<SPLIT>(G0 + vb + out_ji, G1 ? G1 + vb + out_ji : nullptr, G1 ? G1 + vb + out_ji : nullptr, ldo, lam, 0,
+                     nI, vout_ji, g);
+      if (kMinus) put_row<SPLIT>(M0 + vb + out_ji, M1 ? M1 + vb + out_ji : nullptr, M1 ? M1 + vb + out_ji : nullptr,
                                ldo, lam, 0, nI, vout_ji, q);
     }
     if (v + 1 < nvec) {
@@ -225,7 +225,7 @@ __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, co
 // diagonal block of a super-atom: one-centre Coulomb and exchange, the
 // two-centre Coulomb of the diagonal blocks (J2), and for a hydrogen run the
 // exchange between its hydrogens
-template <GMode MODE, bool SPLIT>
+template <GMode MODE, bool SPLIT, int OUT>
 __device__ __forceinline__ void diag_block(int n, int np, int nvec, int4 I, const double* __restrict__ par,
                                            const float* __restrict__ W, const float* __restrict__ J2, int ldj,
                                            const float* __restrict__ R, const PairOut& o) {
@@ -254,7 +254,7 @@ __device__ __forceinline__ void diag_block(int n, int np, int nvec, int4 I, cons
             g = kRpa ? -(K1ab + K1ba) : -K1ab;
             if (kRpa) gm = -(K1ab - K1ba);
           } else {
-            const float J = J1 + (J2 ? J2[(long long)(I.z + pidx(a, b)) * ldj + v] : 0.0f);
+            const float J = J1 + J2[(long long)(I.z + pidx(a, b)) * ldj + v];
             if (!kRpa) {
               g = 2.0f * J - K1ab;
             } else {
@@ -262,7 +262,7 @@ __device__ __forceinline__ void diag_block(int n, int np, int nvec, int4 I, cons
               gm = -(K1ab - K1ba);
             }
           }
-          put<SPLIT, kRpa>(o, n, v * (long long)n, I.x + a, I.x + b, g, gm);
+          put<SPLIT, kRpa, OUT>(o, n, v * (long long)n, I.x + a, I.x + b, g, gm);
         }
     }
     return;
@@ -292,7 +292,7 @@ __device__ __forceinline__ void diag_block(int n, int np, int nvec, int4 I, cons
           if (kTriplet) {
             g = kRpa ? -2.0f * k1 : -k1;
           } else {
-            const float J = k1 + (J2 ? J2[(long long)(I.z + i) * ldj + v] : 0.0f);
+            const float J = k1 + J2[(long long)(I.z + i) * ldj + v];
             g = kRpa ? 4.0f * J - 2.0f * k1 : 2.0f * J - k1;
           }
         } else {
@@ -300,14 +300,14 @@ __device__ __forceinline__ void diag_block(int n, int np, int nvec, int4 I, cons
           g = kRpa ? -(kr + krt) : -kr;
           gm = -(kr - krt);
         }
-        put<SPLIT, kRpa>(o, n, v * (long long)n, I.x + i, I.x + j, g, gm);
+        put<SPLIT, kRpa, OUT>(o, n, v * (long long)n, I.x + i, I.x + j, g, gm);
       }
   }
 }
 
 // One super-atom pair of the pair list, all nvec matrices; ws: 100 floats of
 // shared memory owned by the calling thread.
-template <GMode MODE, bool SPLIT>
+template <GMode MODE, bool SPLIT, int OUT = kOutBoth>
 __device__ __forceinline__ void gpair_one(int n, int np, int nvec, int2 pr, const int4* __restrict__ sa,
                                           const double* __restrict__ par, const float* __restrict__ W,
                                           const float* __restrict__ J2, int ldj, const float* __restrict__ R,
@@ -315,7 +315,7 @@ __device__ __forceinline__ void gpair_one(int n, int np, int nvec, int2 pr, cons
   if (pr.x < 0) return;
   const int4 I = sa[pr.x];
   if (pr.x == pr.y) {
-    diag_block<MODE, SPLIT>(n, np, nvec, I, par, W, J2, ldj, R, o);
+    diag_block<MODE, SPLIT, OUT>(n, np, nvec, I, par, W, J2, ldj, R, o);
     return;
   }
   const int4 J = sa[pr.y];
@@ -326,10 +326,10 @@ __device__ __forceinline__ void gpair_one(int n, int np, int nvec, int2 pr, cons
       ws[a * 10 + b] = (a < npI && b < npJ) ? __ldg(W + (long long)(I.z + a) * np + J.z + b) : 0.0f;
   const int kind = (hI ? 2 : 0) + (hJ ? 1 : 0);
   switch (kind) {
-    case 3: offdiag_pair<MODE, SPLIT, true, true>(n, nvec, I, J, R, o, ws, 10); break;
-    case 2: offdiag_pair<MODE, SPLIT, true, false>(n, nvec, I, J, R, o, ws, 10); break;
-    case 1: offdiag_pair<MODE, SPLIT, false, true>(n, nvec, I, J, R, o, ws, 10); break;
-    default: offdiag_pair<MODE, SPLIT, false, false>(n, nvec, I, J, R, o, ws, 10); break;
+    case 3: offdiag_pair<MODE, SPLIT, OUT, true, true>(n, nvec, I, J, R, o, ws, 10); break;
+    case 2: offdiag_pair<MODE, SPLIT, OUT, true, false>(n, nvec, I, J, R, o, ws, 10); break;
+    case 1: offdiag_pair<MODE, SPLIT, OUT, false, true>(n, nvec, I, J, R, o, ws, 10); break;
+    default: offdiag_pair<MODE, SPLIT, OUT, false, false>(n, nvec, I, J, R, o, ws, 10); break;
   }
 }
 
