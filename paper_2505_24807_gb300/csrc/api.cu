@@ -1,4 +1,7 @@
 // C ABI of libxs (declared and documented in include/xs.h).
+#include <cuda.h>
+#include <cudaTypedefs.h>
+
 #include <atomic>
 #include <chrono>
 #include <cmath>
@@ -34,6 +37,11 @@ int guarded(xs_ctx* ctx, F&& f) {
     XS_CUDA(cudaSetDevice(ctx->c.device));
     return f(ctx->c);
   } catch (const Error& e) {
+    if (e.status == XS_ENOMEM) {   // give back what is only kept for speed
+      ctx->c.io.release();
+      ctx->c.oz_work.reset();
+      ctx->c.mg_work.reset();
+    }
     ctx->c.err = e.what();
     return e.status;
   } catch (const std::bad_alloc&) {
@@ -62,6 +70,64 @@ void upload(cudaStream_t s, DevBuf<T>& d, const std::vector<T>& h) {
 void copy_any(cudaStream_t s, void* dst, const void* src, size_t bytes) {
   if (bytes == 0) return;
   XS_CUDA(cudaMemcpyAsync(dst, src, bytes, cudaMemcpyDefault, s));
+}
+
+// Whether the kernels may use the caller's array where it is: 16-byte aligned
+// memory of this device, all `bytes` of it inside one allocation.  Anything else
+// (host memory, another device, a short allocation) goes through a copy, which
+// reports what it cannot reach.
+bool on_device(const Ctx& c, const void* p, size_t bytes) {
+  if (reinterpret_cast<uintptr_t>(p) & 15) return false;
+  cudaPointerAttributes a;
+  if (cudaPointerGetAttributes(&a, p) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  if (a.type != cudaMemoryTypeDevice || a.device != c.device) return false;
+  static const PFN_cuMemGetAddressRange_v3020 range = [] {
+    void* f = nullptr;
+    cudaDriverEntryPointQueryResult q;
+    const bool ok = cudaGetDriverEntryPointByVersion("cuMemGetAddressRange", &f, 3020, cudaEnableDefault, &q) ==
+                        cudaSuccess && q == cudaDriverEntryPointSuccess;
+    return ok ? reinterpret_cast<PFN_cuMemGetAddressRange_v3020>(f) : nullptr;
+  }();
+  CUdeviceptr base = 0;
+  size_t size = 0;
+  if (!range || range(&base, &size, reinterpret_cast<CUdeviceptr>(p)) != CUDA_SUCCESS) return false;
+  return reinterpret_cast<CUdeviceptr>(p) + bytes <= base + size;
+}
+
+// count elements of an input: in place, or staged in a scratch slot
+const double* input(Ctx& c, int slot, const double* p, size_t count) {
+  const size_t bytes = sizeof(double) * count;
+  if (on_device(c, p, bytes)) return p;
+  void* d = c.io.get(slot, bytes);
+  copy_any(c.stream, d, p, bytes);
+  return static_cast<const double*>(d);
+}
+
+// room for an output: in place unless it overlaps the inputs, else a scratch
+// slot that finish() copies out
+struct Output {
+  double* user;
+  double* dev;
+  size_t bytes;
+};
+Output output(Ctx& c, int slot, double* p, size_t count, const double* in, size_t in_count) {
+  const size_t bytes = sizeof(double) * count;
+  const uintptr_t a = reinterpret_cast<uintptr_t>(p), b = reinterpret_cast<uintptr_t>(in);
+  const bool apart = a + bytes <= b || b + sizeof(double) * in_count <= a;
+  if (apart && on_device(c, p, bytes)) return {p, p, bytes};
+  return {p, static_cast<double*>(c.io.get(slot, bytes)), bytes};
+}
+void finish(Ctx& c, const Output& o) {
+  if (o.dev != o.user) copy_any(c.stream, o.user, o.dev, o.bytes);
+  XS_CUDA(cudaStreamSynchronize(c.stream));
+  c.io.trim();
+  if (c.oz_work) {
+    const xs::OzWork& w = *static_cast<xs::OzWork*>(c.oz_work.get());
+    if (sizeof(double) * w.part.n > xs::CallScratch::kKeep / 8) c.oz_work.reset();
+  }
 }
 
 // A worker context for batched solves: the parent's parameters, its own
@@ -165,6 +231,8 @@ int xs_ground_state(xs_ctx* ctx, int n_mol, const int* natoms, const int* Z, con
     if (!(scf_tol > 0.0)) scf_tol = 1e-10;
     if (max_iter <= 0) max_iter = 300;
     cudaStream_t s = c.stream;
+    c.io.release();
+    c.oz_work.reset();
     c.mols.clear();
     c.mols.resize(n_mol);
     int off = 0, maxit = 0;
@@ -263,27 +331,25 @@ int xs_apply(xs_ctx* ctx, int mol, int kind, int nvec, const double* in, double*
     if (nvec < 0 || (nvec > 0 && (!in || !out))) throw Error(XS_EINVAL, "bad vectors");
     if (precision != XS_FP64 && precision != XS_MIXED) throw Error(XS_EINVAL, "bad precision");
     if (nvec == 0) return XS_OK;
-    cudaStream_t s = c.stream;
     const long long ov = (long long)m.o * m.v, nn = (long long)m.n * m.n;
     if (kind == XS_KIND_G) {
-      DevBuf<double> R((size_t)nvec * nn), G((size_t)nvec * nn);
-      copy_any(s, R.get(), in, sizeof(double) * nvec * nn);
-      xs::gmatrix(c, m, precision, nvec, R.get(), G.get());
-      copy_any(s, out, G.get(), sizeof(double) * nvec * nn);
+      const double* R = input(c, 0, in, (size_t)nvec * nn);
+      const Output G = output(c, 1, out, (size_t)nvec * nn, in, (size_t)nvec * nn);
+      xs::gmatrix(c, m, precision, nvec, R, G.dev);
+      finish(c, G);
     } else if (kind == XS_KIND_A || kind == XS_KIND_APB || kind == XS_KIND_AMB || kind == XS_KIND_A_TRIPLET ||
                kind == XS_KIND_APB_TRIPLET) {
       const bool triplet = kind == XS_KIND_A_TRIPLET || kind == XS_KIND_APB_TRIPLET;
-      DevBuf<double> X((size_t)nvec * ov), Y((size_t)nvec * ov);
-      copy_any(s, X.get(), in, sizeof(double) * nvec * ov);
+      const double* X = input(c, 0, in, (size_t)nvec * ov);
+      const Output Y = output(c, 1, out, (size_t)nvec * ov, in, (size_t)nvec * ov);
       const bool cis = kind == XS_KIND_A || kind == XS_KIND_A_TRIPLET, minus = kind == XS_KIND_AMB;
-      xs::products(c, m, cis ? XS_CIS : XS_TDHF, precision, nvec, X.get(), minus ? nullptr : Y.get(),
-                   minus ? Y.get() : nullptr, triplet);
+      xs::products(c, m, cis ? XS_CIS : XS_TDHF, precision, nvec, X, minus ? nullptr : Y.dev,
+                   minus ? Y.dev : nullptr, triplet);
       xs::check_device_error(c);
-      copy_any(s, out, Y.get(), sizeof(double) * nvec * ov);
+      finish(c, Y);
     } else {
       throw Error(XS_EINVAL, "unknown product kind");
     }
-    XS_CUDA(cudaStreamSynchronize(s));
     return XS_OK;
   });
 }
@@ -313,6 +379,7 @@ int xs_excited(xs_ctx* ctx, const xs_ex_opts* opts, double* omega, double* osc, 
     std::vector<int> rcs(nmol, XS_OK);
     if (o.batched < 0 || o.batched > 2) throw Error(XS_EINVAL, "batched must be 0, 1 or 2");
     const int form = o.batched;
+    if (form != 0) c.io.release();   // batched solvers size their arenas by the free memory
     if (form == 1) {
       long long replays = 0;
       xs::davidson_batched(c, o, stats, rcs, &replays);
@@ -671,32 +738,35 @@ int xs_subspace_gram(xs_ctx* ctx, int M, int N, long long L, const double* A, co
     if (M == 0 || N == 0) return XS_OK;
     if (L > (1LL << 31) - 1024) throw Error(XS_EINVAL, "vectors too long");
     cudaStream_t s = c.stream;
-    DevBuf<double> dA((size_t)M * L), dB((size_t)N * L), dC((size_t)M * N);
-    copy_any(s, dA.get(), A, sizeof(double) * M * L);
-    copy_any(s, dB.get(), B, sizeof(double) * N * L);
+    const double* dA = input(c, 0, A, (size_t)M * L);
+    const double* dB = input(c, 1, B, (size_t)N * L);
+    // C is read by nothing before the last kernel writes it, but may overlap an input: always staged (M x N is small)
+    const Output dC{C, static_cast<double*>(c.io.get(2, sizeof(double) * M * N)), sizeof(double) * M * N};
     if (emulated) {
       if (!c.tc_err.get()) {
         c.tc_err.alloc(1);
         XS_CUDA(cudaMemsetAsync(c.tc_err.get(), 0, sizeof(int), s));
       }
       const long long Lp = xs::oz_lp(L);
-      DevBuf<xs::oz_t> ta((size_t)M * xs::kOzDigits * Lp), tb((size_t)N * xs::kOzDigits * Lp);
-      DevBuf<int> eA(M), eB(N);
-      xs::OzWork w;
-      xs::oz_exponents(s, M, L, dA.get(), L, eA.get(), w, c.tc_err.get());
-      xs::oz_exponents(s, N, L, dB.get(), L, eB.get(), w, c.tc_err.get());
+      const size_t na = (size_t)M * xs::kOzDigits * Lp, nb = (size_t)N * xs::kOzDigits * Lp;
+      xs::oz_t* ta = static_cast<xs::oz_t*>(c.io.get(3, sizeof(xs::oz_t) * (na + nb)));
+      xs::oz_t* tb = ta + na;
+      int* eA = static_cast<int*>(c.io.get(4, sizeof(int) * ((size_t)M + N)));
+      int* eB = eA + M;
+      if (!c.oz_work) c.oz_work = std::make_shared<xs::OzWork>();
+      xs::OzWork& w = *static_cast<xs::OzWork*>(c.oz_work.get());
+      xs::oz_exponents(s, M, L, dA, L, eA, w, c.tc_err.get());
+      xs::oz_exponents(s, N, L, dB, L, eB, w, c.tc_err.get());
       const long long PA = (long long)M * xs::kOzDigits, PB = (long long)N * xs::kOzDigits;   // plane capacities
-      xs::oz_slice(s, M, L, dA.get(), L, eA.get(), ta.get(), PA, 0, nullptr, 0, 0);
-      xs::oz_slice(s, N, L, dB.get(), L, eB.get(), tb.get(), PB, 0, nullptr, 0, 0);
-      xs::oz_gram(s, M, N, L, ta.get(), PA, eA.get(), tb.get(), PB, eB.get(), 1.0, 0.0, dC.get(), N, w,
-                  c.tc_err.get());
+      xs::oz_slice(s, M, L, dA, L, eA, ta, PA, 0, nullptr, 0, 0);
+      xs::oz_slice(s, N, L, dB, L, eB, tb, PB, 0, nullptr, 0, 0);
+      xs::oz_gram(s, M, N, L, ta, PA, eA, tb, PB, eB, 1.0, 0.0, dC.dev, N, w, c.tc_err.get());
       xs::check_device_error(c);
     } else {
-      xs::gram<double>(s, M, N, static_cast<int>(L), dA.get(), static_cast<int>(L), dB.get(), static_cast<int>(L),
-                       dC.get(), N, 1.0, 0.0, c.ws0);
+      xs::gram<double>(s, M, N, static_cast<int>(L), dA, static_cast<int>(L), dB, static_cast<int>(L), dC.dev, N, 1.0,
+                       0.0, c.ws0);
     }
-    copy_any(s, C, dC.get(), sizeof(double) * M * N);
-    XS_CUDA(cudaStreamSynchronize(s));
+    finish(c, dC);
     return XS_OK;
   });
 }
@@ -724,38 +794,44 @@ int xs_subspace_combine(xs_ctx* ctx, int nb, int S, int nout, long long L, const
     if (nout == 0) return XS_OK;
     if (L > (1LL << 31) - 1024) throw Error(XS_EINVAL, "vectors too long");
     cudaStream_t s = c.stream;
-    DevBuf<double> dX((size_t)nb * S * L), dc((size_t)nb * S * nout), dY((size_t)nout * L);
-    copy_any(s, dX.get(), X, sizeof(double) * nb * S * L);
-    copy_any(s, dc.get(), coef, sizeof(double) * nb * S * nout);
+    const double* dX = input(c, 0, X, (size_t)nb * S * L);
+    // the coefficients are small: always staged, so that only X can overlap the output
+    double* dc = static_cast<double*>(c.io.get(1, sizeof(double) * nb * S * nout));
+    copy_any(s, dc, coef, sizeof(double) * nb * S * nout);
+    const Output dY = output(c, 2, Y, (size_t)nout * L, X, (size_t)nb * S * L);
     if (emulated) {
       if (!c.tc_err.get()) {
         c.tc_err.alloc(1);
         XS_CUDA(cudaMemsetAsync(c.tc_err.get(), 0, sizeof(int), s));
       }
       const int ldk = xs::oz_ldk(S);
-      DevBuf<xs::oz_t> nn((size_t)nb * L * ldk);
-      // digit columns past S * 8 are read (times zero coefficients): clear them
-      XS_CUDA(cudaMemsetAsync(nn.get(), 0, sizeof(xs::oz_t) * nb * L * ldk, s));
-      DevBuf<int> e((size_t)nb * S);
-      xs::OzWork w;
+      xs::oz_t* nn = static_cast<xs::oz_t*>(c.io.get(3, sizeof(xs::oz_t) * nb * L * ldk));
+      // digit columns past S * 8 are read (times zero coefficients): clear the
+      // block of 64 columns that holds them
+      const int tail = S * xs::kOzDigits / 64 * 64;
+      if (tail < ldk)
+        for (int b = 0; b < nb; ++b)
+          XS_CUDA(cudaMemsetAsync(nn + (size_t)b * L * ldk + (size_t)tail * L, 0,
+                                  sizeof(xs::oz_t) * (size_t)(ldk - tail) * L, s));
+      int* e = static_cast<int*>(c.io.get(4, sizeof(int) * nb * S));
+      if (!c.oz_work) c.oz_work = std::make_shared<xs::OzWork>();
+      xs::OzWork& w = *static_cast<xs::OzWork*>(c.oz_work.get());
       xs::OzBlock blk[3];
       for (int b = 0; b < nb; ++b) {
-        const double* Xb = dX.get() + (size_t)b * S * L;
-        xs::oz_exponents(s, S, L, Xb, L, e.get() + b * S, w, c.tc_err.get());
-        xs::oz_slice(s, S, L, Xb, L, e.get() + b * S, nullptr, 0, 0, nn.get() + (size_t)b * L * ldk, ldk, 0);
-        blk[b] = xs::OzBlock{nn.get() + (size_t)b * L * ldk, ldk, e.get() + b * S, dc.get() + (size_t)b * S * nout,
-                             nout};
+        const double* Xb = dX + (size_t)b * S * L;
+        xs::oz_exponents(s, S, L, Xb, L, e + b * S, w, c.tc_err.get());
+        xs::oz_slice(s, S, L, Xb, L, e + b * S, nullptr, 0, 0, nn + (size_t)b * L * ldk, ldk, 0);
+        blk[b] = xs::OzBlock{nn + (size_t)b * L * ldk, ldk, e + b * S, dc + (size_t)b * S * nout, nout};
       }
-      xs::oz_combine(s, nb, blk, S, nout, L, 1.0, 0.0, dY.get(), L, w, c.tc_err.get());
+      xs::oz_combine(s, nb, blk, S, nout, L, 1.0, 0.0, dY.dev, L, w, c.tc_err.get());
       xs::check_device_error(c);
     } else {
       for (int b = 0; b < nb; ++b)
-        xs::gemm<double>(s, true, false, nout, static_cast<int>(L), S, 1.0, dc.get() + (size_t)b * S * nout, nout, 0,
-                         dX.get() + (size_t)b * S * L, static_cast<int>(L), 0, b == 0 ? 0.0 : 1.0, dY.get(),
+        xs::gemm<double>(s, true, false, nout, static_cast<int>(L), S, 1.0, dc + (size_t)b * S * nout, nout, 0,
+                         dX + (size_t)b * S * L, static_cast<int>(L), 0, b == 0 ? 0.0 : 1.0, dY.dev,
                          static_cast<int>(L), 0, 1);
     }
-    copy_any(s, Y, dY.get(), sizeof(double) * nout * L);
-    XS_CUDA(cudaStreamSynchronize(s));
+    finish(c, dY);
     return XS_OK;
   });
 }

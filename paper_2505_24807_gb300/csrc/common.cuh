@@ -104,6 +104,30 @@ struct DevMol {
   int iterations = 0;
 };
 
+// Device scratch of the API entries (staged arrays, digit operands), kept
+// between calls: a cudaMalloc / cudaFree pair costs 20 to 800 us by size, and
+// the cudaFree waits for the device (a 120 x 20 subspace projection over 373100
+// amplitudes took 1.9 ms for 0.6 ms of kernels).  Held memory is bounded: an
+// entry calls trim() at its end, and ground states and Davidson solves that run
+// short of memory release it.
+struct CallScratch {
+  static constexpr int kSlots = 5;
+  static constexpr size_t kKeep = size_t(2) << 30;   // bytes kept between calls
+  DevBuf<unsigned char> buf[kSlots];
+  void* get(int slot, size_t bytes) {
+    buf[slot].ensure(bytes);
+    return buf[slot].get();
+  }
+  void release() {
+    for (auto& b : buf) b.release();
+  }
+  void trim() {
+    size_t held = 0;
+    for (auto& b : buf) held += b.n;
+    if (held > kKeep) release();
+  }
+};
+
 struct Ctx {
   int device = 0;
   cudaStream_t stream = nullptr;
@@ -114,11 +138,13 @@ struct Ctx {
   std::vector<DevMol> mols;
   DevBuf<double> d_par;   // XS_NELEM x XS_NPARAM on the device
   void* solver = nullptr; // cusolverDnHandle_t, created on first use
+  CallScratch io;
   // scratch reused across calls
   DevBuf<double> ws0, ws1, ws2, ws3, ws4, ws5;
   DevBuf<float> fs0, fs1, fs2;
   Profiler prof;
   DevBuf<int> tc_err;   // error word of the tensor-core kernels' bounded waits
+  std::shared_ptr<void> oz_work;    // scratch of the subspace entries' digit products (ozaki.h)
   std::shared_ptr<void> mg_work;    // scratch of the residue products (modgemm.h)
   std::shared_ptr<void> dav_cache;  // Davidson workspace kept between solves (davidson.cu)
   std::shared_ptr<void> batch_cache;  // lock-step batched solver's arenas (batch.cu)

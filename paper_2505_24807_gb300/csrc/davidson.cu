@@ -372,6 +372,8 @@ int davidson(Ctx& c, DevMol& m, const xs_ex_opts& opt, SolveStats& st) {
     if (!(budget > 0.0)) {
       size_t free_b = 0, total_b = 0;
       XS_CUDA(cudaMemGetInfo(&free_b, &total_b));
+      // scratch of other entries counts as free: given back when the cap needs it
+      for (auto& b : c.io.buf) free_b += b.n;
       double held = 0.0;   // this context's subspace buffers are reused
       if (c.dav_cache) {
         const Work& w0 = *static_cast<const Work*>(c.dav_cache.get());
@@ -387,7 +389,10 @@ int davidson(Ctx& c, DevMol& m, const xs_ex_opts& opt, SolveStats& st) {
       throw Error(XS_ENOMEM, "subspace needs " + std::to_string(static_cast<long long>(Smin * per_vec)) +
                                  " bytes for its first " + std::to_string(Smin) + " vectors; budget " +
                                  std::to_string(static_cast<long long>(budget)));
-    if (cap < Smax) Smax = static_cast<int>(cap);
+    if (cap < Smax) {
+      Smax = static_cast<int>(cap);
+      c.io.release();
+    }
   }
   st.smax = Smax;
   // Mixed-precision products carry rounding noise of ~1e-6 relative, so their

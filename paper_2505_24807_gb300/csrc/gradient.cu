@@ -451,10 +451,28 @@ void parameter_gradient(Ctx& c, DevMol& m, int root, double* grad_host, int* cg_
   // amplitudes: CIS X; TDHF U = X+Y and W = X-Y
   const double* Y1 = m.U.get() + (size_t)root * ov;
   const double* Y2 = rpa ? m.Wv.get() + (size_t)root * ov : nullptr;
-  DevBuf<double> R(nn), R2(rpa ? nn : 1), Q(nn), GR(nn), Dl(nn), GD(nn), Dh(nn), tmp((size_t)n * std::max(o, v)),
-      Gvv((size_t)v * v), Goo((size_t)o * o), T((size_t)std::max(o, v) * std::max(o, v)), L(ov), Z(ov), r(ov), zv(ov),
-      p(ov), Ap(ov), RZ(nn), P(nn), pk((size_t)3 * m.np), grad((size_t)XS_NELEM * XS_NPARAM), part;
-  DevBuf<double> ws;
+  // work arrays carved from one kept block (starts on 256-byte boundaries)
+  const size_t big = std::max(o, v);
+  struct Carved {
+    double* p = nullptr;
+    size_t n = 0;
+    double* get() const { return p; }
+  };
+  Carved R{nullptr, (size_t)nn}, R2{nullptr, rpa ? (size_t)nn : 1}, Q{nullptr, (size_t)nn}, GR{nullptr, (size_t)nn},
+      Dl{nullptr, (size_t)nn}, GD{nullptr, (size_t)nn}, Dh{nullptr, (size_t)nn}, tmp{nullptr, n * big},
+      Gvv{nullptr, (size_t)v * v}, Goo{nullptr, (size_t)o * o}, T{nullptr, big * big}, L{nullptr, (size_t)ov},
+      Z{nullptr, (size_t)ov}, r{nullptr, (size_t)ov}, zv{nullptr, (size_t)ov}, p{nullptr, (size_t)ov},
+      Ap{nullptr, (size_t)ov}, RZ{nullptr, (size_t)nn}, P{nullptr, (size_t)nn}, pk{nullptr, (size_t)3 * m.np},
+      grad{nullptr, (size_t)XS_NELEM * XS_NPARAM};
+  Carved* all[] = {&R, &R2, &Q, &GR, &Dl, &GD, &Dh, &tmp, &Gvv, &Goo, &T, &L, &Z, &r, &zv, &p, &Ap, &RZ, &P, &pk, &grad};
+  size_t total = 0;
+  for (Carved* q : all) total += (q->n + 31) / 32 * 32;
+  double* at = static_cast<double*>(c.io.get(0, sizeof(double) * total));
+  for (Carved* q : all) {
+    q->p = at;
+    at += (q->n + 31) / 32 * 32;
+  }
+  DevBuf<double>&part = c.ws5, &ws = c.ws0;
   auto transition = [&](const double* Y, double* out) {   // C_occ Y C_vir^T
     gemm<double>(s, true, false, n, v, o, 1.0, CTocc, n, 0, Y, v, 0, 0.0, tmp.get(), v, 0, 1);
     gemm<double>(s, false, false, n, n, v, 1.0, tmp.get(), v, 0, CTvir, n, 0, 0.0, out, n, 0, 1);
@@ -552,6 +570,7 @@ void parameter_gradient(Ctx& c, DevMol& m, int root, double* grad_host, int* cg_
   XS_CHECK_LAUNCH();
   XS_CUDA(cudaMemcpyAsync(grad_host, grad.get(), sizeof(double) * XS_NELEM * XS_NPARAM, cudaMemcpyDeviceToHost, s));
   XS_CUDA(cudaStreamSynchronize(s));
+  c.io.trim();
 }
 
 }  // namespace xs

@@ -79,3 +79,39 @@ def test_residue_products_in_chunks():
             assert rel_err(Y[k:k + 1], one) < 1e-13
     finally:
         ctx.close()
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_device_arrays_in_place(precision):
+    """Products on device arrays are used in place: aligned, misaligned (8 bytes),
+    overlapping and identical input and output give the host arrays' result."""
+    torch = pytest.importorskip("torch")
+    params = molgen.make_params(0)
+    Z, xyz = molgen.make_chain(3, 30, 41)
+    ctx = context(params)
+    try:
+        xs.xs_ground_state(ctx.h, [(Z, xyz)], scf_tol=1e6)
+        n, o, _ = xs.xs_get_sizes(ctx.h, 0)
+        ov = o * (n - o)
+        X = molgen.trial_vectors(5, 3, o, n - o).reshape(3, -1)
+        ref = xs.xs_apply(ctx.h, 0, 1, X, precision=precision)
+        buf = torch.zeros(8 * ov + 8, dtype=torch.float64, device="cuda")
+        for at_in, at_out in ((0, 4 * ov), (1, 4 * ov + 1), (0, ov), (2 * ov, 0), (0, 0)):
+            x, y = buf[at_in:at_in + 3 * ov].view(3, ov), buf[at_out:at_out + 3 * ov].view(3, ov)
+            x.copy_(torch.from_numpy(X))
+            torch.cuda.synchronize()
+            xs.xs_apply(ctx.h, 0, 1, x, precision=precision, out=y)
+            assert np.array_equal(y.cpu().numpy(), ref)
+        A = torch.randn(5, 1001, dtype=torch.float64, device="cuda")
+        B = torch.randn(3, 1001, dtype=torch.float64, device="cuda")
+        out = torch.empty(5, 3, dtype=torch.float64, device="cuda")
+        torch.cuda.synchronize()
+        xs._check(ctx.h, xs.load().xs_subspace_gram(ctx.h, 5, 3, 1001, xs._ptr(A), xs._ptr(B), xs._ptr(out), 1))
+        assert np.array_equal(out.cpu().numpy(), xs.xs_subspace_gram(ctx.h, A.cpu().numpy(), B.cpu().numpy()))
+        # the output on top of the input
+        Xs, c = torch.randn(1, 5, 1001, dtype=torch.float64, device="cuda"), np.random.default_rng(1).standard_normal((1, 5, 3))
+        ref = xs.xs_subspace_combine(ctx.h, Xs.cpu().numpy(), c)
+        xs._check(ctx.h, xs.load().xs_subspace_combine(ctx.h, 1, 5, 3, 1001, xs._ptr(Xs), xs._ptr(c), xs._ptr(Xs), 1))
+        assert np.array_equal(Xs[0, :3].cpu().numpy(), ref)
+    finally:
+        ctx.close()
