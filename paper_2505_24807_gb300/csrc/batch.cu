@@ -108,6 +108,7 @@ struct BCfg {
   double tol;
   int pass;                           // Gram-Schmidt pass of the launch (0 or 1)
   int smax;                           // largest subspace cap of the group
+  int eig_k;                          // most eigenvectors per molecule whose solver scratch shares shared memory (0: none)
 };
 
 __device__ __forceinline__ double de_of(const BMol& d, long long l) {
@@ -966,7 +967,7 @@ __global__ void __launch_bounds__(256) bcopy_kernel(const BMol* __restrict__ mol
 // (upper triangle of a1 valid); TDHF: a- = L L^T, M = L^T a+ L, M z = omega^2 z,
 // X+Y = V L z / sqrt(omega), X-Y = V a+ (X+Y)~ / omega.  Writes omega and the
 // coefficient blocks of the Ritz-vector and residual combinations.
-__global__ void __launch_bounds__(1024) beig_kernel(const BMol* __restrict__ mols, int* __restrict__ st, BCfg cfg) {
+__global__ void __launch_bounds__(512) beig_kernel(const BMol* __restrict__ mols, int* __restrict__ st, BCfg cfg) {
   const int m = blockIdx.x;
   if (m >= cfg.nmol || !active(st, m)) return;
   const BMol& d = mols[m];
@@ -981,7 +982,7 @@ __global__ void __launch_bounds__(1024) beig_kernel(const BMol* __restrict__ mol
     }
     __syncthreads();
     const int kq = min(S, kk2);
-    syevk_body<true>(S, kq, d.Mb, ld, d.wts, d.Q, kk2, d.syw, nullptr);
+    syevk_body<true>(S, kq, d.Mb, ld, d.wts, d.Q, kk2, d.syw, nullptr, cfg.eig_k > 0);
     __syncthreads();
     if (tid == 0) st[m * kSt + F_KQ] = kq;
     for (int j = tid; j < kk; j += nt) d.omega[j] = j < k ? d.wts[j] : 0.0;
@@ -1025,7 +1026,7 @@ __global__ void __launch_bounds__(1024) beig_kernel(const BMol* __restrict__ mol
     d.Nb[(size_t)i * ld + j] = acc;
   }
   __syncthreads();
-  syevk_body<true>(S, k, d.Nb, ld, d.wts, d.E, kk2, d.syw, nullptr);
+  syevk_body<true>(S, k, d.Nb, ld, d.wts, d.E, kk2, d.syw, nullptr, cfg.eig_k > 0);
   __syncthreads();
   if (tid == 0) {
     int bad = 0;
@@ -1465,7 +1466,8 @@ template <typename T, int MODE>
 int enqueue_iteration(cudaStream_t s, const BMol* mols, int* st, const BCfg& cfg, const double* par, int* nact,
                       int* hnact) {
   const int kCombSmem = 3 * cfg.smax * 32 * 8;
-  const size_t kEigSmem = sizeof(double) * syevk_work_doubles(cfg.smax);
+  const size_t kEigSmem =
+      sizeof(double) * (syevk_work_doubles(cfg.smax) + (cfg.eig_k ? syevk_z_doubles(cfg.smax, cfg.eig_k) : 0));
   int launches = 0;
   auto L = [&]() { BATCH_LAUNCHED(); ++launches; };
   // products of the appended vectors
@@ -1486,7 +1488,7 @@ int enqueue_iteration(cudaStream_t s, const BMol* mols, int* st, const BCfg& cfg
   // projected matrices and the Rayleigh-Ritz step
   bgram_kernel<GR_PROJ><<<kGridCTAs, 256, 0, s>>>(mols, st, cfg); L();
   bgram_reduce_kernel<GR_PROJ><<<kGridCTAs, 256, 0, s>>>(mols, st, cfg); L();
-  beig_kernel<<<cfg.nmol, 1024, kEigSmem, s>>>(mols, st, cfg); L();
+  beig_kernel<<<cfg.nmol, 512, kEigSmem, s>>>(mols, st, cfg); L();
   if (!cfg.rpa) {
     britz_kernel<false><<<kGridCTAs, 256, 0, s>>>(mols, st, cfg); L();
   } else {
@@ -1526,7 +1528,7 @@ void set_attributes() {
   static const bool eig_attr = [] {
     XS_CUDA(cudaFuncSetAttribute(reinterpret_cast<const void*>(beig_kernel),
                                  cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(sizeof(double) * syevk_work_doubles(kBatchMaxSub))));
+                                 static_cast<int>(sizeof(double) * kEigSmemDoubles)));
     return true;
   }();
   (void)eig_attr;
@@ -1698,7 +1700,11 @@ void solve_group(Ctx& c, BatchWork& bw, const xs_ex_opts& opt, int first, int co
     d.U = m.U.get();
     d.Wv = m.Wv.get();
   }
-  for (int q = 0; q < count; ++q) cfg.smax = std::max(cfg.smax, h[q].Smax);
+  for (int q = 0; q < count; ++q) {
+    cfg.smax = std::max(cfg.smax, h[q].Smax);
+    cfg.eig_k = std::max(cfg.eig_k, (rpa ? 1 : 2) * h[q].kk);
+  }
+  if (!syevk_z_fits(cfg.smax, cfg.eig_k)) cfg.eig_k = 0;
   bw.dmols.ensure(count);
   XS_CUDA(cudaMemcpyAsync(bw.dmols.get(), h.data(), sizeof(BMol) * count, cudaMemcpyHostToDevice, s));
   std::vector<int> hst((size_t)count * kSt, 0);

@@ -7,25 +7,29 @@
 // costs ~640 cycles, so the kernel keeps float64 work in as few warps as hold
 // data and moves what can be approximate to float32:
 //   1. Householder tridiagonalisation Q^T A Q = T in float64 on the packed
-//      lower triangle (half the rank-2 update's float64 instructions; shared
-//      memory up to S = kSmemMax = 224, else global scratch, which runs ~3x
-//      slower per step); the reflectors go to
-//      global scratch, the matrix-vector product of each step is split over
-//      row segments, reductions run only in the warps that hold data;
+//      lower triangle (shared memory up to S = kSmemMax = 224, else global
+//      scratch); the reflectors stay in the triangle's columns, reductions run
+//      in integers in the warps that hold data, scalars come from float32
+//      estimates;
 //   2. the k lowest eigenvalues of T by Sturm-count multisection in float32,
 //      one warp per eigenvalue and 32 counts per round, to ~2e-7 |T|;
-//   3. float64 inverse iteration on T (pivoted tridiagonal LU, one thread per
-//      eigenvector, vector and LU in the freed shared memory when they fit):
-//      two solves with the float32 shift, then a third shifted by the
-//      Rayleigh quotient; the Rayleigh quotient of the result is the float64
-//      eigenvalue (its error is quadratic in the vector's).  Shifts closer
-//      than 2e-6 |T| form clusters: spread apart, solved three times with
-//      their own shift, re-orthogonalised (Gram-Schmidt) and, up to four
-//      members, rotated by a Rayleigh-Ritz step inside the cluster;
-//   4. back-transformation z = H_0 H_1 ... H_{S-3} y, one warp per vector.
+//   3. inverse iteration on T (pivoted tridiagonal LU, one thread per
+//      eigenvector): two float32 solves with the float32 shift, then two
+//      float64 solves shifted by the Rayleigh quotient; the Rayleigh quotient
+//      of the result is the float64 eigenvalue (its error is quadratic in the
+//      vector's).  Shifts closer than 2e-6 |T| form clusters: spread apart,
+//      solved three times in float64 with their own shift, re-orthogonalised
+//      (Gram-Schmidt) and, up to four members, rotated by a Rayleigh-Ritz step
+//      inside the cluster;
+//   4. back-transformation z = H_0 H_1 ... H_{S-3} y in blocks of eight
+//      reflectors (compact WY form).
+// Figures are at syevk_body.
 //
 // Also: Cholesky factorisation a = L L^T of the TDHF matrix a- (positive
-// definite unless the reference is unstable).
+// definite unless the reference is unstable); 70 x 70 104 -> 70 us, 100 x 100
+// 177 -> 127 us since the pivot's root and reciprocal come from a float32
+// estimate in the warps that scale the column and the trailing update has no
+// idle lanes.
 #include <cfloat>
 
 #include "kernels.h"
@@ -37,15 +41,17 @@ namespace xs {
 
 namespace {
 
+// (S <= kSmemMax runs with 512 threads: the float64 pipe is full at four warps a
+// sub-partition, and barriers cost half of what 1024 threads pay)
 template <bool SMEM>
-__global__ void __launch_bounds__(1024) syevk_kernel(int S, int k, const double* __restrict__ Ain, int lda,
+__global__ void __launch_bounds__(SMEM ? 512 : 1024) syevk_kernel(int S, int k, const double* __restrict__ Ain, int lda,
                                                      double* __restrict__ wout, double* __restrict__ Z, int ldz,
-                                                     double* __restrict__ gscratch, int* info) {
-  syevk_body<SMEM>(S, k, Ain, lda, wout, Z, ldz, gscratch, info);
+                                                     double* __restrict__ gscratch, int* info, bool zsm) {
+  syevk_body<SMEM>(S, k, Ain, lda, wout, Z, ldz, gscratch, info, zsm);
 }
 
 template <bool SMEM>
-__global__ void __launch_bounds__(1024) cholesky_kernel(int S, double* A, int lda, int* flag) {
+__global__ void __launch_bounds__(SMEM ? 512 : 1024) cholesky_kernel(int S, double* A, int lda, int* flag) {
   cholesky_body<SMEM>(S, A, lda, flag);
 }
 
@@ -63,16 +69,17 @@ void syevk(cudaStream_t s, int S, int k, const double* A, int lda, double* w, do
   scratch.ensure(syevk_scratch_doubles(S, k));
   ProfScope ps(s, "syevk_f64", 0.0, (4.0 / 3.0) * S * (double)S * S);
   if (S <= kSmemMax) {
-    const size_t smem = sizeof(double) * wd;
+    const bool zsm = syevk_z_fits(S, k);
+    const size_t smem = sizeof(double) * (wd + (zsm ? syevk_z_doubles(S, k) : 0));
     static const bool attr = [&] {   // once per process (thread-safe initialisation)
       XS_CUDA(cudaFuncSetAttribute(syevk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   static_cast<int>(sizeof(double) * syevk_work_doubles(kSmemMax))));
+                                   static_cast<int>(sizeof(double) * kEigSmemDoubles)));
       return true;
     }();
     (void)attr;
-    syevk_kernel<true><<<1, 1024, smem, s>>>(S, k, A, lda, w, Z, ldz, scratch.get(), info);
+    syevk_kernel<true><<<1, 512, smem, s>>>(S, k, A, lda, w, Z, ldz, scratch.get(), info, zsm);
   } else {
-    syevk_kernel<false><<<1, 1024, 0, s>>>(S, k, A, lda, w, Z, ldz, scratch.get(), info);
+    syevk_kernel<false><<<1, 1024, 0, s>>>(S, k, A, lda, w, Z, ldz, scratch.get(), info, false);
   }
   XS_CHECK_LAUNCH();
 }
@@ -88,7 +95,7 @@ void cholesky(cudaStream_t s, int S, double* A, int lda, int* flag) {
       return true;
     }();
     (void)attr;
-    cholesky_kernel<true><<<1, 1024, smem, s>>>(S, A, lda, flag);
+    cholesky_kernel<true><<<1, 512, smem, s>>>(S, A, lda, flag);
   } else {
     cholesky_kernel<false><<<1, 1024, 0, s>>>(S, A, lda, flag);
   }

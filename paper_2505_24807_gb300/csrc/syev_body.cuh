@@ -17,7 +17,7 @@ constexpr int kSeg = 8;         // row segments of the tridiagonalisation's matr
 constexpr int kMaxRR = 4;       // clusters up to this size get a Rayleigh-Ritz rotation
 
 // packed lower triangle: element (i, j), j <= i
-__host__ __device__ __forceinline__ size_t tri(int i, int j) { return (size_t)i * (i + 1) / 2 + j; }
+__host__ __device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }   // i <= 1024
 
 __device__ __forceinline__ double warp_sum(double x) {
   for (int o = 16; o > 0; o >>= 1) x += __shfl_xor_sync(0xffffffffu, x, o);
@@ -40,14 +40,87 @@ __device__ double block_sum(double x, double* red) {
   return red[32];
 }
 
+// |x| as an integer that orders like it: comparisons stay off the float64 pipe
+__device__ __forceinline__ long long mag_bits(double x) { return __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll; }
+
+// float32 of a double and back by their fields (the conversion instructions run
+// on the float64 pipe, 64 cycles each), for 2^-120 < |x| < 2^120
+__device__ __forceinline__ bool float_range(double x) {
+  const int e = (__double2hiint(x) >> 20) & 0x7FF;
+  return e > 1023 - 120 && e < 1023 + 120;
+}
+__device__ __forceinline__ float narrow_bits(double x) {
+  const unsigned hi = static_cast<unsigned>(__double2hiint(x)), lo = static_cast<unsigned>(__double2loint(x));
+  return __uint_as_float((hi & 0x80000000u) | (((hi & 0x7FFFFFFFu) - (896u << 20)) << 3) | (lo >> 29));
+}
+__device__ __forceinline__ double widen_bits(float x) {
+  const unsigned u = __float_as_uint(x);
+  return __hiloint2double(static_cast<int>((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + (896u << 20))),
+                          static_cast<int>(u << 29));
+}
+__device__ __forceinline__ float rcp_estimate(float x) {
+  float r;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+__device__ __forceinline__ float rsqrt_estimate(float x) {
+  float r;
+  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
+  return r;
+}
+
 // reciprocal to ~1e-14 relative: a float32 estimate refined by one Newton
 // step (inverse iteration needs directions, not correctly rounded quotients)
 __device__ __forceinline__ double rcp_fast(double x) {
-  const float xf = static_cast<float>(x);
-  const float ax = fabsf(xf);
-  if (!(ax > 1e-36f && ax < 1e36f)) return 1.0 / x;
-  const double r = static_cast<double>(__frcp_rn(xf));
+  if (!float_range(x)) return 1.0 / x;
+  const double r = widen_bits(rcp_estimate(narrow_bits(x)));
   return r * fma(-x, r, 2.0);
+}
+
+// square root, its reciprocal and the reciprocal to rounding (x > 0 for the
+// roots): float32 estimates with one third-order correction each, whose
+// remainder is 2^-66 relative
+__device__ __forceinline__ double sqrt_fast(double x) {
+  if (!float_range(x)) return sqrt(x);
+  const double r = widen_bits(rsqrt_estimate(narrow_bits(x)));
+  const double t = x * r;
+  const double e = fma(-t, r, 1.0);
+  return fma(t, e * fma(0.375, e, 0.5), t);
+}
+__device__ __forceinline__ double rsqrt_full(double x) {
+  if (!float_range(x)) return 1.0 / sqrt(x);
+  const double r = widen_bits(rsqrt_estimate(narrow_bits(x)));
+  const double e = fma(-(x * r), r, 1.0);
+  return fma(r, e * fma(0.375, e, 0.5), r);
+}
+__device__ __forceinline__ double rcp_full(double x) {
+  if (!float_range(x)) return 1.0 / x;
+  const double r = widen_bits(rcp_estimate(narrow_bits(x)));
+  const double e = fma(-x, r, 1.0);
+  return fma(r, fma(e, e, e), r);
+}
+
+// Sum of a warp's 32 values off the float64 pipe (a shuffle tree of adds takes
+// 540 cycles, this 300): the values as integers of 2^(emax - 57), emax the
+// largest exponent, added by the warp's integer reduction in 26-bit limbs.
+// Each is truncated at 2^-57 of the largest, below the rounding of the tree.
+__device__ __forceinline__ double warp_sum_int(double x) {
+  const unsigned long long bits = static_cast<unsigned long long>(__double_as_longlong(x));
+  const int ex = static_cast<int>((bits >> 52) & 0x7FF);
+  const int emax = __reduce_max_sync(0xffffffffu, ex);
+  if (emax > 1900 || emax < 100) return warp_sum(x);   // non-finite, or near the ends of the range
+  const int sh = emax - ex;
+  const unsigned long long mant = ex ? (((bits & 0xFFFFFFFFFFFFFull) | (1ull << 52)) << 5) : 0ull;
+  const unsigned long long m = sh > 63 ? 0ull : mant >> sh;
+  const long long q = (bits >> 63) ? -static_cast<long long>(m) : static_cast<long long>(m);
+  const unsigned l0 = __reduce_add_sync(0xffffffffu, static_cast<unsigned>(q) & 0x3FFFFFFu);
+  const unsigned l1 = __reduce_add_sync(0xffffffffu, static_cast<unsigned>(q >> 26) & 0x3FFFFFFu);
+  const int l2 = __reduce_add_sync(0xffffffffu, static_cast<int>(q >> 52));
+  const long long t =
+      static_cast<long long>(l0) + (static_cast<long long>(l1) << 26) + static_cast<long long>(static_cast<unsigned long long>(l2) << 52);
+  if (t == 0) return 0.0;
+  const double d = static_cast<double>(t);              // exponent field 1023 .. 1086
+  return __hiloint2double(__double2hiint(d) + (emax - 1080) * (1 << 20), __double2loint(d));
 }
 
 // number of eigenvalues of the float32 tridiagonal (d, e^2) below x
@@ -77,60 +150,143 @@ __device__ double rayleigh(int n, const double* d, const double* e, const double
 
 // Solve (T - shift I) x = y in place (y: stride ldy), factoring the pivoted
 // LU into lu (5 n doubles: 1/pivot, the two super-diagonals of U, the
-// multiplier, the row-swap flag) when factor is set, else reusing it; then
-// normalise y.  Pivots below tiny are raised to tiny.
+// multiplier, the row-swap flag; field f of row i at lu[(f n + i) ldy]) when
+// factor is set, else reusing it; then normalise y unless raw.  Pivots below
+// tiny are raised to tiny.
 __device__ void inverse_step(int n, const double* d, const double* e, double shift, double tiny, bool factor,
-                             double* lu, double* y, int ldy) {
+                             double* lu, double* y, int ldy, bool raw = false) {
+  const int fs = n * ldy;
   double* rc = lu;
-  double* u1 = lu + n;
-  double* u2 = lu + 2 * n;
-  double* fm = lu + 3 * n;
-  double* sw = lu + 4 * n;
+  double* u1 = lu + fs;
+  double* u2 = lu + 2 * fs;
+  double* fm = lu + 3 * fs;
+  double* sw = lu + 4 * fs;
   double cur = y[0];
   if (factor) {
+    // the next row's entries are loaded a step ahead of the elimination chain
     double c0 = d[0] - shift, c1 = n > 1 ? e[0] : 0.0, c2 = 0.0;
+    double pe = c1, pd = n > 1 ? d[1] : 0.0, py = n > 1 ? y[ldy] : 0.0;
     for (int i = 0; i + 1 < n; ++i) {
-      double n0 = e[i], n1 = d[i + 1] - shift, n2 = (i + 2 < n) ? e[i + 1] : 0.0;
-      double nr = y[(long long)(i + 1) * ldy];
-      const bool swp = fabs(n0) > fabs(c0);
-      if (swp) {
-        double t0 = c0, t1 = c1, t2 = c2, tr = cur;
-        c0 = n0; c1 = n1; c2 = n2; cur = nr;
-        n0 = t0; n1 = t1; n2 = t2; nr = tr;
-      }
-      if (fabs(c0) < tiny) c0 = c0 < 0.0 ? -tiny : tiny;
+      double n0 = pe, n1 = pd - shift, nr = py;
+      const bool more = i + 2 < n;
+      pe = more ? e[i + 1] : 0.0;
+      pd = more ? d[i + 2] : 0.0;
+      py = more ? y[(i + 2) * ldy] : 0.0;
+      double n2 = pe;
+      const bool swp = mag_bits(n0) > mag_bits(c0);
+      const double t0 = c0, t1 = c1, t2 = c2, tr = cur;
+      c0 = swp ? n0 : t0; c1 = swp ? n1 : t1; c2 = swp ? n2 : t2; cur = swp ? nr : tr;
+      n0 = swp ? t0 : n0; n1 = swp ? t1 : n1; n2 = swp ? t2 : n2; nr = swp ? tr : nr;
+      if (mag_bits(c0) < mag_bits(tiny)) c0 = copysign(tiny, c0);
       const double r = rcp_fast(c0);
       const double f = n0 * r;
-      rc[i] = r; u1[i] = c1; u2[i] = c2; fm[i] = f; sw[i] = swp ? 1.0 : 0.0;
-      y[(long long)i * ldy] = cur;
+      const int at = i * ldy;
+      rc[at] = r; u1[at] = c1; u2[at] = c2; fm[at] = f; sw[at] = swp ? 1.0 : 0.0;
+      y[at] = cur;
       c0 = fma(-f, c1, n1);
       c1 = fma(-f, c2, n2);
       c2 = 0.0;
       cur = fma(-f, cur, nr);
     }
-    if (fabs(c0) < tiny) c0 = c0 < 0.0 ? -tiny : tiny;
-    rc[n - 1] = rcp_fast(c0); u1[n - 1] = 0.0; u2[n - 1] = 0.0;
-    y[(long long)(n - 1) * ldy] = cur;
+    if (mag_bits(c0) < mag_bits(tiny)) c0 = copysign(tiny, c0);
+    const int at = (n - 1) * ldy;
+    rc[at] = rcp_fast(c0); u1[at] = 0.0; u2[at] = 0.0;
+    y[at] = cur;
   } else {
+    double py = n > 1 ? y[ldy] : 0.0, ps = sw[0], pf = fm[0];
     for (int i = 0; i + 1 < n; ++i) {
-      double nr = y[(long long)(i + 1) * ldy];
-      if (sw[i] != 0.0) { const double t = cur; cur = nr; nr = t; }
-      y[(long long)i * ldy] = cur;
-      cur = fma(-fm[i], cur, nr);
+      double nr = py;
+      const double swi = ps, f = pf;
+      const bool more = i + 2 < n;
+      py = more ? y[(i + 2) * ldy] : 0.0;
+      ps = more ? sw[(i + 1) * ldy] : 0.0;
+      pf = more ? fm[(i + 1) * ldy] : 0.0;
+      const bool swp = __double2hiint(swi) != 0;
+      const double t = cur;
+      cur = swp ? nr : t;
+      nr = swp ? t : nr;
+      y[i * ldy] = cur;
+      cur = fma(-f, cur, nr);
     }
-    y[(long long)(n - 1) * ldy] = cur;
+    y[(n - 1) * ldy] = cur;
   }
   // back substitution, then normalisation
   double y1 = 0.0, y2 = 0.0, nrm = 0.0;
+  int at = (n - 1) * ldy;
+  double qy = y[at], q1 = u1[at], q2 = u2[at], qr = rc[at];
   for (int i = n - 1; i >= 0; --i) {
-    const double yi = (y[(long long)i * ldy] - u1[i] * y1 - u2[i] * y2) * rc[i];
-    y[(long long)i * ldy] = yi;
-    nrm = fma(yi, yi, nrm);
+    const double yy = qy, a1 = q1, a2 = q2, ar = qr;
+    const int here = at;
+    at -= ldy;
+    if (i > 0) { qy = y[at]; q1 = u1[at]; q2 = u2[at]; qr = rc[at]; }
+    const double yi = fma(-a1, y1, fma(-a2, y2, yy)) * ar;
+    y[here] = yi;
+    if (!raw) nrm = fma(yi, yi, nrm);
     y2 = y1;
     y1 = yi;
   }
+  if (raw) return;
   const double inv = 1.0 / sqrt(nrm);
   for (int i = 0; i < n; ++i) y[(long long)i * ldy] *= inv;
+}
+
+// Two float32 inverse-iteration solves of (T - shift I) from the start vector in
+// y, one factorisation (fields as in inverse_step); pivots below tiny are raised
+// to it, which also bounds the growth of the unnormalised result.
+__device__ void inverse_step_f(int n, const float* d, const float* e, float shift, float tiny, float* lu, float* y,
+                               int ldy) {
+  const int fs = n * ldy;
+  float* rc = lu;
+  float* u1 = lu + fs;
+  float* u2 = lu + 2 * fs;
+  float* fm = lu + 3 * fs;
+  float* sw = lu + 4 * fs;
+  for (int pass = 0; pass < 2; ++pass) {
+    float cur = y[0];
+    if (pass == 0) {
+      float c0 = d[0] - shift, c1 = n > 1 ? e[0] : 0.0f, c2 = 0.0f;
+      for (int i = 0; i + 1 < n; ++i) {
+        float n0 = e[i], n1 = d[i + 1] - shift, n2 = i + 2 < n ? e[i + 1] : 0.0f, nr = y[(i + 1) * ldy];
+        const bool swp = fabsf(n0) > fabsf(c0);
+        const float t0 = c0, t1 = c1, t2 = c2, tr = cur;
+        c0 = swp ? n0 : t0; c1 = swp ? n1 : t1; c2 = swp ? n2 : t2; cur = swp ? nr : tr;
+        n0 = swp ? t0 : n0; n1 = swp ? t1 : n1; n2 = swp ? t2 : n2; nr = swp ? tr : nr;
+        if (fabsf(c0) < tiny) c0 = copysignf(tiny, c0);
+        const float r = __fdividef(1.0f, c0), f = n0 * r;
+        const int at = i * ldy;
+        rc[at] = r; u1[at] = c1; u2[at] = c2; fm[at] = f; sw[at] = swp ? 1.0f : 0.0f;
+        y[at] = cur;
+        c0 = fmaf(-f, c1, n1);
+        c1 = fmaf(-f, c2, n2);
+        c2 = 0.0f;
+        cur = fmaf(-f, cur, nr);
+      }
+      if (fabsf(c0) < tiny) c0 = copysignf(tiny, c0);
+      const int at = (n - 1) * ldy;
+      rc[at] = __fdividef(1.0f, c0); u1[at] = 0.0f; u2[at] = 0.0f;
+      y[at] = cur;
+    } else {
+      for (int i = 0; i + 1 < n; ++i) {
+        float nr = y[(i + 1) * ldy];
+        const int at = i * ldy;
+        const bool swp = sw[at] != 0.0f;
+        const float t = cur;
+        cur = swp ? nr : t;
+        nr = swp ? t : nr;
+        y[at] = cur;
+        cur = fmaf(-fm[at], cur, nr);
+      }
+      y[(n - 1) * ldy] = cur;
+    }
+    float y1 = 0.0f, y2 = 0.0f;
+    for (int i = n - 1; i >= 0; --i) {
+      const int at = i * ldy;
+      const float yi = fmaf(-u1[at], y1, fmaf(-u2[at], y2, y[at])) * rc[at];
+      y[at] = yi;
+      y2 = y1;
+      y1 = yi;
+    }
+  }
 }
 
 // Jacobi eigen-decomposition of a c x c symmetric matrix (c <= kMaxRR), one
@@ -175,145 +331,195 @@ __device__ void jacobi_small(int c, double (*H)[kMaxRR], double (*R)[kMaxRR]) {
       }
 }
 
-// sum over the first nact threads' x (red: 33 doubles); only the warps that
-// hold data spend float64 instructions (each costs 64 cycles of its
-// sub-partition's float64 pipe, whether or not its lanes are active)
-__device__ double active_sum(double x, double* red, int nact) {
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  const int nw = (nact + 31) >> 5;
-  if (w < nw) {
-    x = warp_sum(x);
-    if (l == 0) red[w] = x;
-  }
-  __syncthreads();
-  if (w == 0) {
-    double y = l < nw ? red[l] : 0.0;
-    if (nw > 1) y = warp_sum(y);
-    if (l == 0) red[32] = y;
-  }
-  __syncthreads();
-  return red[32];
+// working set of syevk_body in doubles (matrix, tridiagonal, reflectors,
+// products, eigenvalues, float32 copy, cluster indices); shared memory when
+// S <= kSmemMax
+__host__ __device__ constexpr size_t syevk_work_doubles(int n) {
+  return (size_t)n * (n + 1) / 2 + (size_t)(8 + kSeg) * n + (n + 1) / 2 + 64;
+}
+// eigenvectors, inverse-iteration factors and back-transformation scratch: after
+// the working set in shared memory when both fit (syevk_z_fits), else in
+// global scratch
+__host__ __device__ constexpr size_t syevk_z_doubles(int S, int k) { return (size_t)6 * S * k + (size_t)16 * k; }
+constexpr size_t kEigSmemDoubles = 28968;   // 226.3 KB: the working set at S = 224
+__host__ __device__ constexpr bool syevk_z_fits(int S, int k) {
+  return S <= kSmemMax && syevk_work_doubles(S) + syevk_z_doubles(S, k) <= kEigSmemDoubles;
+}
+__host__ __device__ constexpr size_t syevk_scratch_doubles(int S, int k) {
+  return (S <= kSmemMax ? 0 : syevk_work_doubles(S)) + syevk_z_doubles(S, k) + 64;
 }
 
+constexpr int kWy = 8;          // reflectors per block of the back-transformation
+
+// zsm: the dynamic shared memory holds syevk_z_doubles(S, k) more doubles after
+// the working set, else they are in gscratch.
+//
+// Every float64 instruction of a warp holds its sub-partition's pipe for 64
+// cycles whatever the number of active lanes (latency 64 too), so the body is
+// bound by the number of float64 instructions on its critical path.  Solve times
+// before -> after the present form (one CTA): 48 x 48, 10 vectors 438 -> 203 us
+// (tridiagonalisation 221 -> 106, inverse iteration 141 -> 56,
+// back-transformation 72 -> 29); 100 x 100 1117 -> 567 us; 200 x 200 3316 ->
+// 2474 us.
 template <bool SMEM>
 __device__ void syevk_body(int S, int k, const double* __restrict__ Ain, int lda, double* __restrict__ wout,
-                           double* __restrict__ Z, int ldz, double* __restrict__ gscratch, int* info) {
+                           double* __restrict__ Z, int ldz, double* __restrict__ gscratch, int* info, bool zsm) {
   extern __shared__ double sh[];
   __shared__ double red[33];
   __shared__ double scal[8];
   double* base = SMEM ? sh : gscratch;
-  double* a = base;                          // packed lower triangle; later Z and LU scratch
+  double* a = base;                          // packed lower triangle; column j keeps reflector j below the diagonal
   double* d = a + tri(S, 0);
   double* e = d + S;
-  double* v = e + S;                         // current reflector
-  double* p = v + S;                         // B v, then w
+  double* beta = e + S;                      // reflector j: H_j = I - beta_j u_j u_j^T
+  double* vb = beta + S;                     // two buffers of the current reflector u
+  double* p = vb + 2 * S;                    // B u, then w
   double* ps = p + S;                        // kSeg x S matrix-vector partials
-  double* lam = ps + (size_t)kSeg * S;       // eigenvalues
+  double* lam = ps + (size_t)kSeg * S + 64;  // eigenvalues
   float* df = reinterpret_cast<float*>(lam + S);
   float* e2f = df + S;
   int* cl = reinterpret_cast<int*>(e2f + S); // first index of each eigenvalue's cluster
-  double* gfree = gscratch + (SMEM ? 0 : (tri(S, 0) + (size_t)(5 + kSeg) * S + 2 * S));
-  double* R = gfree;                         // reflectors: row j holds v_j (S - j - 1 entries)
-  // eigenvectors and inverse-iteration LU rows: in the freed matrix area of
-  // shared memory when they fit, else in global scratch
-  const bool zsm = SMEM && 12 * k <= S + 1;   // 6 S k doubles in the S (S + 1) / 2 of the matrix
-  double* Zw = zsm ? a : gfree + (size_t)S * S;      // S x k, row stride k
-  double* lu = Zw + (size_t)S * k;                    // 5 S per vector
+  double* gfree = gscratch + (SMEM ? 0 : syevk_work_doubles(S));
+  double* Zw = SMEM && zsm ? sh + syevk_work_doubles(S) : gfree;   // S x k, row stride k
+  double* lu = Zw + (size_t)S * k;                                 // 5 S x k, then 16 k
   const int tid = threadIdx.x, nt = blockDim.x;
   const int warp = tid >> 5, lane = tid & 31, nwarp = nt >> 5;
 
-  for (int idx = tid; idx < S * S; idx += nt) {
-    const int i = idx / S, j = idx % S;
-    if (j <= i) a[tri(i, j)] = Ain[(long long)i * lda + j];
-  }
+  for (int i = warp; i < S; i += nwarp)
+    for (int j = lane; j <= i; j += 32) a[tri(i, j)] = Ain[(long long)i * lda + j];
   __syncthreads();
 
-  // 1. tridiagonalisation
+  // 1. Tridiagonalisation by Householder reflectors H = I - beta u u^T on the
+  // packed lower triangle.  The products of a step of m remaining rows take m^2
+  // cycles (matrix-vector product and rank-2 update at two multiply-adds per
+  // clock); the chain of reductions and scalars between them is kept short:
+  // integer reductions, scalars from float32 estimates, u left unnormalised so
+  // that beta is formed beside the matrix-vector product, and the next column's
+  // norm formed beside the rank-2 update.
+
+  // row segments of the matrix-vector product by remaining rows (segment count
+  // and length): the split with the fewest float64 instructions on the critical
+  // path, the segments' sum included
+  short* segs = reinterpret_cast<short*>(lam);   // the eigenvalues come later
+  for (int m = tid + 1; m < S; m += nt) {
+    int best = 1 | (m << 4), cost = 1 << 30;
+    for (int g = 1; g <= kSeg; ++g) {
+      if (g > 1 && g * m > nt - 32) break;
+      const int len = (m + g - 1) / g;
+      const int c = ((g * m + 127) >> 7) * len + g;
+      if (c < cost) { cost = c; best = g | (len << 4); }
+    }
+    segs[m] = static_cast<short>(best);
+  }
+
+  // reflector of column j from its m entries below the diagonal: x is entry idx,
+  // held by the threads of the first nw warps (0 outside 0 <= idx < m)
+  auto reflector = [&](int j, int m, int idx, int nw, double x, double* u) {
+    double sig = warp_sum_int(x * x);
+    if (idx == 0) scal[0] = x;
+    if (nw > 1) {
+      if (lane == 0) red[warp] = sig;
+      asm volatile("bar.sync 1, %0;" ::"r"(32 * nw) : "memory");
+      sig = red[0];
+      for (int w = 1; w < nw; ++w) sig += red[w];
+    } else {
+      __syncwarp();
+    }
+    const double x0 = scal[0];
+    // a column that is zero to rounding keeps its first entry (H = I)
+    const bool skip = mag_bits(sig) < mag_bits(1e-300);
+    const double nx = skip ? 0.0 : sqrt_fast(sig);
+    const double al = skip ? x0 : -copysign(nx, x0);
+    if (idx >= 0 && idx < m) {
+      const double ui = skip ? 0.0 : (idx == 0 ? x0 - al : x);
+      u[idx] = ui;
+      a[tri(j + 1 + idx, j)] = ui;
+    }
+    if (idx == 0) {
+      e[j] = al;
+      scal[1] = skip ? 0.0 : fma(fabs(x0), nx, sig);   // 1 / beta
+    }
+  };
+  if (S > 2 && warp < (S + 30) / 32)
+    reflector(0, S - 1, tid, (S + 30) / 32, tid < S - 1 ? a[tri(1 + tid, 0)] : 0.0, vb);
+  __syncthreads();
   for (int j = 0; j + 2 < S; ++j) {
-    const int r0 = j + 1, m = S - r0;
-    double part = 0.0;
-    if (tid < m) {
-      const double x = a[tri(r0 + tid, j)];
-      part = x * x;
+    const int r0 = j + 1, m = S - r0, nw = (m + 31) >> 5;
+    const double* v = vb + (j & 1) * S;
+    // B u, B symmetric and held as its lower triangle (B[i][l] read from row
+    // max(i, l)), split over nseg row segments; the last warp forms beta
+    const int nseg = segs[m] & 15, len = segs[m] >> 4;
+    const float rm = __fdividef(1.0f, static_cast<float>(m));
+    if (warp == nwarp - 1 && lane == 0) {
+      const double q = scal[1];
+      const double b = mag_bits(q) ? rcp_full(q) : 0.0;
+      scal[2] = b;
+      scal[3] = 0.5 * b;
+      beta[j] = b;
     }
-    // column norm; the final reduction's lane forms the step's scalars (in
-    // one thread: float64 instructions in every warp would cost 32 times as
-    // much) and broadcasts them through shared memory
+    for (int q = tid; q < nseg * m; q += nt) {
+      const int g = static_cast<int>((static_cast<float>(q) + 0.5f) * rm), i = q - g * m;
+      const int l0 = g * len, l1 = min(m, l0 + len);
+      double acc = 0.0;
+      int at = l0 <= i ? tri(r0 + i, r0 + l0) : tri(r0 + l0, r0 + i);
+      for (int l = l0; l < l1; ++l) {
+        acc = fma(a[at], v[l], acc);
+        at += l < i ? 1 : r0 + l + 1;
+      }
+      ps[g * m + i] = acc;
+    }
+    __syncthreads();
+    double ui = 0.0, wi = 0.0;
+    if (warp < nw) {
+      if (tid < m) {
+        for (int g = 0; g < nseg; ++g) wi += ps[g * m + tid];
+        wi *= scal[2];
+        ui = v[tid];
+      }
+      double K = warp_sum_int(ui * wi);
+      if (nw > 1) {
+        if (lane == 0) red[warp] = K;
+        asm volatile("bar.sync 1, %0;" ::"r"(32 * nw) : "memory");
+        K = red[0];
+        for (int w = 1; w < nw; ++w) K += red[w];
+      }
+      wi = fma(-(K * scal[3]), ui, wi);      // w = beta B u - (beta / 2) (u . beta B u) u
+      if (tid < m) p[tid] = wi;
+    }
+    __syncthreads();
+    // rank-2 update B -= u w^T + w u^T of the lower triangle: column 0 and the
+    // next reflector by the vector warps, the other columns by the rest
+    if (warp < nw) {
+      double x = 0.0;
+      if (tid < m) {
+        x = fma(-ui, p[0], fma(-wi, v[0], a[tri(r0 + tid, r0)]));
+        if (tid == 0) d[r0] = x;
+        a[tri(r0 + tid, r0)] = x;
+        if (tid == 0) x = 0.0;               // the diagonal is not part of the column below it
+      }
+      if (j + 3 < S) reflector(r0, m - 1, tid - 1, nw, x, vb + ((j + 1) & 1) * S);
+    }
     {
-      const int nw = (m + 31) >> 5;
-      if (warp < nw) {
-        part = warp_sum(part);
-        if (lane == 0) red[warp] = part;
-      }
-      __syncthreads();
-      if (warp == 0) {
-        double y = lane < nw ? red[lane] : 0.0;
-        if (nw > 1) y = warp_sum(y);
-        if (lane == 0) {
-          const double sigma = y;
-          const double x0 = a[tri(r0, j)];
-          const double nx = sqrt(sigma);
-          const double scale_ref = fabs(a[tri(j, j)]) + nx;
-          const bool sk = !(nx > 1e-300) || nx <= 1e-300 * scale_ref;
-          const double al = sk ? x0 : ((x0 > 0.0) ? -nx : nx);
-          scal[0] = al;
-          scal[1] = sk ? 0.0 : rsqrt(2.0 * (sigma - x0 * al));
-          scal[2] = sk ? 1.0 : 0.0;
+      // rows 1..m-1, columns 1..row, all lanes busy: rows i and m - i have m entries together
+      const bool apart = nwarp > nw;
+      const int nup = apart ? nt - 32 * nw : nt, t0 = apart ? tid - 32 * nw : tid;
+      const int work = (m >> 1) * m;
+      if (t0 >= 0)
+        for (int q = t0; q < work; q += nup) {
+          int pr = static_cast<int>((static_cast<float>(q) + 0.5f) * rm);
+          int off = q - pr * m;
+          if (off < 0) { --pr; off += m; }
+          if (off >= m) { ++pr; off -= m; }
+          const int ia = pr + 1, ib = m - ia;
+          if (off >= ia && ia == ib) continue;       // the middle row of an even m
+          const int i = off < ia ? ia : ib, l = off < ia ? off + 1 : off - ia + 1;
+          double* at = a + tri(r0 + i, r0 + l);
+          *at = fma(-v[i], p[l], fma(-p[i], v[l], *at));
         }
-      }
-      __syncthreads();
-    }
-    const bool skip = scal[2] != 0.0;
-    const double alpha = scal[0];
-    double* Rj = R + (size_t)j * S;
-    if (!skip) {
-      const double inv = scal[1];
-      if (tid < m) {
-        const double x = a[tri(r0 + tid, j)];
-        const double vi = ((tid == 0) ? (x - alpha) : x) * inv;
-        v[tid] = vi;
-        Rj[tid] = vi;
-      }
-      __syncthreads();
-      // p = B v, B symmetric and held as its lower triangle (B[i][l] read
-      // from row max(i, l)), split over nseg row segments summed in order
-      const int nseg = min(kSeg, nt / m);
-      const int len = (m + nseg - 1) / nseg;
-      if (tid < nseg * m) {
-        const int i = tid % m, g = tid / m;
-        const int l1 = min(m, (g + 1) * len);
-        double acc = 0.0;
-        for (int l = g * len; l < l1; ++l) {
-          const size_t at = (l >= i) ? tri(r0 + l, r0 + i) : tri(r0 + i, r0 + l);
-          acc = fma(a[at], v[l], acc);
-        }
-        ps[g * m + i] = acc;
-      }
-      __syncthreads();
-      double kp = 0.0, pi = 0.0;
-      if (tid < m) {
-        for (int g = 0; g < nseg; ++g) pi += ps[g * m + tid];
-        kp = v[tid] * pi;
-      }
-      const double K = active_sum(kp, red, m);
-      if (tid < m) p[tid] = 2.0 * pi - 2.0 * K * v[tid];   // w
-      __syncthreads();
-      // rank-2 update of the lower triangle only: B -= v w^T + w v^T
-      for (int i = warp; i < m; i += nwarp) {
-        const double vi = v[i], wi = p[i];
-        double* row = a + tri(r0 + i, r0);
-        for (int l = lane; l <= i; l += 32) row[l] = fma(-vi, p[l], fma(-wi, v[l], row[l]));
-      }
-    } else if (tid < m) {
-      v[tid] = 0.0;
-      Rj[tid] = 0.0;
-    }
-    if (tid == 0) {
-      d[j] = a[tri(j, j)];
-      e[j] = alpha;
     }
     __syncthreads();
   }
+  if (tid == 0) d[0] = a[0];
   if (tid == 0) {
     if (S >= 2) {
       d[S - 2] = a[tri(S - 2, S - 2)];
@@ -409,13 +615,67 @@ __device__ void syevk_body(int S, int k, const double* __restrict__ Ain, int lda
     const double inv = nrm > 0.0 ? 1.0 / sqrt(nrm) : 0.0;
     for (int i = 0; i < S; ++i) y[(long long)i * k] *= inv;
   };
+  auto isolated = [&](int t) { return cl[t] == t && (t + 1 == k || cl[t + 1] != t); };
+  // isolated eigenvalues, a thread each in step: two float32 solves with the
+  // float32 shift leave an error of about 1e-7 |T| / gap in the vector and its
+  // square in the Rayleigh quotient; two float64 solves with that shift (one
+  // factorisation) raise it to the fifth power.  Norms and quotients by a warp
+  // per vector in between.
+  auto normalise = [&]() {
+    for (int t = warp; t < k; t += nwarp) {
+      if (!isolated(t)) continue;
+      double* y = Zw + t;
+      double nn = 0.0, rq = 0.0;
+      for (int i = lane; i < S; i += 32) {
+        const double yi = y[(long long)i * k];
+        double ty = d[i] * yi;
+        if (i > 0) ty = fma(e[i - 1], y[(long long)(i - 1) * k], ty);
+        if (i + 1 < S) ty = fma(e[i], y[(long long)(i + 1) * k], ty);
+        nn = fma(yi, yi, nn);
+        rq = fma(yi, ty, rq);
+      }
+      nn = warp_sum_int(nn);
+      rq = warp_sum_int(rq);
+      const double inv = rsqrt_full(nn);
+      for (int i = lane; i < S; i += 32) y[(long long)i * k] *= inv;
+      if (lane == 0) lam[t] = rq * rcp_full(nn);
+    }
+    __syncthreads();
+  };
+  {
+    // float32 solves: the tridiagonal in vb, factors and vectors in lu
+    float* ef = reinterpret_cast<float*>(vb);
+    float* luf = reinterpret_cast<float*>(lu);
+    float* yf = luf + (size_t)5 * S * k;
+    for (int i = tid; i + 1 < S; i += nt) ef[i] = static_cast<float>(e[i]);
+    for (int q = tid; q < S * k; q += nt) {
+      const int i = q / k, t = q - i * k;
+      yf[q] = 1.0f + 0.01f * ((i * 7 + t * 3) % 11);
+    }
+    __syncthreads();
+    const float tinyf = 1e-8f * static_cast<float>(tnorm);
+    for (int t = tid; t < k; t += nt)
+      if (isolated(t)) inverse_step_f(S, df, ef, static_cast<float>(lam[t]), tinyf, luf + t, yf + t, k);
+    __syncthreads();
+    for (int q = tid; q < S * k; q += nt) Zw[q] = static_cast<double>(yf[q]);
+    __syncthreads();
+  }
+  normalise();
+  for (int t = tid; t < k; t += nt) {
+    if (!isolated(t)) continue;
+    inverse_step(S, d, e, lam[t], tiny, true, lu + t, Zw + t, k, true);
+    inverse_step(S, d, e, lam[t], tiny, false, lu + t, Zw + t, k, true);
+  }
+  __syncthreads();
+  normalise();
+  // clusters, a thread each
   for (int c0 = tid; c0 < k; c0 += nt) {
-    if (cl[c0] != c0) continue;   // not the first member of its cluster
+    if (cl[c0] != c0 || isolated(c0)) continue;
     int c1 = c0 + 1;
     while (c1 < k && cl[c1] == c0) ++c1;
     for (int t = c0; t < c1; ++t) {
       double* y = Zw + t;
-      double* lut = lu + (size_t)t * 5 * S;
+      double* lut = lu + t;
       for (int i = 0; i < S; ++i) y[(long long)i * k] = 1.0 + 0.01 * ((i * 7 + t * 3) % 11);
       inverse_step(S, d, e, lam[t], tiny, true, lut, y, k);
       orth_against(y, c0, t);
@@ -427,7 +687,7 @@ __device__ void syevk_body(int S, int k, const double* __restrict__ Ain, int lda
       // Rayleigh quotient they fall by a further (spread inside / gap)
       const double rq = rayleigh(S, d, e, y, k);
       inverse_step(S, d, e, rq, tiny, true, lut, y, k);
-      if (c1 - c0 > 1) orth_against(y, c0, t);
+      orth_against(y, c0, t);
     }
     for (int t = c0; t < c1; ++t) lam[t] = rayleigh(S, d, e, Zw + t, k);
   }
@@ -498,20 +758,92 @@ __device__ void syevk_body(int S, int k, const double* __restrict__ Ain, int lda
     }
   }
   __syncthreads();
-  // 4. back-transformation z = H_0 ... H_{S-3} y, one warp per eigenvector,
-  //    then the result into Z
-  for (int t = warp; t < k; t += nwarp) {
-    for (int j = S - 3; j >= 0; --j) {
-      const int r0 = j + 1, m = S - r0;
-      const double* Rj = R + (size_t)j * S;
-      double sacc = 0.0;
-      for (int l = lane; l < m; l += 32) sacc = fma(Rj[l], Zw[(r0 + l) * k + t], sacc);
-      sacc = warp_sum(sacc);
-      for (int l = lane; l < m; l += 32) Zw[(r0 + l) * k + t] -= 2.0 * sacc * Rj[l];
+  // 4. Back-transformation z = H_0 ... H_{S-3} y in blocks of kWy reflectors,
+  // H_jb ... H_jb+7 = I - U T U^T (T upper triangular): the dot products of a
+  // block are independent, so the cross-thread sums come once per block instead
+  // of once per reflector.
+  const int nref = S > 2 ? S - 2 : 0, nblk = (nref + kWy - 1) / kWy;
+  double* T = vb;                            // nblk x 64 (vb, p and ps are free now)
+  auto refl = [&](int i, int jb, int r) { return i > jb + r && jb + r < nref ? a[tri(i, jb + r)] : 0.0; };
+  for (int b = warp; b < nblk; b += nwarp) {
+    const int jb = b * kWy;
+    double* Tb = T + b * 64;
+    // strictly upper part: u_q . u_r for q < r, one lane each
+    int r = 1;
+    while (r * (r + 1) / 2 <= lane) ++r;     // lane = r (r - 1) / 2 + q
+    const int q = lane - r * (r - 1) / 2;
+    double g = 0.0;
+    if (r < kWy)
+      for (int i = jb + r + 1; i < S; ++i) g = fma(refl(i, jb, q), refl(i, jb, r), g);
+    if (r < kWy) Tb[q * kWy + r] = g;
+    __syncwarp();
+    for (int c = 0; c < kWy; ++c) {
+      const double bc = jb + c < nref ? beta[jb + c] : 0.0;
+      double t = 0.0;
+      if (lane < c) {
+        for (int w = lane; w < c; ++w) t = fma(Tb[lane * kWy + w], Tb[w * kWy + c], t);
+        t *= -bc;
+      }
+      __syncwarp();
+      if (lane < c) Tb[lane * kWy + c] = t;
+      if (lane == c) Tb[c * kWy + c] = bc;
       __syncwarp();
     }
-    for (int i = lane; i < S; i += 32) Z[(long long)i * ldz + t] = Zw[i * k + t];
   }
+  const int tg = (k + 3) / 4;                // groups of four vectors
+  const int nsg = max(1, min(nwarp / tg, 5 * S / kWy));
+  double* P = lu;                            // nsg x kWy x k partial dot products
+  double* sv = lu + (size_t)5 * S * k;       // kWy x k: U^T z, then T U^T z after it
+  double* yv = sv + kWy * k;
+  const float rk = 1.0f / static_cast<float>(k);
+  auto div_k = [&](int q) {                  // q / k (q < 2^20)
+    int g = static_cast<int>((static_cast<float>(q) + 0.5f) * rk);
+    if (g * k > q) --g;
+    return g;
+  };
+  __syncthreads();
+  for (int b = nblk - 1; b >= 0; --b) {
+    const int jb = b * kWy, i0 = jb + 1, rows = S - i0;
+    const int len = (rows + nsg - 1) / nsg;
+    for (int w = warp; w < tg * nsg; w += nwarp) {
+      const int sg = w / tg, r = lane & 7, t = (w - sg * tg) * 4 + (lane >> 3);
+      const int i1 = min(S, i0 + (sg + 1) * len);
+      double acc = 0.0;
+      if (t < k && jb + r < nref) {
+        const int ib = max(i0 + sg * len, jb + r + 1);
+        int at = tri(ib, jb + r);
+        for (int i = ib; i < i1; ++i) {
+          acc = fma(a[at], Zw[i * k + t], acc);
+          at += i + 1;
+        }
+      }
+      if (t < k) P[(sg * kWy + r) * k + t] = acc;
+    }
+    __syncthreads();
+    for (int q = tid; q < kWy * k; q += nt) {
+      double t = P[q];
+      for (int sg = 1; sg < nsg; ++sg) t += P[sg * kWy * k + q];
+      sv[q] = t;
+    }
+    __syncthreads();
+    for (int q = tid; q < kWy * k; q += nt) {
+      const int r = div_k(q), t = q - r * k;
+      double y = 0.0;
+      for (int w = r; w < kWy; ++w) y = fma(T[b * 64 + r * kWy + w], sv[w * k + t], y);
+      yv[q] = y;
+    }
+    __syncthreads();
+    for (int q = tid; q < rows * k; q += nt) {
+      const int g = div_k(q), i = i0 + g, t = q - g * k;
+      const int nr = min(min(kWy, nref - jb), g + 1);     // reflectors that reach row i
+      const double* u = a + tri(i, jb);
+      double z = Zw[i0 * k + q];
+      for (int r = 0; r < nr; ++r) z = fma(-u[r], yv[r * k + t], z);
+      Zw[i0 * k + q] = z;
+    }
+    __syncthreads();
+  }
+  for (int q = tid; q < S * k; q += nt) Z[(long long)(q / k) * ldz + q % k] = Zw[q];
   for (int t = tid; t < k; t += nt) wout[t] = lam[t];
   if (tid == 0 && info) *info = 0;
 }
@@ -525,34 +857,43 @@ constexpr int kCholSmemMax = 224;
 template <bool SMEM>
 __device__ void cholesky_body(int S, double* A, int lda, int* flag) {
   extern __shared__ double sh[];
-  __shared__ double inv;
   const int tid = threadIdx.x, nt = blockDim.x;
   const int warp = tid >> 5, lane = tid & 31, nwarp = nt >> 5;
   // element (i, l), l <= i: packed in shared memory, else in place in A
   auto at = [&](int i, int l) -> double& { return SMEM ? sh[tri(i, l)] : A[(long long)i * lda + l]; };
   if (SMEM) {
-    for (int idx = tid; idx < S * S; idx += nt) {
-      const int i = idx / S, l = idx % S;
-      if (l <= i) sh[tri(i, l)] = A[(long long)i * lda + l];
-    }
-    __syncthreads();
+    for (int i = warp; i < S; i += nwarp)
+      for (int l = lane; l <= i; l += 32) sh[tri(i, l)] = A[(long long)i * lda + l];
   }
+  __syncthreads();
   for (int j = 0; j < S; ++j) {
+    const int m = S - 1 - j;                 // rows below the pivot
+    // the warps that scale the column each form 1 / sqrt(pivot) from a float32
+    // estimate (sqrt and divide took 1100 cycles on one thread)
+    double x = at(j, j);
+    const long long xb = __double_as_longlong(x);
+    const bool bad = xb <= 0 || xb > 0x7FF0000000000000ll;   // not positive, or NaN
+    if (bad) x = 1e-300;
+    const double r = 32 * warp < max(m, 1) ? rsqrt_full(x) : 0.0;
+    for (int i = tid; i < m; i += nt) at(j + 1 + i, j) *= r;
+    __syncthreads();
     if (tid == 0) {
-      double x = at(j, j);
-      if (!(x > 0.0)) { *flag = 1; x = 1e-300; }
-      const double piv = sqrt(x);
-      at(j, j) = piv;
-      inv = 1.0 / piv;
+      if (bad) *flag = 1;
+      at(j, j) = x * r;
     }
-    __syncthreads();
-    const double r = inv;
-    for (int i = j + 1 + tid; i < S; i += nt) at(i, j) *= r;
-    __syncthreads();
-    // trailing update of the lower triangle
-    for (int i = j + 1 + warp; i < S; i += nwarp) {
-      const double lij = at(i, j);
-      for (int l = j + 1 + lane; l <= i; l += 32) at(i, l) = fma(-lij, at(l, j), at(i, l));
+    // trailing update, all lanes busy: rows i and m - 1 - i of the triangle have m + 1 entries together
+    const float rm = 1.0f / static_cast<float>(m + 1);
+    const int work = ((m + 1) >> 1) * (m + 1);
+    for (int q = tid; q < work; q += nt) {
+      int pr = static_cast<int>((static_cast<float>(q) + 0.5f) * rm);
+      int off = q - pr * (m + 1);
+      if (off < 0) { --pr; off += m + 1; }
+      if (off > m) { ++pr; off -= m + 1; }
+      const int ib = m - 1 - pr;
+      if (off > pr && pr == ib) continue;    // the middle row of an odd m
+      const int i = off <= pr ? pr : ib, l = off <= pr ? off : off - pr - 1;
+      double& c = at(j + 1 + i, j + 1 + l);
+      c = fma(-at(j + 1 + i, j), at(j + 1 + l, j), c);
     }
     __syncthreads();
   }
@@ -563,19 +904,6 @@ __device__ void cholesky_body(int S, double* A, int lda, int* flag) {
   }
 }
 
-
-// working set of syevk_body in doubles (matrix, tridiagonal, reflector,
-// products, eigenvalues, float32 copy, cluster indices); shared memory when
-// S <= kSmemMax
-__host__ __device__ constexpr size_t syevk_work_doubles(int n) {
-  return (size_t)n * (n + 1) / 2 + (size_t)(5 + kSeg) * n + 2 * (size_t)n;
-}
-// global scratch of syevk_body: the working set past kSmemMax, the
-// reflectors (S x S), then eigenvectors and inverse-iteration LU rows (6 S per
-// vector) when they do not fit in the freed shared-memory matrix area
-__host__ __device__ constexpr size_t syevk_scratch_doubles(int S, int k) {
-  return (S <= kSmemMax ? 0 : syevk_work_doubles(S)) + (size_t)S * S + (size_t)k * 6 * S + 64;
-}
 
 }  // namespace
 }  // namespace xs
