@@ -116,12 +116,15 @@ __global__ void resid_kernel(long long len, const double* __restrict__ A, const 
   }
 }
 
+// one warp per row: partials strided over the lanes, then a fixed tree (one
+// thread per row, adding 256 partials at 64 cycles each, took 15 us)
 __global__ void sum_sqrt_kernel(int nvec, int nblocks, const double* __restrict__ part, double* out) {
-  int k = blockIdx.x * blockDim.x + threadIdx.x;
+  const int k = blockIdx.x * (blockDim.x >> 5) + (threadIdx.x >> 5), lane = threadIdx.x & 31;
   if (k >= nvec) return;
   double s = 0.0;
-  for (int b = 0; b < nblocks; ++b) s += part[(long long)k * nblocks + b];
-  out[k] = sqrt(s);
+  for (int b = lane; b < nblocks; b += 32) s += part[(long long)k * nblocks + b];
+  s = warp_sum(s);
+  if (lane == 0) out[k] = sqrt(s);
 }
 
 __global__ void sqrt_kernel(int n, double* x) {
@@ -234,13 +237,17 @@ void precondition(cudaStream_t s, int nvec, int o, int v, const double* eps, con
 void residual_norms(cudaStream_t s, int nvec, long long len, const double* A, const double* B, const double* omega,
                     double* out_norm, double* R) {
   if (nvec == 0) return;
-  const int blocks = static_cast<int>(std::min<long long>(256, (len + 255) / 256));
+  // about 8 CTAs per SM over all rows, at least 2048 elements per CTA: a CTA's
+  // reduction costs eleven float64 adds per warp, so CTAs of one or two elements a
+  // thread spend their time there (10 rows of 90000: 17 us with 256 CTAs a row)
+  const int blocks = static_cast<int>(
+      std::max<long long>(1, std::min<long long>((8LL * 152 + nvec - 1) / nvec, (len + 2047) / 2048)));
   static thread_local DevBuf<double> part;
   part.ensure((size_t)nvec * blocks);
   ProfScope ps(s, "resid_norms", 8.0 * nvec * len * (B ? 2.0 : 1.0) + (R ? 8.0 * nvec * len : 0.0), 0.0);
   resid_kernel<<<dim3(blocks, nvec), 256, 0, s>>>(len, A, B, omega, part.get(), R);
   XS_CHECK_LAUNCH();
-  sum_sqrt_kernel<<<grid1(nvec, 64), 64, 0, s>>>(nvec, blocks, part.get(), out_norm);
+  sum_sqrt_kernel<<<grid1(nvec, 8), 256, 0, s>>>(nvec, blocks, part.get(), out_norm);
   XS_CHECK_LAUNCH();
 }
 
