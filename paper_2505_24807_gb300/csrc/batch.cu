@@ -40,6 +40,7 @@
 #include "gbuild_dev.cuh"
 #include "gpair_dev.cuh"
 #include "jacobi.cuh"
+#include "orth.cuh"
 #include "kernels.h"
 #include "mlp.h"
 #include "syev_body.cuh"
@@ -1069,7 +1070,9 @@ __global__ void __launch_bounds__(512) beig_kernel(const BMol* __restrict__ mols
   }
 }
 
-// Loewdin factor of the Gram matrix G (n x n, row stride ldg): eigenvalues
+// Orthonormalising factor of the Gram matrix G (n x n, row stride ldg): the
+// triangular one (orth.cuh, transposed) where the rows are well apart, else
+// Loewdin's: eigenvalues
 // above thresh * max(lambda_max, 1) kept from the largest down; B[s][q] =
 // Q[s][j_q] / sqrt(lambda_{j_q}) (row stride ldb); returns the count.  One
 // CTA, matrices up to 32 x 32 in shared memory.
@@ -1078,11 +1081,24 @@ __device__ int lowdin_block(int nd, const double* G, int ldg, double* B, int ldb
   __shared__ double lam[32];
   __shared__ int ord[32], nkeep;
   const int tid = threadIdx.x, nt = blockDim.x;
-  for (int idx = tid; idx < nd * nd; idx += nt) {
-    const int i = idx / nd, j = idx - i * nd;
-    As[i * 33 + j] = 0.5 * (G[(size_t)i * ldg + j] + G[(size_t)j * ldg + i]);
+  auto load = [&]() {
+    for (int idx = tid; idx < nd * nd; idx += nt) {
+      const int i = idx / nd, j = idx - i * nd;
+      As[i * 33 + j] = 0.5 * (G[(size_t)i * ldg + j] + G[(size_t)j * ldg + i]);
+    }
+    __syncthreads();
+  };
+  load();
+  if (gram_inverse_factor(nd, As, Vs, 33)) {
+    for (int idx = tid; idx < nd * nd; idx += nt) {
+      const int s = idx / nd, q = idx - s * nd;
+      B[(size_t)s * ldb + q] = Vs[q * 33 + s];
+    }
+    __syncthreads();
+    return nd;
   }
   __syncthreads();
+  load();
   jacobi_sweeps(nd, As, 33, Vs, 33, scr, 64);
   __syncthreads();
   if (tid == 0) {

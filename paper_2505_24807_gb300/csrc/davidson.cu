@@ -183,8 +183,8 @@ __global__ void inv_norms_kernel(int n, const double* __restrict__ nrm, double* 
 }
 
 // Orthonormalise the nnew rows of T against V[0:S] (classical Gram-Schmidt,
-// repeated when the first pass cancels much of a row) and among themselves (Loewdin, dropping directions whose Gram
-// eigenvalue is below kLowdinThresh); writes the kept rows to Vout (and,
+// repeated when the first pass cancels much of a row) and among themselves (triangular factors, or Loewdin's where
+// they are nearly dependent, dropping directions whose Gram eigenvalue is below kLowdinThresh); writes the kept rows to Vout (and,
 // on the tensor-core subspace, their maxima to vmax when given).
 int orthonormalise_append(Ctx& c, Work& w, int S, int nnew, long long ov, double* Vout,
                           unsigned int* vmax = nullptr) {
@@ -226,11 +226,11 @@ int orthonormalise_append(Ctx& c, Work& w, int S, int nnew, long long ov, double
     gram<double>(s, nnew, nnew, static_cast<int>(ov), w.T.get(), static_cast<int>(ov), w.T.get(),
                  static_cast<int>(ov), w.E2.get(), nnew, 1.0, 0.0, w.gws);
   }
-  // Gram matrices of nearly dependent directions have eigenvalues spread over
-  // many decades; two-sided Jacobi resolves the small ones to high relative
-  // accuracy, which the Loewdin factors 1/sqrt(lambda) need
-  jacobi_eig(s, nnew, w.E2.get(), nnew, w.Q2.get(), nnew, w.w2.get(), w.flag.get() + 1);
-  lowdin(s, nnew, w.w2.get(), w.Q2.get(), nnew, kLowdinThresh, w.Bm.get(), nnew, w.flag.get() + 2);
+  // triangular factors; Gram matrices of nearly dependent directions have
+  // eigenvalues spread over many decades: two-sided Jacobi resolves the small
+  // ones to high relative accuracy, which the Loewdin factors 1/sqrt(lambda) need
+  orthonormaliser(s, nnew, w.E2.get(), nnew, w.Q2.get(), nnew, w.w2.get(), kLowdinThresh, w.Bm.get(), nnew,
+                  w.flag.get() + 2, w.flag.get() + 1);
   int nkeep = 0;
   sync_copy(s, &nkeep, w.flag.get() + 2, sizeof(int));
   if (nkeep > 0) {
@@ -791,8 +791,8 @@ int davidson(Ctx& c, DevMol& m, const xs_ex_opts& opt, SolveStats& st) {
         // Gram (2k x 2k) of the coefficient columns
         gemm<double>(s, true, false, 2 * k, 2 * k, S, 1.0, w.tS.get(), 2 * k, 0, w.tS.get(), 2 * k, 0, 0.0,
                      w.E2.get(), 2 * k, 0, 1);
-        jacobi_eig(s, 2 * k, w.E2.get(), 2 * k, w.Q2.get(), 2 * k, w.w2.get(), w.flag.get() + 1);
-        lowdin(s, 2 * k, w.w2.get(), w.Q2.get(), 2 * k, kLowdinThresh, w.Bm.get(), 2 * k, w.flag.get() + 2);
+        orthonormaliser(s, 2 * k, w.E2.get(), 2 * k, w.Q2.get(), 2 * k, w.w2.get(), kLowdinThresh, w.Bm.get(), 2 * k,
+                        w.flag.get() + 2, w.flag.get() + 1);
         sync_copy(s, &nc, w.flag.get() + 2, sizeof(int));
         // Cn = Ycoef Bm^T (S x nc)
         gemm<double>(s, false, true, S, nc, 2 * k, 1.0, w.tS.get(), 2 * k, 0, w.Bm.get(), 2 * k, 0, 0.0, w.E.get(),

@@ -11,6 +11,7 @@
 #include "small.h"
 #include "prof.h"
 #include "jacobi.cuh"
+#include "orth.cuh"
 
 namespace xs {
 
@@ -53,9 +54,9 @@ __global__ void __launch_bounds__(1024) jacobi_kernel(int n, double* A, int lda,
 // unchanged.
 constexpr int kJacobiSmemMax = 64;
 
-__global__ void __launch_bounds__(256) jacobi_smem_kernel(int n, const double* __restrict__ A, int lda,
-                                                          double* __restrict__ V, int ldv, double* __restrict__ w,
-                                                          int* info, int max_sweeps) {
+// the eigen-decomposition in shared memory (V, w in global memory)
+__device__ void jacobi_smem_body(int n, const double* __restrict__ A, int lda, double* __restrict__ V, int ldv,
+                                 double* __restrict__ w, int* info, int max_sweeps) {
   extern __shared__ double sh[];
   const int ld = n + 1;
   const int m = n + (n & 1);
@@ -90,6 +91,12 @@ __global__ void __launch_bounds__(256) jacobi_smem_kernel(int n, const double* _
   if (tid == 0 && info) *info = (sweep >= max_sweeps) ? 1 : 0;
 }
 
+__global__ void __launch_bounds__(256) jacobi_smem_kernel(int n, const double* __restrict__ A, int lda,
+                                                          double* __restrict__ V, int ldv, double* __restrict__ w,
+                                                          int* info, int max_sweeps) {
+  jacobi_smem_body(n, A, lda, V, ldv, w, info, max_sweeps);
+}
+
 // E[i][j] = a[min(i,j)][max(i,j)]: full symmetric copy from the valid upper part
 __global__ void sym_upper_kernel(int S, const double* __restrict__ a, int lda, double* __restrict__ E, int lde) {
   int idx = blockIdx.x * blockDim.x + threadIdx.x;
@@ -112,8 +119,8 @@ __global__ void scale_cols_kernel(int rows, int ncols, double* A, int lda, const
 // Loewdin canonical orthonormalisation coefficients: eigenpairs (lam, Q) of a
 // Gram matrix (ascending); keep lam > thresh * max(lam, 1) and write
 // B[k][:] = Q[:, j]^T / sqrt(lam_j) for the kept j (largest first).
-__global__ void lowdin_kernel(int n, const double* __restrict__ lam, const double* __restrict__ Q, int ldq,
-                              double thresh, double* __restrict__ Bm, int ldb, int* nkeep) {
+__device__ void lowdin_body(int n, const double* lam, const double* Q, int ldq, double thresh, double* Bm, int ldb,
+                            int* nkeep) {
   __shared__ int first;
   if (threadIdx.x == 0) {
     double lmax = lam[n - 1] > 1.0 ? lam[n - 1] : 1.0;
@@ -131,6 +138,38 @@ __global__ void lowdin_kernel(int n, const double* __restrict__ lam, const doubl
     int j = n - 1 - k;
     Bm[(long long)k * ldb + i] = Q[(long long)i * ldq + j] / sqrt(lam[j]);
   }
+}
+
+__global__ void lowdin_kernel(int n, const double* lam, const double* Q, int ldq, double thresh, double* Bm, int ldb,
+                              int* nkeep) {
+  lowdin_body(n, lam, Q, ldq, thresh, Bm, ldb, nkeep);
+}
+
+// Coefficients B with B G B^T = I for the Gram matrix A of n <= kJacobiSmemMax
+// rows: the inverse Cholesky factor when the rows are well apart (orth.cuh),
+// else the Loewdin factors of the Jacobi eigen-decomposition, which drop
+// directions below thresh.
+__global__ void __launch_bounds__(256) orth_kernel(int n, const double* __restrict__ A, int lda, double* V, int ldv,
+                                                   double* w, double thresh, double* Bm, int ldb, int* nkeep,
+                                                   int* info, int max_sweeps) {
+  extern __shared__ double sh[];
+  const int ld = n + 1;
+  double* As = sh;
+  double* Bs = As + (size_t)n * ld;
+  for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) As[(idx / n) * ld + idx % n] = A[(long long)(idx / n) * lda + idx % n];
+  __syncthreads();
+  if (gram_inverse_factor(n, As, Bs, ld)) {
+    for (int idx = threadIdx.x; idx < n * n; idx += blockDim.x) {
+      const int i = idx / n, j = idx % n;
+      Bm[(long long)i * ldb + j] = Bs[i * ld + j];
+    }
+    if (threadIdx.x == 0) *nkeep = n;
+    return;
+  }
+  __syncthreads();
+  jacobi_smem_body(n, A, lda, V, ldv, w, info, max_sweeps);
+  __syncthreads();
+  lowdin_body(n, w, V, ldv, thresh, Bm, ldb, nkeep);
 }
 
 // omega[j] = sqrt(w2[j]) for j < k; flag[0] = 1 if any w2 <= 0
@@ -185,6 +224,28 @@ void jacobi_eig(cudaStream_t s, int n, double* A, int lda, double* V, int ldv, d
   size_t smem2 = sizeof(double) * n + sizeof(int) * n;
   if (smem2 > smem) smem = smem2;
   jacobi_kernel<<<1, 1024, smem, s>>>(n, A, lda, V, ldv, w, info, 60);
+  XS_CHECK_LAUNCH();
+}
+
+void orthonormaliser(cudaStream_t s, int n, double* G, int ldg, double* V, int ldv, double* w, double thresh,
+                     double* Bm, int ldb, int* nkeep, int* info) {
+  if (n <= 0) return;
+  if (n > kJacobiSmemMax) {
+    jacobi_eig(s, n, G, ldg, V, ldv, w, info);
+    lowdin(s, n, w, V, ldv, thresh, Bm, ldb, nkeep);
+    return;
+  }
+  ProfScope ps(s, "orth_f64", 0.0, 0.0);
+  const int m = n + (n & 1);
+  const size_t smem = sizeof(double) * (2 * (size_t)n * (n + 1) + 2 * m) + sizeof(int) * n;
+  static const bool attr = [] {   // once per process (thread-safe initialisation)
+    const size_t most = sizeof(double) * (2 * (size_t)kJacobiSmemMax * (kJacobiSmemMax + 1) + 2 * kJacobiSmemMax) +
+                        sizeof(int) * kJacobiSmemMax;
+    XS_CUDA(cudaFuncSetAttribute(orth_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most)));
+    return true;
+  }();
+  (void)attr;
+  orth_kernel<<<1, 256, smem, s>>>(n, G, ldg, V, ldv, w, thresh, Bm, ldb, nkeep, info, 60);
   XS_CHECK_LAUNCH();
 }
 

@@ -7,6 +7,7 @@
 #include <cfloat>
 
 #include "common.cuh"
+#include "f64_estimates.cuh"
 
 namespace xs {
 namespace {
@@ -38,66 +39,6 @@ __device__ double block_sum(double x, double* red) {
   }
   __syncthreads();
   return red[32];
-}
-
-// |x| as an integer that orders like it: comparisons stay off the float64 pipe
-__device__ __forceinline__ long long mag_bits(double x) { return __double_as_longlong(x) & 0x7FFFFFFFFFFFFFFFll; }
-
-// float32 of a double and back by their fields (the conversion instructions run
-// on the float64 pipe, 64 cycles each), for 2^-120 < |x| < 2^120
-__device__ __forceinline__ bool float_range(double x) {
-  const int e = (__double2hiint(x) >> 20) & 0x7FF;
-  return e > 1023 - 120 && e < 1023 + 120;
-}
-__device__ __forceinline__ float narrow_bits(double x) {
-  const unsigned hi = static_cast<unsigned>(__double2hiint(x)), lo = static_cast<unsigned>(__double2loint(x));
-  return __uint_as_float((hi & 0x80000000u) | (((hi & 0x7FFFFFFFu) - (896u << 20)) << 3) | (lo >> 29));
-}
-__device__ __forceinline__ double widen_bits(float x) {
-  const unsigned u = __float_as_uint(x);
-  return __hiloint2double(static_cast<int>((u & 0x80000000u) | (((u & 0x7FFFFFFFu) >> 3) + (896u << 20))),
-                          static_cast<int>(u << 29));
-}
-__device__ __forceinline__ float rcp_estimate(float x) {
-  float r;
-  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-__device__ __forceinline__ float rsqrt_estimate(float x) {
-  float r;
-  asm("rsqrt.approx.ftz.f32 %0, %1;" : "=f"(r) : "f"(x));
-  return r;
-}
-
-// reciprocal to ~1e-14 relative: a float32 estimate refined by one Newton
-// step (inverse iteration needs directions, not correctly rounded quotients)
-__device__ __forceinline__ double rcp_fast(double x) {
-  if (!float_range(x)) return 1.0 / x;
-  const double r = widen_bits(rcp_estimate(narrow_bits(x)));
-  return r * fma(-x, r, 2.0);
-}
-
-// square root, its reciprocal and the reciprocal to rounding (x > 0 for the
-// roots): float32 estimates with one third-order correction each, whose
-// remainder is 2^-66 relative
-__device__ __forceinline__ double sqrt_fast(double x) {
-  if (!float_range(x)) return sqrt(x);
-  const double r = widen_bits(rsqrt_estimate(narrow_bits(x)));
-  const double t = x * r;
-  const double e = fma(-t, r, 1.0);
-  return fma(t, e * fma(0.375, e, 0.5), t);
-}
-__device__ __forceinline__ double rsqrt_full(double x) {
-  if (!float_range(x)) return 1.0 / sqrt(x);
-  const double r = widen_bits(rsqrt_estimate(narrow_bits(x)));
-  const double e = fma(-(x * r), r, 1.0);
-  return fma(r, e * fma(0.375, e, 0.5), r);
-}
-__device__ __forceinline__ double rcp_full(double x) {
-  if (!float_range(x)) return 1.0 / x;
-  const double r = widen_bits(rcp_estimate(narrow_bits(x)));
-  const double e = fma(-x, r, 1.0);
-  return fma(r, fma(e, e, e), r);
 }
 
 // Sum of a warp's 32 values off the float64 pipe (a shuffle tree of adds takes
