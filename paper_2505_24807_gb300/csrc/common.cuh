@@ -92,6 +92,7 @@ struct DevMol {
   std::shared_ptr<void> mg_orb;  // residue operands of the orbitals for the float64 products (products.cu)
   DevBuf<double> dip;            // MO dipole integrals <i|r_x|a>, 3 x nocc x nvir (lazily)
   DevBuf<int> gb_rows, gb_cols;  // atom-aligned G tiles (first AO, count, first atom, end atom)
+  DevBuf<int> gb_prod;           // int2 per on-atom product: its two AOs
   int gb_nrows = 0, gb_ncols = 0;
   DevBuf<int> gp_sa, gp_pairs;   // super-atoms (int4) and unordered super-atom pairs (int2) of the float32 G build
   int gp_nsa = 0, gp_npairs = 0;

@@ -24,9 +24,8 @@ __device__ __forceinline__ int pidx(int a, int b) {
   return ((lo * (9 - lo)) >> 1) + (hi - lo);
 }
 
-// product vectors of the diagonal atom blocks: r[q][v] (TR = false) or its
-// transpose r[v][q] (TR = true, the operand of the split-K product W r)
-template <typename T, bool TR>
+// product vectors of the diagonal atom blocks, r[q][v]
+template <typename T>
 __global__ void pack_diag_kernel(int natoms, int n, int np, int nvec, const int* __restrict__ atom_ao_off,
                                  const int* __restrict__ atom_nao, const int* __restrict__ atom_prod_off,
                                  const T* __restrict__ R, T* __restrict__ r) {
@@ -36,7 +35,7 @@ __global__ void pack_diag_kernel(int natoms, int n, int np, int nvec, const int*
   for (; v < nvec; v += blockDim.x) {
     const T* Rv = R + (long long)v * n * n;
     int o = atom_ao_off[A], P = atom_prod_off[A];
-    auto at = [&](int q) -> T& { return TR ? r[(long long)v * np + q] : r[(long long)q * nvec + v]; };
+    auto at = [&](int q) -> T& { return r[(long long)q * nvec + v]; };
     if (atom_nao[A] == 1) {
       at(P) = Rv[(long long)o * n + o];
     } else {

@@ -41,7 +41,7 @@ inline GMode gmode(bool rpa, bool triplet) {
 // nvec AO matrices R (n x n each, row-major, consecutive) -> G (CIS/Fock:
 // 2J(R) - K(R)) or G+ = 4J(Rs) - 2K(Rs) and G- = -2K(Ra) (RPA).
 // Gm is unused for G_CIS; in the TDHF modes either output may be null (not
-// formed).  ws: scratch of at least 2 * np * nvec.
+// formed).  ws: scratch, grown as needed.
 template <typename T>
 void gbuild(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const T* R,
             T* G, T* Gm, DevBuf<T>& ws);
@@ -73,9 +73,8 @@ void gpair_build_split(cudaStream_t s, const DevMol& m, const double* d_par, GMo
                        const float* J2, int ldj, const float* R, float* Gh, float* Gl, float* Gmh, float* Gml,
                        int ldo);
 // The same with caller-provided scratch: r and J2 of np * nvec elements each.
-template <typename T>
-void gbuild_raw(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const T* R, T* G,
-                T* Gm, T* r, T* J2);
+void gbuild_raw(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const double* R, double* G,
+                double* Gm, double* r, double* J2);
 
 // ---- elementwise helpers (vec.cu) ---------------------------------------------
 template <typename T>
