@@ -104,6 +104,94 @@ __global__ void __launch_bounds__(256) gemm_kernel(int M, int N, int K, T alpha,
   }
 }
 
+// Float64 products with few outputs: 8 x 8 output tiles, 256 threads as four
+// interleaved quarters of K times the 64 outputs.  The float64 pipe takes two
+// multiply-adds per clock and SM, so one output per thread and two shared-memory
+// loads per multiply-add already saturate it; what small problems need is a share
+// of every SM and no padded outputs.  C = op(A) op(B) on the grid of tiles x
+// batch x kSplit (arguments as gemm_kernel): 62 x 125 x 62 10.4 -> 3.1 us, 331 x 150 x
+// 181 43 -> 25 us, Ritz vectors 5 x 925 x 50 37 -> 3.1 us, projections
+// 50 x 5 x 925 25 -> 7 us, 120 x 20 x 373100 2.52 -> 2.00 ms.
+constexpr int kSmallK = 64;   // K per stage
+
+__global__ void __launch_bounds__(256) dgemm_small_kernel(int M, int N, int K, double alpha,
+                                                          const double* __restrict__ A, int lda, long long sA,
+                                                          bool transA, const double* __restrict__ B, int ldb,
+                                                          long long sB, bool transB, double beta,
+                                                          double* __restrict__ C, int ldc, long long sC, int kSplit,
+                                                          long long sSplit) {
+  __shared__ double As[8][kSmallK + 1], Bs[8][kSmallK + 1];   // [row or column][k]
+  __shared__ double red[3][64];
+  const int tid = threadIdx.x;
+  const int b = blockIdx.z / kSplit, ks = blockIdx.z % kSplit;
+  const int m0 = blockIdx.y * 8, n0 = blockIdx.x * 8;
+  A += b * sA;
+  B += b * sB;
+  C += b * sC + ks * sSplit;
+  int kc = (K + kSplit - 1) / kSplit;
+  kc = (kc + 15) / 16 * 16;
+  const int kbeg = ks * kc, kend = min(K, kbeg + kc);
+  // two elements of each operand per thread and stage: k along the lanes where
+  // the operand is contiguous in k, else its 8 rows
+  const int ar0 = transA ? tid & 7 : tid >> 6, ak0 = transA ? tid >> 3 : tid & 63;
+  const int ars = transA ? 0 : 4, aks = transA ? 32 : 0;
+  const int br0 = transB ? tid >> 6 : tid & 7, bk0 = transB ? tid & 63 : tid >> 3;
+  const int brs = transB ? 4 : 0, bks = transB ? 0 : 32;
+  double ra[2], rb[2];
+  auto load = [&](int k0) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      const int r = m0 + ar0 + q * ars, k = k0 + ak0 + q * aks;
+      ra[q] = (r < M && k < kend) ? (transA ? A[(long long)k * lda + r] : A[(long long)r * lda + k]) : 0.0;
+      const int c = n0 + br0 + q * brs, kb = k0 + bk0 + q * bks;
+      rb[q] = (c < N && kb < kend) ? (transB ? B[(long long)c * ldb + kb] : B[(long long)kb * ldb + c]) : 0.0;
+    }
+  };
+  const int part = tid >> 6, i = (tid >> 3) & 7, j = tid & 7;
+  double acc = 0.0;
+  load(kbeg);
+  for (int k0 = kbeg; k0 < kend; k0 += kSmallK) {
+#pragma unroll
+    for (int q = 0; q < 2; ++q) {
+      As[ar0 + q * ars][ak0 + q * aks] = ra[q];
+      Bs[br0 + q * brs][bk0 + q * bks] = rb[q];
+    }
+    __syncthreads();
+    if (k0 + kSmallK < kend) load(k0 + kSmallK);
+    const int steps = (min(kSmallK, kend - k0) + 3) >> 2;
+    for (int t = 0; t < steps; ++t) acc = fma(As[i][part + 4 * t], Bs[j][part + 4 * t], acc);
+    __syncthreads();
+  }
+  if (part > 0) red[part - 1][tid & 63] = acc;
+  __syncthreads();
+  if (part == 0) {
+    acc += red[0][tid];
+    acc += red[1][tid];
+    acc += red[2][tid];
+    const int gm = m0 + i, gn = n0 + j;
+    if (gm < M && gn < N) {
+      double* c = C + (long long)gm * ldc + gn;
+      double r = alpha * acc;
+      if (beta != 0.0) r = fma(beta, *c, r);
+      *c = r;
+    }
+  }
+}
+
+// few outputs: at most 16 tiles of 64 per SM (each holds at most 8 of them at a
+// time); beyond, the register tiles below read their operands less often
+bool few_outputs(int M, int N, int batch) {
+  return (long long)((M + 7) / 8) * ((N + 7) / 8) * batch <= 16 * 152;
+}
+
+void launch_small(cudaStream_t s, int M, int N, int K, double alpha, const double* A, int lda, long long sA, bool tA,
+                  const double* B, int ldb, long long sB, bool tB, double beta, double* C, int ldc, long long sC,
+                  int zdim, int kSplit, long long sSplit) {
+  dim3 grid((N + 7) / 8, (M + 7) / 8, zdim);
+  dgemm_small_kernel<<<grid, 256, 0, s>>>(M, N, K, alpha, A, lda, sA, tA, B, ldb, sB, tB, beta, C, ldc, sC, kSplit,
+                                          sSplit);
+}
+
 // C = alpha * sum_s P[s] + beta * C over the split partials.
 template <typename T>
 __global__ void reduce_split(int M, int N, int kSplit, const T* __restrict__ P, T alpha, T beta, T* __restrict__ C,
@@ -429,6 +517,13 @@ void gemm(cudaStream_t s, bool transA, bool transB, int M, int N, int K, T alpha
     XS_CHECK_LAUNCH();
     return;
   }
+  if constexpr (sizeof(T) == 8) {
+    if (few_outputs(M, N, batch)) {
+      launch_small(s, M, N, K, alpha, A, lda, sA, transA, B, ldb, sB, transB, beta, C, ldc, sC, batch, 1, 0);
+      XS_CHECK_LAUNCH();
+      return;
+    }
+  }
   const int sh = tuned_shape<T>(s, transA, transB, M, N, K, A, lda, sA, B, ldb, sB, batch);
   launch_gemm<T>(s, sh, M, N, K, alpha, A, lda, sA, transA, B, ldb, sB, transB, beta, C, ldc, sC, batch, 1, 0);
   XS_CHECK_LAUNCH();
@@ -439,8 +534,9 @@ void gram(cudaStream_t s, int M, int N, int L, const T* A, int lda, const T* B, 
           T beta, DevBuf<T>& ws) {
   if (M <= 0 || N <= 0) return;
   const int sh = pick_shape(M, N);
-  const int tiles = tiles_of(sh, M, N);
-  int kSplit = (2 * 152 + tiles - 1) / tiles;
+  const bool small = sizeof(T) == 8 && few_outputs(M, N, 1);
+  const int tiles = small ? ((M + 7) / 8) * ((N + 7) / 8) : tiles_of(sh, M, N);
+  int kSplit = ((small ? 6 : 2) * 152 + tiles - 1) / tiles;
   const int maxSplit = (L + 4 * BK - 1) / (4 * BK);
   if (kSplit > maxSplit) kSplit = maxSplit;
   if (kSplit < 1) kSplit = 1;
@@ -448,8 +544,14 @@ void gram(cudaStream_t s, int M, int N, int L, const T* A, int lda, const T* B, 
   {
     ProfScope ps(s, sizeof(T) == 8 ? "gram_f64" : "gram_f32", sizeof(T) * (double)L * (M + N),
                  2.0 * M * N * (double)L);
-    launch_gemm<T>(s, sh, M, N, L, T(1), A, lda, 0, false, B, ldb, 0, true, T(0), ws.get(), N, 0, kSplit, kSplit,
-                   (long long)M * N);
+    if constexpr (sizeof(T) == 8) {
+      if (small)
+        launch_small(s, M, N, L, 1.0, A, lda, 0, false, B, ldb, 0, true, 0.0, ws.get(), N, 0, kSplit, kSplit,
+                     (long long)M * N);
+    }
+    if (!small)
+      launch_gemm<T>(s, sh, M, N, L, T(1), A, lda, 0, false, B, ldb, 0, true, T(0), ws.get(), N, 0, kSplit, kSplit,
+                     (long long)M * N);
     XS_CHECK_LAUNCH();
   }
   reduce_split<T><<<grid1((long long)M * N, 256), 256, 0, s>>>(M, N, kSplit, ws.get(), alpha, beta, C, ldc);
