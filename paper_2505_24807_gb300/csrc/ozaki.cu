@@ -592,8 +592,9 @@ void oz_exponents(cudaStream_t s, int nvec, long long L, const double* X, long l
   w.mx.ensure(nvec);
   XS_CUDA(cudaMemsetAsync(w.mx.get(), 0, sizeof(unsigned int) * nvec, s));
   if (L > 0) {
-    // about 8 CTAs per SM over all rows, at least 1024 amplitudes per CTA
-    const long long per_row = std::max<long long>(1, std::min<long long>((8LL * 152 + nvec - 1) / nvec, (L + 1023) / 1024));
+    // at most 8 CTAs per SM over all rows (one wave: a few CTAs past it doubled
+    // the time), at least 1024 amplitudes per CTA
+    const long long per_row = std::max<long long>(1, std::min<long long>(8LL * 152 / nvec, (L + 1023) / 1024));
     dim3 grid(static_cast<unsigned>(per_row), nvec);
     oz_absmax_kernel<<<grid, 256, 0, s>>>(L, X, ldx, w.mx.get());
     XS_CHECK_LAUNCH();
