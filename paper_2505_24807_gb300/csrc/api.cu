@@ -151,6 +151,9 @@ void invalidate_mixed(DevMol& m) {
   m.CTf_hi.release();
   m.CTf_lo.release();
   m.CTf.release();
+  m.CTh_hi.release();
+  m.CTh_lo.release();
+  m.CTh_e.release();
   m.mg_orb.reset();
 }
 

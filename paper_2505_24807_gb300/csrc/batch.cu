@@ -527,7 +527,7 @@ __global__ void __launch_bounds__(256, 2) bgpair_kernel(const BMol* __restrict__
     const int t = (u - pref[m]) * 256 + threadIdx.x;
     if (t >= d.gp_npairs) continue;
     PairOut o{static_cast<float*>(d.Gp), static_cast<float*>(d.Gq), nullptr, nullptr, nullptr, nullptr, 0};
-    gpair_one<static_cast<GMode>(MODE), false>(d.n, d.np, sf(st, m, F_NNEW), d.gp_pairs[t], d.gp_sa, par,
+    gpair_one<static_cast<GMode>(MODE), kPlain>(d.n, d.np, sf(st, m, F_NNEW), d.gp_pairs[t], d.gp_sa, par,
                                                 static_cast<const float*>(d.W), static_cast<const float*>(d.J2),
                                                 d.pmax, static_cast<const float*>(d.Rm), o, wsm + threadIdx.x * 100);
   }

@@ -2,6 +2,7 @@
 // buffers, per-molecule device state and the context.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <cstdio>
@@ -88,6 +89,9 @@ struct DevMol {
   DevBuf<double> CT;      // MO coefficients, MO-major: CT[p * n + mu] = C[mu][p]
   DevBuf<double> eps;     // n orbital energies
   DevBuf<float> CTf_hi, CTf_lo;  // TF32-pair operand copies of CT for the tensor-core path
+  DevBuf<__half> CTh_hi, CTh_lo; // float16-pair operand copies of CT, with their exponent and the largest |W| (abs_hi)
+  DevBuf<int> CTh_e;
+  DevBuf<unsigned int> w_max;
   DevBuf<float> CTf;             // float32 copy of CT for the float32 SIMT products
   std::shared_ptr<void> mg_orb;  // residue operands of the orbitals for the float64 products (products.cu)
   DevBuf<double> dip;            // MO dipole integrals <i|r_x|a>, 3 x nocc x nvir (lazily)

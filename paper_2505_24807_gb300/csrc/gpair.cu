@@ -33,7 +33,7 @@ namespace {
 
 constexpr int kPairThreads = 256;
 
-template <GMode MODE, bool SPLIT, int OUT>
+template <GMode MODE, int SPLIT, int OUT>
 __global__ void __launch_bounds__(kPairThreads, 2) gpair_kernel(int n, int np, int nvec, int npairs,
                                                                 const int2* __restrict__ pairs,
                                                                 const int4* __restrict__ sa,
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(kPairThreads, 2) gpair_kernel(int n, int np, i
   gpair_one<MODE, SPLIT, OUT>(n, np, nvec, pairs[t], sa, par, W, J2, ldj, R, o, wsm + threadIdx.x * 100);
 }
 
-template <GMode MODE, bool SPLIT, int OUT>
+template <GMode MODE, int SPLIT, int OUT>
 void launch_mode(cudaStream_t s, const DevMol& m, const double* d_par, int nvec, const float* W, const float* J2,
                  int ldj, const float* R, const PairOut& o) {
   const size_t smem = sizeof(float) * 100 * kPairThreads;
@@ -64,10 +64,11 @@ void launch_mode(cudaStream_t s, const DevMol& m, const double* d_par, int nvec,
   XS_CHECK_LAUNCH();
 }
 
-template <bool SPLIT>
+template <int SPLIT>
 void launch_pairs(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const float* W,
                   const float* J2, int ldj, const float* R, const PairOut& o) {
-  const bool plus = SPLIT ? o.Gh != nullptr : o.G != nullptr, minus = SPLIT ? o.Gmh != nullptr : o.Gm != nullptr;
+  const bool plus = SPLIT == kHalfPair ? o.Hh != nullptr : (SPLIT == kTf32Pair ? o.Gh != nullptr : o.G != nullptr);
+  const bool minus = SPLIT == kHalfPair ? o.Hmh != nullptr : (SPLIT == kTf32Pair ? o.Gmh != nullptr : o.Gm != nullptr);
 #define XS_PAIRS(MODE, OUT) launch_mode<MODE, SPLIT, OUT>(s, m, d_par, nvec, W, J2, ldj, R, o)
   if (mode == G_CIS) XS_PAIRS(G_CIS, kOutPlus);
   else if (mode == G_CIS_T) XS_PAIRS(G_CIS_T, kOutPlus);
@@ -123,6 +124,49 @@ __global__ void j2_reduce_kernel(int np, int nvec, int nchunk, const float* __re
   J2[idx] = s;
 }
 
+// Exponents of the float16 pairs of G and G-, one CTA per matrix: a bound of
+// |G| from the largest |R| (bits in rmax), the largest |J2| of the matrix and the
+// largest integral w (two-centre products, abs_hi in wmax, and one-centre
+// parameters): the exchange of a block sums at most 16 products w R, the
+// one-centre Coulomb and exchange 4, G+ twice and four times those.
+__global__ void __launch_bounds__(256) g_exponents_kernel(int np, int nvec, const float* __restrict__ J2, int ldj,
+                                                          const unsigned int* __restrict__ rmax,
+                                                          const unsigned int* __restrict__ wmax,
+                                                          const double* __restrict__ par, int* __restrict__ e,
+                                                          int* __restrict__ em) {
+  __shared__ unsigned int top;
+  const int v = blockIdx.x;
+  if (threadIdx.x == 0) top = 0;
+  __syncthreads();
+  unsigned int j = 0;
+  if (J2)
+    for (int q = threadIdx.x; q < np; q += blockDim.x) j = max(j, __float_as_uint(J2[(long long)q * ldj + v]) & 0x7FFFFFFFu);
+  j = __reduce_max_sync(0xffffffffu, j);
+  if ((threadIdx.x & 31) == 0) atomicMax(&top, j);
+  __syncthreads();
+  if (threadIdx.x > 0) return;
+  float w = static_cast<float>(__hiloint2double(static_cast<int>(*wmax + 1), 0));
+  for (int z = 0; z < XS_NELEM; ++z)
+    for (int q = 4; q <= 8; ++q) w = fmaxf(w, fabsf(static_cast<float>(par[z * XS_NPARAM + q])));
+  const float r = __uint_as_float(rmax[v]), jm = __uint_as_float(top);
+  auto exponent = [](float bound) {          // bound < 2^(e + 15)
+    const int ex = static_cast<int>(__float_as_uint(bound) >> 23);
+    return ex == 0 || ex == 0xFF ? 0 : ex - 127 - 14;
+  };
+  // rounding of the sums stays far below the factor 48 / 32 over the exchange alone
+  if (e) e[v] = exponent(48.0f * w * r + 4.0f * jm);
+  if (em) em[v] = exponent(33.0f * w * r);
+}
+
+__global__ void zero_pad_half_kernel(int rows, int n, int ldo, int nvec, __half* a, __half* b) {
+  const int w = ldo - n;
+  const long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  if (idx >= (long long)nvec * rows * w) return;
+  const long long at = (idx / w) * ldo + n + idx % w;
+  a[at] = __float2half_rn(0.0f);
+  b[at] = __float2half_rn(0.0f);
+}
+
 }  // namespace
 
 void build_gpairs(cudaStream_t s, DevMol& m) {
@@ -175,14 +219,44 @@ void coulomb_j2(cudaStream_t s, int np, int nvec, const float* W, const float* r
 void gpair_build(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const float* W,
                  const float* J2, int ldj, const float* R, float* G, float* Gm) {
   PairOut o{G, Gm, nullptr, nullptr, nullptr, nullptr, 0};
-  launch_pairs<false>(s, m, d_par, mode, nvec, W, J2, ldj, R, o);
+  launch_pairs<kPlain>(s, m, d_par, mode, nvec, W, J2, ldj, R, o);
 }
 
 void gpair_build_split(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const float* W,
                        const float* J2, int ldj, const float* R, float* Gh, float* Gl, float* Gmh, float* Gml,
                        int ldo) {
   PairOut o{nullptr, nullptr, Gh, Gl, Gmh, Gml, ldo};
-  launch_pairs<true>(s, m, d_par, mode, nvec, W, J2, ldj, R, o);
+  launch_pairs<kTf32Pair>(s, m, d_par, mode, nvec, W, J2, ldj, R, o);
+}
+
+void gbuild_half(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const float* R,
+                 const unsigned int* rmax, const unsigned int* wmax, const GHalf& o, int ldo, DevBuf<float>& ws) {
+  if (nvec <= 0) return;
+  const int n = m.n, np = m.np;
+  ws.ensure((size_t)2 * np * nvec);
+  float* r = ws.get();
+  float* J2 = r + (size_t)np * nvec;
+  const bool coulomb = (mode == G_CIS || mode == G_RPA) && o.h;   // G- has no Coulomb part
+  if (coulomb) {
+    pack_diag_kernel<float><<<(m.L.natoms + 31) / 32, dim3(8, 32), 0, s>>>(
+        m.L.natoms, n, np, nvec, m.atom_ao_off.get(), m.atom_nao.get(), m.atom_prod_off.get(), R, r);
+    XS_CHECK_LAUNCH();
+    static thread_local DevBuf<float> j2_ws;
+    coulomb_j2(s, np, nvec, m.Wf.get(), r, J2, j2_ws);
+  }
+  g_exponents_kernel<<<nvec, 256, 0, s>>>(np, nvec, coulomb ? J2 : nullptr, nvec, rmax, wmax, d_par, o.e, o.em);
+  XS_CHECK_LAUNCH();
+  if (ldo > n) {
+    const long long cnt = (long long)nvec * n * (ldo - n);
+    if (o.h) zero_pad_half_kernel<<<grid1(cnt, 256), 256, 0, s>>>(n, n, ldo, nvec, o.h, o.l);
+    if (o.mh) zero_pad_half_kernel<<<grid1(cnt, 256), 256, 0, s>>>(n, n, ldo, nvec, o.mh, o.ml);
+    XS_CHECK_LAUNCH();
+  }
+  PairOut p{nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, ldo, o.h, o.l, o.mh, o.ml, o.e, o.em};
+  // algorithmic traffic: read R, write the float16 pairs, read the pair integrals once
+  const double outs = (o.h ? 1.0 : 0.0) + (o.mh ? 1.0 : 0.0);
+  ProfScope ps(s, "gbuild_assemble_f32", 4.0 * ((double)nvec * n * n * (1.0 + outs) + (double)np * np), 0.0);
+  launch_pairs<kHalfPair>(s, m, d_par, mode, nvec, m.Wf.get(), J2, nvec, R, p);
 }
 
 }  // namespace xs

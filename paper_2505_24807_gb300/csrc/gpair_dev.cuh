@@ -3,6 +3,7 @@
 // molecule per launch) and batch.cu (all molecules of a batch per launch).
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -33,11 +34,40 @@ struct PairOut {
   float *G, *Gm;                 // plain outputs (row stride n)
   float *Gh, *Gl, *Gmh, *Gml;    // TF32 pairs (row stride ldo)
   int ldo;
+  // float16 pairs of G 2^-e[matrix], G- 2^-em[matrix] (row stride ldo)
+  __half *Hh = nullptr, *Hl = nullptr, *Hmh = nullptr, *Hml = nullptr;
+  const int *e = nullptr, *em = nullptr;
 };
 
-template <bool SPLIT, bool RPA, int OUT>
-__device__ __forceinline__ void put(const PairOut& o, int n, long long vb, int row, int col, float g, float gm) {
-  if (SPLIT) {
+// forms of the outputs (template parameter SPLIT)
+constexpr int kPlain = 0, kTf32Pair = 1, kHalfPair = 2;
+
+// float16 pair of x f1 f2 (a power of two in two factors), the value below 2^15
+__device__ __forceinline__ void half_split(float x, float f1, float f2, __half& hi, __half& lo) {
+  x = x * f1 * f2;
+  hi = __float2half_rn(x);
+  lo = __float2half_rn(x - __half2float(hi));
+}
+__device__ __forceinline__ void pow2_factors(int e, float& f1, float& f2) {   // 2^-e, |e| <= 250
+  f1 = __int_as_float((-e / 2 + 127) << 23);
+  f2 = __int_as_float((-e - (-e / 2) + 127) << 23);
+}
+
+template <int SPLIT, bool RPA, int OUT>
+__device__ __forceinline__ void put(const PairOut& o, int n, int v, int row, int col, float g, float gm) {
+  const long long vb = v * static_cast<long long>(n);
+  if (SPLIT == kHalfPair) {
+    const long long at = vb * o.ldo + (long long)row * o.ldo + col;
+    float f1, f2;
+    if (!RPA || (OUT & kOutPlus)) {
+      pow2_factors(o.e[v], f1, f2);
+      half_split(g, f1, f2, o.Hh[at], o.Hl[at]);
+    }
+    if (RPA && (OUT & kOutMinus)) {
+      pow2_factors(o.em[v], f1, f2);
+      half_split(gm, f1, f2, o.Hmh[at], o.Hml[at]);
+    }
+  } else if (SPLIT == kTf32Pair) {
     const long long at = vb * o.ldo + (long long)row * o.ldo + col;
     float h, l;
     if (!RPA || (OUT & kOutPlus)) {
@@ -125,7 +155,33 @@ __device__ __forceinline__ void store4(float* base, long long ld, int row, int c
 
 // one output row segment (4 values): plain into A, or its TF32 pair into
 // A (hi) and B (lo)
-template <bool SPLIT>
+// four float16 pairs of g f1 f2 into H (hi) and L (lo)
+__device__ __forceinline__ void put_row_half(__half* H, __half* L, long long ld, int row, int cnt, bool vec,
+                                             const float (&g)[4], float f1, float f2) {
+  __half2 hh[2], ll[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    const float x = g[2 * j] * f1 * f2, y = g[2 * j + 1] * f1 * f2;
+    hh[j] = __floats2half2_rn(x, y);
+    const float2 f = __half22float2(hh[j]);
+    ll[j] = __floats2half2_rn(x - f.x, y - f.y);
+  }
+  H += row * ld;
+  L += row * ld;
+  if (vec) {
+    *reinterpret_cast<uint2*>(H) = *reinterpret_cast<uint2*>(hh);
+    *reinterpret_cast<uint2*>(L) = *reinterpret_cast<uint2*>(ll);
+  } else {
+#pragma unroll
+    for (int j = 0; j < 4; ++j)
+      if (j < cnt) {
+        H[j] = j & 1 ? __high2half(hh[j >> 1]) : __low2half(hh[j >> 1]);
+        L[j] = j & 1 ? __high2half(ll[j >> 1]) : __low2half(ll[j >> 1]);
+      }
+  }
+}
+
+template <int SPLIT>
 __device__ __forceinline__ void put_row(float* A, float* B, float* unused, long long ld, int row, int col, int cnt,
                                         bool vec, const float (&g)[4]) {
   (void)unused;
@@ -140,7 +196,7 @@ __device__ __forceinline__ void put_row(float* A, float* B, float* unused, long 
   }
 }
 
-template <GMode MODE, bool SPLIT, int OUT, bool HI, bool HJ>
+template <GMode MODE, int SPLIT, int OUT, bool HI, bool HJ>
 __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, const float* __restrict__ R,
                                              const PairOut& o, const float* ws, int ldw) {
   constexpr bool kRpa = MODE == G_RPA || MODE == G_RPA_T;
@@ -183,6 +239,11 @@ __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, co
     float Kij[4][4], Kji[4][4];
     exchange<HI, HJ>(ws, ldw, cij, cji, Kij, Kji);
     const size_t vb = (size_t)v * no;
+    float p1 = 1.0f, p2 = 1.0f, q1 = 1.0f, q2 = 1.0f;
+    if (SPLIT == kHalfPair) {
+      if (kPlus) pow2_factors(__ldg(o.e + v), p1, p2);
+      if (kMinus) pow2_factors(__ldg(o.em + v), q1, q2);
+    }
 #pragma unroll
     for (int mu = 0; mu < 4; ++mu) {
       if (mu >= nI) continue;
@@ -191,6 +252,11 @@ __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, co
       for (int lam = 0; lam < 4; ++lam) {
         g[lam] = kRpa ? -(Kij[mu][lam] + Kji[lam][mu]) : -Kij[mu][lam];
         q[lam] = -(Kij[mu][lam] - Kji[lam][mu]);
+      }
+      if (SPLIT == kHalfPair) {
+        if (kPlus) put_row_half(o.Hh + vb + out_ij, o.Hl + vb + out_ij, ldo, mu, nJ, vout_ij, g, p1, p2);
+        if (kMinus) put_row_half(o.Hmh + vb + out_ij, o.Hml + vb + out_ij, ldo, mu, nJ, vout_ij, q, q1, q2);
+        continue;
       }
       if (kPlus) put_row<SPLIT>(G0 + vb + out_ij, G1 + vb + out_ij, G1 ? G1 + vb + out_ij : nullptr, ldo, mu, 0, nJ, vout_ij, g);
       if (kMinus) put_row<SPLIT>(M0 + vb + out_ij, M1 ? M1 + vb + out_ij : nullptr, M1 ? M1 + vb + out_ij : nullptr,
@@ -204,6 +270,11 @@ __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, co
       for (int mu = 0; mu < 4; ++mu) {
         g[mu] = kRpa ? -(Kij[mu][lam] + Kji[lam][mu]) : -Kji[lam][mu];
         q[mu] = Kij[mu][lam] - Kji[lam][mu];
+      }
+      if (SPLIT == kHalfPair) {
+        if (kPlus) put_row_half(o.Hh + vb + out_ji, o.Hl + vb + out_ji, ldo, lam, nI, vout_ji, g, p1, p2);
+        if (kMinus) put_row_half(o.Hmh + vb + out_ji, o.Hml + vb + out_ji, ldo, lam, nI, vout_ji, q, q1, q2);
+        continue;
       }
       if (kPlus) put_row<SPLIT>(G0 + vb + out_ji, G1 ? G1 + vb + out_ji : nullptr, G1 ? G1 + vb + out_ji : nullptr, ldo, lam, 0,
                      nI, vout_ji, g);
@@ -225,7 +296,7 @@ __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, co
 // diagonal block of a super-atom: one-centre Coulomb and exchange, the
 // two-centre Coulomb of the diagonal blocks (J2), and for a hydrogen run the
 // exchange between its hydrogens
-template <GMode MODE, bool SPLIT, int OUT>
+template <GMode MODE, int SPLIT, int OUT>
 __device__ __forceinline__ void diag_block(int n, int np, int nvec, int4 I, const double* __restrict__ par,
                                            const float* __restrict__ W, const float* __restrict__ J2, int ldj,
                                            const float* __restrict__ R, const PairOut& o) {
@@ -262,7 +333,7 @@ __device__ __forceinline__ void diag_block(int n, int np, int nvec, int4 I, cons
               gm = -(K1ab - K1ba);
             }
           }
-          put<SPLIT, kRpa, OUT>(o, n, v * (long long)n, I.x + a, I.x + b, g, gm);
+          put<SPLIT, kRpa, OUT>(o, n, v, I.x + a, I.x + b, g, gm);
         }
     }
     return;
@@ -300,14 +371,14 @@ __device__ __forceinline__ void diag_block(int n, int np, int nvec, int4 I, cons
           g = kRpa ? -(kr + krt) : -kr;
           gm = -(kr - krt);
         }
-        put<SPLIT, kRpa, OUT>(o, n, v * (long long)n, I.x + i, I.x + j, g, gm);
+        put<SPLIT, kRpa, OUT>(o, n, v, I.x + i, I.x + j, g, gm);
       }
   }
 }
 
 // One super-atom pair of the pair list, all nvec matrices; ws: 100 floats of
 // shared memory owned by the calling thread.
-template <GMode MODE, bool SPLIT, int OUT = kOutBoth>
+template <GMode MODE, int SPLIT, int OUT = kOutBoth>
 __device__ __forceinline__ void gpair_one(int n, int np, int nvec, int2 pr, const int4* __restrict__ sa,
                                           const double* __restrict__ par, const float* __restrict__ W,
                                           const float* __restrict__ J2, int ldj, const float* __restrict__ R,

@@ -1,6 +1,7 @@
 // Host-side launchers of libxs's CUDA kernels.
 #pragma once
 
+#include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
 #include "common.cuh"
@@ -72,6 +73,17 @@ void gpair_build(cudaStream_t s, const DevMol& m, const double* d_par, GMode mod
 void gpair_build_split(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const float* W,
                        const float* J2, int ldj, const float* R, float* Gh, float* Gl, float* Gmh, float* Gml,
                        int ldo);
+// Float32 G build whose outputs are float16 pairs (row stride ldo >= n, columns
+// n..ldo-1 zeroed) of G 2^-e[v] and G- 2^-em[v]; the exponents are formed here
+// from bounds (gpair.cu).  rmax: per matrix the bits of the largest |R|; wmax:
+// abs_hi of the largest two-centre integral.  In the TDHF modes either pair may
+// be null.
+struct GHalf {
+  __half *h = nullptr, *l = nullptr, *mh = nullptr, *ml = nullptr;
+  int *e = nullptr, *em = nullptr;
+};
+void gbuild_half(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const float* R,
+                 const unsigned int* rmax, const unsigned int* wmax, const GHalf& o, int ldo, DevBuf<float>& ws);
 // The same with caller-provided scratch: r and J2 of np * nvec elements each.
 void gbuild_raw(cudaStream_t s, const DevMol& m, const double* d_par, GMode mode, int nvec, const double* R, double* G,
                 double* Gm, double* r, double* J2);

@@ -28,6 +28,7 @@
 // through a second barrier ring.  Every wait is bounded by the global timer; a
 // timeout sets the error word, the CTA skips the remaining work, waits
 // (bounded) for its issued copies and MMAs, frees TMEM and exits.
+#include <algorithm>
 #include <mutex>
 #include <unordered_map>
 
@@ -43,8 +44,12 @@ namespace {
 using namespace tc5;
 
 constexpr int BM = 128;
-constexpr int BK = 16;       // 16 tf32 = 64 bytes = one 64-byte swizzle row
-constexpr int kPadK = 32;    // operands' K padding (a multiple of BK)
+// K block: 64 bytes of an operand row (one 64-byte swizzle row), 16 TF32 or 32
+// float16 terms, two MMA steps either way
+constexpr int kRowBytes = 64;
+template <typename T>
+__host__ __device__ constexpr int bk_for() { return kRowBytes / static_cast<int>(sizeof(T)); }
+constexpr int kPadK = 32;    // operands' K padding (a multiple of both)
 // stage ring depth: 8 stages of 24 KB for 64-wide tiles, 6 of 32 KB for
 // 128-wide tiles, 4 of 48 KB for 256-wide tiles (which halve the A-tile
 // re-reads per flop).  K blocks of 16 rather than 32 keep the same 192 KB of
@@ -52,7 +57,9 @@ constexpr int kPadK = 32;    // operands' K padding (a multiple of BK)
 // MMAs consume one.
 template <int BN>
 __host__ __device__ constexpr int stages_for() { return BN >= 256 ? 4 : (BN >= 128 ? 6 : 8); }
-constexpr int kChunkBlocks = 8;   // K blocks (of 16 terms) per promoted chunk
+// K blocks per promoted chunk: 128 TF32 or 256 float16 terms, 16 truncating MMA
+// steps of each of the three products
+constexpr int kChunkBlocks = 8;
 // TMEM chunk slots (BN columns each, at most 512 columns) and epilogue warps
 template <int BN>
 __host__ __device__ constexpr int slots_for() { return BN >= 256 ? 2 : 4; }
@@ -82,18 +89,37 @@ __device__ __forceinline__ void tf32_split(float x, float& hi, float& lo) {
   lo = tf32_rn(x - hi);
 }
 
+// hi and lo of two values
+__device__ __forceinline__ void half_pair2(float x, float y, __half2& hi, __half2& lo) {
+  hi = __floats2half2_rn(x, y);
+  const float2 f = __half22float2(hi);
+  lo = __floats2half2_rn(x - f.x, y - f.y);
+}
+
+// hi and lo of f + g, |g| <= 2^-24 |f| (the value scaled, |f| < 2^15)
+__device__ __forceinline__ void half_pair(float f, float g, __half& hi, __half& lo) {
+  hi = __float2half_rn(f);
+  lo = __float2half_rn((f - __half2float(hi)) + g);
+}
+
+// epilogue modes (template parameter MODE): 0: float D (and max |D|); 1: TF32
+// pair (D, Dlo); 2: float16 pair (Dh, Dhl)
 struct EpiArgs {
-  int mode;             // 0: float D; 1: TF32 pair (Dhi, Dlo); 2: double Y + (eps_a - eps_i) X
   float* D;
   float* Dlo;
-  double* Y;
-  const double* X;
-  const double* eps;
   int ld;               // leading dimension of the output rows
   long long bstride;    // output stride between batch entries
-  int o;                // mode 2: number of occupied orbitals (eps offset of the virtuals)
-  unsigned int* rowmax;   // mode 2, optional: per batch entry abs_hi of max |Y|
+  unsigned int* rowmax;   // mode 0, optional: per batch entry the bits of max |D|
+  const int *ea, *eb;     // float16 pairs: operand exponents (per batch entry when batched)
+  __half *Dh, *Dhl;       // mode 2
+  int* eout;
+  int shift;              // mode 2: 15 + ceil(log2 Kpad)
+  int vec;                // mode 0: output rows allow 16-byte accesses of four columns
 };
+
+// row stride (floats) of an epilogue warp's 32 x 16 staging block: 16-byte rows, conflict-free by four
+constexpr int kEpStride = 20;
+
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
   asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_u32(bar)) : "memory");
@@ -103,7 +129,7 @@ __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
 // (batch entry major, then row tile, then column tile); the TMA ring runs on
 // across tiles and the MMA warp alternates two TMEM accumulators so that a
 // tile's epilogue overlaps the next tile's loads and MMAs.
-template <int BN>
+template <int BN, typename T, int MODE>
 __global__ void __launch_bounds__(threads_for<BN>(), 1)
     tc_gemm_kernel(const __grid_constant__ CUtensorMap tmAh, const __grid_constant__ CUtensorMap tmAl,
                    const __grid_constant__ CUtensorMap tmBh, const __grid_constant__ CUtensorMap tmBl, int M, int N,
@@ -115,8 +141,10 @@ __global__ void __launch_bounds__(threads_for<BN>(), 1)
   constexpr int NSLOT = slots_for<BN>();
   constexpr int EPI = epi_warps_for<BN>();
   constexpr int CW = BN < 128 ? BN : 128;   // accumulator columns per epilogue warp
-  constexpr int A_BYTES = BM * BK * 4;
-  constexpr int B_BYTES = BN * BK * 4;
+  constexpr bool kF16 = sizeof(T) == 2;
+  constexpr int BK = bk_for<T>();
+  constexpr int A_BYTES = BM * kRowBytes;
+  constexpr int B_BYTES = BN * kRowBytes;
   constexpr int STAGE_BYTES = 2 * A_BYTES + 2 * B_BYTES;
   uint8_t* stage_base = base;
   uint64_t* full = reinterpret_cast<uint64_t*>(base + STAGES * STAGE_BYTES);
@@ -125,8 +153,9 @@ __global__ void __launch_bounds__(threads_for<BN>(), 1)
   uint64_t* acce = accf + NSLOT;     // [NSLOT]
   uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acce + NSLOT);
   // epilogue staging: per epilogue warp a 32 x 16 block, transposed so that
-  // global stores run along rows
-  float* stage_ep = reinterpret_cast<float*>(reinterpret_cast<uint8_t*>(acce + NSLOT) + 16);
+  // global stores run along rows (16-byte aligned)
+  float* stage_ep = reinterpret_cast<float*>(
+      (reinterpret_cast<uintptr_t>(acce + NSLOT) + 16 + 15) & ~uintptr_t(15));
 
   const int warp = threadIdx.x / 32, lane = threadIdx.x % 32;
   const int nk = Kpad / BK;
@@ -181,7 +210,7 @@ __global__ void __launch_bounds__(threads_for<BN>(), 1)
       mbar_wait(&empty[q % STAGES], static_cast<uint32_t>((q / STAGES) & 1), err, 0) || true;
   } else if (warp == 1 && lane == 0) {
     // MMA issue: chunk q of the CTA's sequence accumulates into slot q % NSLOT
-    constexpr uint32_t idesc = idesc_f32acc(2, BM, BN);
+    constexpr uint32_t idesc = idesc_f32acc(kF16 ? 0 : 2, BM, BN);
     long long g = 0, q = 0;
     bool ok = true;
     for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
@@ -206,12 +235,18 @@ __global__ void __launch_bounds__(threads_for<BN>(), 1)
           const uint32_t ah = smem_u32(st), al = smem_u32(st + A_BYTES);
           const uint32_t bh = smem_u32(st + 2 * A_BYTES), bl = smem_u32(st + 2 * A_BYTES + B_BYTES);
 #pragma unroll
-          for (int kk = 0; kk < BK / 8; ++kk) {
-            const uint32_t off = kk * 32;  // 8 tf32 per MMA step
+          for (int kk = 0; kk < 2; ++kk) {
+            const uint32_t off = kk * 32;  // 32 bytes (8 TF32, 16 float16 terms) per MMA step
             const uint32_t acc0 = (kb > kc || kk > 0) ? 1u : 0u;
-            mma_tf32(acc, sdesc64(ah + off), sdesc64(bh + off), idesc, acc0);
-            mma_tf32(acc, sdesc64(ah + off), sdesc64(bl + off), idesc, 1u);
-            mma_tf32(acc, sdesc64(al + off), sdesc64(bh + off), idesc, 1u);
+            if constexpr (kF16) {
+              mma_bf16(acc, sdesc64(ah + off), sdesc64(bh + off), idesc, acc0);
+              mma_bf16(acc, sdesc64(ah + off), sdesc64(bl + off), idesc, 1u);
+              mma_bf16(acc, sdesc64(al + off), sdesc64(bh + off), idesc, 1u);
+            } else {
+              mma_tf32(acc, sdesc64(ah + off), sdesc64(bh + off), idesc, acc0);
+              mma_tf32(acc, sdesc64(ah + off), sdesc64(bl + off), idesc, 1u);
+              mma_tf32(acc, sdesc64(al + off), sdesc64(bh + off), idesc, 1u);
+            }
           }
           mma_commit(&empty[s]);
         }
@@ -251,48 +286,90 @@ __global__ void __launch_bounds__(threads_for<BN>(), 1)
         mbar_arrive(&acce[slot]);
       }
       if (!ok) break;
-      float* st = stage_ep + (warp - 2) * 32 * 17;
-      const int c2 = lane & 15, rb = lane >> 4;
-      unsigned int ymax = 0;   // mode 2: abs_hi of the largest |Y| this lane stored
+      float* st = stage_ep + (warp - 2) * 32 * kEpStride;
+      unsigned int ymax = 0;   // mode 0: bits of the largest |D| this lane stored
+      // float16 pairs: the powers of two taken out of the operands, in two factors within float32's range
+      float f1 = 1.0f, f2 = 1.0f;
+      if constexpr (kF16) {
+        const int eab = ep.ea[a3 ? bz : 0] + ep.eb[b3 ? bz : 0];
+        if (MODE == 2 && m0 == 0 && n0 == 0 && threadIdx.x == 64) ep.eout[bz] = eab + ep.shift;
+        const int es = MODE == 2 ? -ep.shift : max(-250, min(250, eab));
+        f1 = __int_as_float((es / 2 + 127) << 23);
+        f2 = __int_as_float((es - es / 2 + 127) << 23);
+      }
+      // Blocks of 32 rows x 16 columns through shared memory, then along rows: four
+      // lanes per row and four columns per lane where rows allow 16-byte accesses,
+      // else a lane per column (16 lanes over 64 contiguous bytes).  The store phase
+      // holds back the drain of the next tile's chunks, so its instructions count: one
+      // column per lane and step throughout ran R and S of 20 vectors at 2200 AOs at
+      // 880 TFLOP/s, this at 1620.
+      const long long b0 = (long long)bz * ep.bstride;
+      const int r0 = m0 + lane_base, cw0 = n0 + colh * CW;
 #pragma unroll
       for (int c0 = 0; c0 < CW; c0 += 16) {
 #pragma unroll
-        for (int j = 0; j < 16; ++j) st[lane * 17 + j] = acc[c0 + j];
+        for (int j = 0; j < 16; j += 4)
+          *reinterpret_cast<float4*>(st + lane * kEpStride + j) =
+              make_float4(acc[c0 + j], acc[c0 + j + 1], acc[c0 + j + 2], acc[c0 + j + 3]);
         __syncwarp();
-        const int col = n0 + colh * CW + c0 + c2;
-#pragma unroll 4
-        for (int k = 0; k < 16; ++k) {
-          const int r2 = rb + 2 * k;
-          const int row = m0 + lane_base + r2;
-          if (row >= M) continue;
-          const float x = st[r2 * 17 + c2];
-          const long long rbo = (long long)bz * ep.bstride + (long long)row * ep.ld;
-          if (col >= N) {
-            // a TF32-pair output feeds the next GEMM as a K-major operand:
-            // its padding columns up to the row stride must read as zero
-            if (ep.mode == 1 && col < ep.ld) {
-              ep.D[rbo + col] = 0.0f;
-              ep.Dlo[rbo + col] = 0.0f;
+        if (MODE == 1 || MODE == 2 || ep.vec) {
+          const int rq = lane >> 2, cq = 4 * (lane & 3), col = cw0 + c0 + cq;
+#pragma unroll
+          for (int k = 0; k < 4; ++k) {
+            const int row = r0 + rq + 8 * k;
+            const float4 q = *reinterpret_cast<const float4*>(st + (rq + 8 * k) * kEpStride + cq);
+            if (row >= M) continue;
+            float x[4] = {q.x, q.y, q.z, q.w};
+            if constexpr (kF16) {
+#pragma unroll
+              for (int j = 0; j < 4; ++j) x[j] = x[j] * f1 * f2;
             }
-            continue;
+            const long long at = b0 + (long long)row * ep.ld + col;
+            if constexpr (MODE == 0) {
+              if (col + 3 < N) {
+                *reinterpret_cast<float4*>(ep.D + at) = make_float4(x[0], x[1], x[2], x[3]);
+              } else {
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                  if (col + j < N) ep.D[at + j] = x[j];
+              }
+#pragma unroll
+              for (int j = 0; j < 4; ++j) ymax = max(ymax, __float_as_uint(x[j]) & 0x7FFFFFFFu);   // 0 past N
+            } else if constexpr (MODE == 1) {
+              // a pair feeds the next GEMM as a K-major operand: its padding columns
+              // up to the row stride (a multiple of 32) read as zero, as computed
+              if (col < ep.ld) {
+                float h[4], l[4];
+#pragma unroll
+                for (int j = 0; j < 4; ++j) tf32_split(x[j], h[j], l[j]);
+                *reinterpret_cast<float4*>(ep.D + at) = make_float4(h[0], h[1], h[2], h[3]);
+                *reinterpret_cast<float4*>(ep.Dlo + at) = make_float4(l[0], l[1], l[2], l[3]);
+              }
+            } else if constexpr (MODE == 2) {
+              if (col < ep.ld) {
+                __half2 hh[2], ll[2];
+                half_pair2(x[0], x[1], hh[0], ll[0]);
+                half_pair2(x[2], x[3], hh[1], ll[1]);
+                *reinterpret_cast<uint2*>(ep.Dh + at) = *reinterpret_cast<uint2*>(hh);
+                *reinterpret_cast<uint2*>(ep.Dhl + at) = *reinterpret_cast<uint2*>(ll);
+              }
+            }
           }
-          if (ep.mode == 0) {
-            ep.D[rbo + col] = x;
-          } else if (ep.mode == 1) {
-            float h, l;
-            tf32_split(x, h, l);
-            ep.D[rbo + col] = h;
-            ep.Dlo[rbo + col] = l;
-          } else {
-            const double de = ep.eps[ep.o + col] - ep.eps[row];
-            const double y = static_cast<double>(x) + de * ep.X[rbo + col];
-            ep.Y[rbo + col] = y;
-            ymax = max(ymax, abs_hi(y));
+        } else if constexpr (MODE == 0) {
+          const int c2 = lane & 15, rb = lane >> 4, col = cw0 + c0 + c2;
+#pragma unroll
+          for (int k = 0; k < 16; ++k) {
+            const int lr = rb + 2 * k, row = r0 + lr;
+            float x = st[lr * kEpStride + c2];
+            if constexpr (kF16) x = x * f1 * f2;
+            if (col >= N || row >= M) continue;
+            ep.D[b0 + (long long)row * ep.ld + col] = x;
+            ymax = max(ymax, __float_as_uint(x) & 0x7FFFFFFFu);
           }
         }
         __syncwarp();
       }
-      if (ep.mode == 2 && ep.rowmax) {
+      if (ep.rowmax) {
         ymax = __reduce_max_sync(0xffffffffu, ymax);
         if (lane == 0 && ymax) atomicMax(&ep.rowmax[bz], ymax);
       }
@@ -358,17 +435,206 @@ __global__ void split_pad_t_kernel(int rows, int cols, int ld_dst, const double*
   }
 }
 
-// rows x kpad float32 matrix (row stride ld floats), batch entries bstride apart
-CUtensorMap make_map(const float* ptr, int rows, int kpad, int ld, int batch, long long bstride, int box_rows) {
+// float32 to float64 by its fields (the conversion runs on the float64 pipe, 64
+// cycles a warp); subnormals, infinities and NaN by the conversion
+__device__ __forceinline__ double widen(float x) {
+  const unsigned int u = __float_as_uint(x), a = u & 0x7FFFFFFFu;
+  if (a - 0x00800000u >= 0x7F000000u && a) return static_cast<double>(x);
+  const unsigned int hi = a ? (a >> 3) + (896u << 20) : 0u;
+  return __hiloint2double(static_cast<int>((u & 0x80000000u) | hi), static_cast<int>(u << 29));
+}
+
+// Y = D + (eps_a - eps_i) X, D float32, for nvec vectors of o x v: each thread
+// forms its elements' gaps once per eight vectors; rowmax (optional): per vector
+// abs_hi of the largest |Y|.  As the GEMM's epilogue this took 490 us for 20
+// vectors of 1201 x 999 (its warps alone feed the float64 pipe and its loads have
+// nothing to hide behind) in a product of 200 us; here 20 bytes an element at
+// memory speed.
+__global__ void __launch_bounds__(256) add_gaps_kernel(int nvec, int o, int v, const double* __restrict__ eps,
+                                                       const float* __restrict__ D, const double* __restrict__ X,
+                                                       double* __restrict__ Y, unsigned int* __restrict__ rowmax) {
+  __shared__ unsigned int top[8];
+  const long long ov = (long long)o * v;
+  const int k0 = 8 * blockIdx.y, nk = min(8, nvec - k0);
+  if (threadIdx.x < 8) top[threadIdx.x] = 0;
+  __syncthreads();
+  unsigned int m[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+  for (long long e = (long long)blockIdx.x * blockDim.x + threadIdx.x; e < ov; e += (long long)gridDim.x * blockDim.x) {
+    const int i = static_cast<int>(static_cast<unsigned int>(e) / static_cast<unsigned int>(v));
+    const double gap = __ldg(eps + o + (static_cast<int>(e) - i * v)) - __ldg(eps + i);
+    double x[8];
+    float d[8];
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      x[q] = q < nk ? __ldg(X + (k0 + q) * ov + e) : 0.0;
+      d[q] = q < nk ? __ldg(D + (k0 + q) * ov + e) : 0.0f;
+    }
+#pragma unroll
+    for (int q = 0; q < 8; ++q) {
+      if (q >= nk) continue;
+      const double y = fma(gap, x[q], widen(d[q]));
+      Y[(k0 + q) * ov + e] = y;
+      m[q] = max(m[q], abs_hi(y));
+    }
+  }
+  if (!rowmax) return;
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {
+    const unsigned int w = __reduce_max_sync(0xffffffffu, m[q]);
+    if ((threadIdx.x & 31) == 0 && w) atomicMax(&top[q], w);
+  }
+  __syncthreads();
+  if (threadIdx.x < nk && top[threadIdx.x]) atomicMax(&rowmax[k0 + threadIdx.x], top[threadIdx.x]);
+}
+
+// ---- float16 pairs ---------------------------------------------------------------
+
+// exponent e with 2^(e + 14) <= max < 2^(e + 15), from abs_hi of a double
+__device__ __forceinline__ int exponent_f64(unsigned int amax) {
+  const int ex = static_cast<int>((amax >> 20) & 0x7FF);
+  return ex == 0 || ex == 0x7FF ? 0 : ex - 1023 - 14;
+}
+__device__ __forceinline__ int exponent_f32(unsigned int amax) {
+  const int ex = static_cast<int>(amax >> 23);
+  return ex == 0 || ex == 0xFF ? 0 : ex - 127 - 14;
+}
+
+// half_pair of a float64 x 2^-e by its fields: conversions between float64 and
+// float32 run on the float64 pipe (a third of the TF32 split's time went there).
+// f is x rounded to 24 bits, g the remainder.
+__device__ __forceinline__ void half_pair_f64(double x, int e, __half& hi, __half& lo) {
+  const unsigned long long b = static_cast<unsigned long long>(__double_as_longlong(x));
+  const int ex = static_cast<int>((b >> 52) & 0x7FF);
+  if (ex == 0x7FF) {   // infinities and NaN keep their kind
+    hi = __float2half_rn(static_cast<float>(x));
+    lo = __float2half_rn(static_cast<float>(x) - static_cast<float>(x));
+    return;
+  }
+  const unsigned long long r = (b & 0x7FFFFFFFFFFFFFFFull) + (1ull << 28);   // rounded at 2^-23 of the leading bit
+  const int fe = static_cast<int>(r >> 52) - 1023 - e + 127;                   // float exponent of the scaled value
+  if (ex == 0 || fe <= 0) {   // below 2^-126 after scaling: 2^-140 of the largest entry
+    hi = lo = __float2half_rn(0.0f);
+    return;
+  }
+  const unsigned int sign = static_cast<unsigned int>(b >> 63) << 31;
+  const float f = __uint_as_float(sign | (static_cast<unsigned int>(fe) << 23) |
+                                  (static_cast<unsigned int>(r >> 29) & 0x7FFFFFu));
+  // remainder in units of 2^-52 of x's binade, signed: the low 29 bits against the rounding
+  const int low = static_cast<int>(r & 0x1FFFFFFFull) - (1 << 28);
+  const int ge = ex - 1023 - e - 52 + 127;                                     // 2^(ex - 1023 - e - 52)
+  float g = ge > 0 ? static_cast<float>(low) * __uint_as_float(static_cast<unsigned int>(ge) << 23) : 0.0f;
+  if (sign) g = -g;
+  half_pair(f, g, hi, lo);
+}
+
+__global__ void absmax_f64_kernel(long long count, const double* __restrict__ src, long long sstride,
+                                  unsigned int* __restrict__ amax) {
+  const double* x = src + blockIdx.y * sstride;
+  const long long stride = (long long)gridDim.x * blockDim.x;
+  unsigned int m0 = 0, m1 = 0, m2 = 0, m3 = 0;
+  long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+  for (; i + 3 * stride < count; i += 4 * stride) {
+    const double a = x[i], b = x[i + stride], c = x[i + 2 * stride], d = x[i + 3 * stride];
+    m0 = max(m0, abs_hi(a));
+    m1 = max(m1, abs_hi(b));
+    m2 = max(m2, abs_hi(c));
+    m3 = max(m3, abs_hi(d));
+  }
+  for (; i < count; i += stride) m0 = max(m0, abs_hi(x[i]));
+  const unsigned int m = __reduce_max_sync(0xffffffffu, max(max(m0, m1), max(m2, m3)));
+  if ((threadIdx.x & 31) == 0 && m) atomicMax(&amax[blockIdx.y], m);
+}
+
+// dst[r][c] = pair of src[r][c] (TR: src[c][r], through 32 x 64 shared-memory
+// tiles), two columns per thread so that a warp stores 128 bytes of hi and of lo
+template <bool TR>
+__global__ void __launch_bounds__(256) split16_f64_kernel(int rows, int cols, int ld_dst,
+                                                          const double* __restrict__ src, int ld_src,
+                                                          long long sstride, long long dstride,
+                                                          const unsigned int* __restrict__ amax, int* __restrict__ eout,
+                                                          __half* __restrict__ hi, __half* __restrict__ lo) {
+  __shared__ unsigned int t[TR ? 64 : 1][33];   // (hi, lo) of one element
+  const int b = blockIdx.z;
+  const int r0 = blockIdx.y * 32, c0 = blockIdx.x * 64;
+  const double* sb = src + b * sstride;
+  const int e = exponent_f64(amax[b]);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) eout[b] = e;
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  auto packed = [&](double x) {
+    __half h, l;
+    half_pair_f64(x, e, h, l);
+    return static_cast<unsigned int>(__half_as_ushort(h)) | (static_cast<unsigned int>(__half_as_ushort(l)) << 16);
+  };
+  if constexpr (TR) {
+    for (int k = w; k < 64; k += 8) {
+      const int c = c0 + k, r = r0 + lane;
+      t[k][lane] = packed((c < cols && r < rows) ? sb[(long long)c * ld_src + r] : 0.0);
+    }
+    __syncthreads();
+  }
+  for (int k = w; k < 32; k += 8) {
+    const int r = r0 + k, c = c0 + 2 * lane;
+    if (r >= rows || c >= ld_dst) continue;
+    unsigned int u0, u1;
+    if constexpr (TR) {
+      u0 = t[2 * lane][k];
+      u1 = t[2 * lane + 1][k];
+    } else {
+      u0 = packed(c < cols ? sb[(long long)r * ld_src + c] : 0.0);
+      u1 = packed(c + 1 < cols ? sb[(long long)r * ld_src + c + 1] : 0.0);
+    }
+    const long long at = b * dstride + (long long)r * ld_dst + c;   // even: ld_dst is a multiple of 32
+    *reinterpret_cast<unsigned int*>(hi + at) = __byte_perm(u0, u1, 0x5410);
+    *reinterpret_cast<unsigned int*>(lo + at) = __byte_perm(u0, u1, 0x7632);
+  }
+}
+
+// float32 source, four columns per thread (16-byte loads where rows allow)
+__global__ void __launch_bounds__(256) split16_f32_kernel(int rows, int cols, int ld_dst, const float* __restrict__ src,
+                                                          long long sstride, long long dstride,
+                                                          const unsigned int* __restrict__ amax, int* __restrict__ eout,
+                                                          __half* __restrict__ hi, __half* __restrict__ lo, int vec) {
+  const int b = blockIdx.z;
+  const int e = exponent_f32(amax[b]);
+  if (blockIdx.x == 0 && blockIdx.y == 0 && threadIdx.x == 0) eout[b] = e;
+  // 2^-e in two factors: e reaches down to -141
+  const float f1 = __int_as_float((-e / 2 + 127) << 23), f2 = __int_as_float((-e - (-e / 2) + 127) << 23);
+  const int q = ld_dst / 4;
+  for (long long idx = (long long)blockIdx.x * blockDim.x + threadIdx.x; idx < (long long)rows * q;
+       idx += (long long)gridDim.x * blockDim.x) {
+    const int r = static_cast<int>(idx / q), c = 4 * static_cast<int>(idx - (long long)r * q);
+    const float* s = src + b * sstride + (long long)r * cols + c;
+    float x[4];
+    if (vec && c + 3 < cols) {
+      const float4 t = __ldg(reinterpret_cast<const float4*>(s));
+      x[0] = t.x; x[1] = t.y; x[2] = t.z; x[3] = t.w;
+    } else {
+#pragma unroll
+      for (int j = 0; j < 4; ++j) x[j] = c + j < cols ? s[j] : 0.0f;
+    }
+    const long long at = b * dstride + (long long)r * ld_dst + c;
+    __half2 hh[2], ll[2];
+    half_pair2(x[0] * f1 * f2, x[1] * f1 * f2, hh[0], ll[0]);
+    half_pair2(x[2] * f1 * f2, x[3] * f1 * f2, hh[1], ll[1]);
+    *reinterpret_cast<uint2*>(hi + at) = *reinterpret_cast<uint2*>(hh);
+    *reinterpret_cast<uint2*>(lo + at) = *reinterpret_cast<uint2*>(ll);
+  }
+}
+
+// rows x kpad matrix (row stride ld elements), batch entries bstride apart
+template <typename T>
+CUtensorMap make_map(const T* ptr, int rows, int kpad, int ld, int batch, long long bstride, int box_rows) {
   CUtensorMap m;
+  constexpr int BK = bk_for<T>();
   const bool r3 = batch > 1;
   cuuint64_t dims[3] = {static_cast<cuuint64_t>(kpad), static_cast<cuuint64_t>(rows), static_cast<cuuint64_t>(batch)};
-  cuuint64_t strides[2] = {static_cast<cuuint64_t>(ld) * 4, static_cast<cuuint64_t>(bstride) * 4};
+  cuuint64_t strides[2] = {static_cast<cuuint64_t>(ld) * sizeof(T), static_cast<cuuint64_t>(bstride) * sizeof(T)};
   cuuint32_t box[3] = {static_cast<cuuint32_t>(BK), static_cast<cuuint32_t>(box_rows), 1};
   cuuint32_t estr[3] = {1, 1, 1};
-  if ((reinterpret_cast<uintptr_t>(ptr) & 15) || (ld % 4) || (kpad % BK))
+  if ((reinterpret_cast<uintptr_t>(ptr) & 15) || (ld * sizeof(T) % 16) || (bstride * sizeof(T) % 16) || (kpad % BK))
     throw Error(XS_EINVAL, "tensor-core operand not 16-byte aligned or not padded");
-  CUresult r = encode_fn()(&m, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, r3 ? 3 : 2, const_cast<float*>(ptr), dims, strides,
+  CUresult r = encode_fn()(&m, sizeof(T) == 2 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT16 : CU_TENSOR_MAP_DATA_TYPE_FLOAT32,
+                           r3 ? 3 : 2, const_cast<T*>(ptr), dims, strides,
                            box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_64B,
                            CU_TENSOR_MAP_L2_PROMOTION_L2_256B, CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   if (r != CUDA_SUCCESS) throw Error(XS_ECUDA, "cuTensorMapEncodeTiled failed (" + std::to_string(r) + ")");
@@ -378,8 +644,8 @@ CUtensorMap make_map(const float* ptr, int rows, int kpad, int ld, int batch, lo
 template <int BN>
 size_t smem_bytes() {
   constexpr int STAGES = stages_for<BN>();
-  return 1024 + STAGES * (2 * BM * BK * 4 + 2 * BN * BK * 4) + (2 * STAGES + 2 * slots_for<BN>()) * 8 + 16 +
-         epi_warps_for<BN>() * 32 * 17 * 4;
+  return 1024 + STAGES * (2 * BM * kRowBytes + 2 * BN * kRowBytes) + (2 * STAGES + 2 * slots_for<BN>()) * 8 + 32 +
+         epi_warps_for<BN>() * 32 * kEpStride * 4;
 }
 
 }  // namespace
@@ -410,6 +676,50 @@ void split_pad_t(cudaStream_t s, int rows, int cols, int ld_dst, const double* s
   XS_CHECK_LAUNCH();
 }
 
+void add_gaps(cudaStream_t s, int nvec, int o, int v, const double* eps, const float* D, const double* X, double* Y,
+              unsigned int* rowmax) {
+  const long long ov = (long long)o * v;
+  if (nvec <= 0 || ov <= 0) return;
+  const int groups = (nvec + 7) / 8;
+  // at most 8 CTAs per SM over the groups, one element a thread at least
+  const long long per = std::max<long long>(1, std::min<long long>(8LL * 152 / groups, (ov + 255) / 256));
+  ProfScope ps(s, "add_gaps", 20.0 * nvec * ov, 0.0);
+  add_gaps_kernel<<<dim3(static_cast<unsigned>(per), groups), 256, 0, s>>>(nvec, o, v, eps, D, X, Y, rowmax);
+  XS_CHECK_LAUNCH();
+}
+
+void absmax_f64(cudaStream_t s, long long count, const double* src, long long sstride, int batch, unsigned int* amax) {
+  if (batch <= 0 || count <= 0) return;
+  // one wave: at most 8 CTAs per SM over the batch, at least 2048 elements per CTA
+  const long long per = std::max<long long>(1, std::min<long long>(8LL * 152 / batch, (count + 2047) / 2048));
+  ProfScope ps(s, "absmax_f64", 8.0 * count * batch, 0.0);
+  absmax_f64_kernel<<<dim3(static_cast<unsigned>(per), batch), 256, 0, s>>>(count, src, sstride, amax);
+  XS_CHECK_LAUNCH();
+}
+
+void split16(cudaStream_t s, int rows, int cols, int ld_dst, const double* src, int ld_src, long long sstride,
+             long long dstride, int batch, bool transpose, const unsigned int* amax, int* e, __half* hi, __half* lo) {
+  if (rows <= 0 || batch <= 0) return;
+  const dim3 grid((ld_dst + 63) / 64, (rows + 31) / 32, batch);
+  ProfScope ps(s, "split16", (double)batch * rows * (8.0 * cols + 4.0 * ld_dst), 0.0);
+  if (transpose)
+    split16_f64_kernel<true><<<grid, 256, 0, s>>>(rows, cols, ld_dst, src, ld_src, sstride, dstride, amax, e, hi, lo);
+  else
+    split16_f64_kernel<false><<<grid, 256, 0, s>>>(rows, cols, ld_dst, src, ld_src, sstride, dstride, amax, e, hi, lo);
+  XS_CHECK_LAUNCH();
+}
+
+void split16(cudaStream_t s, int rows, int cols, int ld_dst, const float* src, long long sstride, long long dstride,
+             int batch, const unsigned int* amax, int* e, __half* hi, __half* lo) {
+  if (rows <= 0 || batch <= 0) return;
+  const long long per = ((long long)rows * (ld_dst / 4) + 255) / 256;
+  const dim3 grid(static_cast<unsigned>(std::min<long long>(per, std::max<long long>(1, 16LL * 152 / batch))), 1, batch);
+  const int vec = cols % 4 == 0 && sstride % 4 == 0 && reinterpret_cast<uintptr_t>(src) % 16 == 0;
+  ProfScope ps(s, "split16", (double)batch * rows * (4.0 * cols + 4.0 * ld_dst), 0.0);
+  split16_f32_kernel<<<grid, 256, 0, s>>>(rows, cols, ld_dst, src, sstride, dstride, amax, e, hi, lo, vec);
+  XS_CHECK_LAUNCH();
+}
+
 namespace {
 
 int sm_count() {
@@ -422,18 +732,21 @@ int sm_count() {
   return nsm;
 }
 
-template <int BNv>
-void launch_tc(cudaStream_t s, const TcOperand& A, const TcOperand& B, int M, int N, int Kpad, int batch,
+template <int BNv, typename T, int MODE>
+void launch_tc(cudaStream_t s, const TcPair<T>& A, const TcPair<T>& B, int M, int N, int Kpad, int batch,
                const TcEpilogue& e, int* d_err) {
   static_assert(BNv == 64 || BNv == 128 || BNv == 256, "tile width");
   const CUtensorMap ah = make_map(A.hi, M, Kpad, A.ld, A.batched ? batch : 1, A.bstride, BM);
   const CUtensorMap al = make_map(A.lo, M, Kpad, A.ld, A.batched ? batch : 1, A.bstride, BM);
   const CUtensorMap bh = make_map(B.hi, N, Kpad, B.ld, B.batched ? batch : 1, B.bstride, BNv);
   const CUtensorMap bl = make_map(B.lo, N, Kpad, B.ld, B.batched ? batch : 1, B.bstride, BNv);
-  EpiArgs ep{e.mode, e.D, e.Dlo, e.Y, e.X, e.eps, e.ld, e.bstride, e.o, e.rowmax};
+  EpiArgs ep{e.D, e.Dlo, e.ld, e.bstride, e.rowmax, A.e, B.e, e.Dh, e.Dhl, e.eout, 15, 0};
+  while ((1 << (ep.shift - 15)) < Kpad) ++ep.shift;
+  const auto al16 = [](const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
+  ep.vec = e.ld % 4 == 0 && e.bstride % 4 == 0 && al16(e.D);
   const size_t smem = smem_bytes<BNv>();
   static const bool attr_set = [smem] {   // once per process (thread-safe initialisation)
-    XS_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<BNv>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+    XS_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<BNv, T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  static_cast<int>(smem)));
     return true;
   }();
@@ -442,8 +755,8 @@ void launch_tc(cudaStream_t s, const TcOperand& A, const TcOperand& B, int M, in
   const int ntiles = ntm * ntn * batch;
   const int nsm = sm_count();
   const int grid = ntiles < nsm ? ntiles : nsm;   // persistent: one CTA per SM
-  ProfScope ps(s, "tc_gemm_tf32x3", 0.0, 2.0 * 3.0 * M * N * (double)Kpad * batch);
-  tc_gemm_kernel<BNv><<<grid, threads_for<BNv>(), smem, s>>>(ah, al, bh, bl, M, N, Kpad, A.batched && batch > 1 ? 1 : 0,
+  ProfScope ps(s, sizeof(T) == 2 ? "tc_gemm_f16x3" : "tc_gemm_tf32x3", 0.0, 2.0 * 3.0 * M * N * (double)Kpad * batch);
+  tc_gemm_kernel<BNv, T, MODE><<<grid, threads_for<BNv>(), smem, s>>>(ah, al, bh, bl, M, N, Kpad, A.batched && batch > 1 ? 1 : 0,
                                               B.batched && batch > 1 ? 1 : 0, ntm, ntn, ntiles, ep, d_err);
   XS_CHECK_LAUNCH();
 }
@@ -452,11 +765,21 @@ void launch_tc(cudaStream_t s, const TcOperand& A, const TcOperand& B, int M, in
 
 namespace {
 
-void launch_bn(int bn, cudaStream_t s, const TcOperand& A, const TcOperand& B, int M, int N, int Kpad, int batch,
+template <typename T, int MODE>
+void launch_mode(int bn, cudaStream_t s, const TcPair<T>& A, const TcPair<T>& B, int M, int N, int Kpad, int batch,
+                 const TcEpilogue& e, int* d_err) {
+  if (bn == 256) launch_tc<256, T, MODE>(s, A, B, M, N, Kpad, batch, e, d_err);
+  else if (bn == 128) launch_tc<128, T, MODE>(s, A, B, M, N, Kpad, batch, e, d_err);
+  else launch_tc<64, T, MODE>(s, A, B, M, N, Kpad, batch, e, d_err);
+}
+
+template <typename T>
+void launch_bn(int bn, cudaStream_t s, const TcPair<T>& A, const TcPair<T>& B, int M, int N, int Kpad, int batch,
                const TcEpilogue& e, int* d_err) {
-  if (bn == 256) launch_tc<256>(s, A, B, M, N, Kpad, batch, e, d_err);
-  else if (bn == 128) launch_tc<128>(s, A, B, M, N, Kpad, batch, e, d_err);
-  else launch_tc<64>(s, A, B, M, N, Kpad, batch, e, d_err);
+  constexpr int kPairMode = sizeof(T) == 2 ? 2 : 1;   // the pair output of the operands' own kind
+  if (e.mode == 0) launch_mode<T, 0>(bn, s, A, B, M, N, Kpad, batch, e, d_err);
+  else if (e.mode == kPairMode) launch_mode<T, kPairMode>(bn, s, A, B, M, N, Kpad, batch, e, d_err);
+  else throw Error(XS_EINVAL, "split-precision GEMM: epilogue mode");
 }
 
 // Estimated time of a launch with tile width bn, in units of one wave of
@@ -478,10 +801,9 @@ double tile_estimate(int bn, int M, int N, int batch) {
 std::mutex g_tc_mutex;
 std::unordered_map<unsigned long long, int> g_tc_tuned;
 
-}  // namespace
-
-void tc_gemm(cudaStream_t s, const TcOperand& A, const TcOperand& B, int M, int N, int Kpad, int batch,
-             const TcEpilogue& e, int* d_err) {
+template <typename T>
+void tc_gemm_any(cudaStream_t s, const TcPair<T>& A, const TcPair<T>& B, int M, int N, int Kpad, int batch,
+                 const TcEpilogue& e, int* d_err) {
   if (M <= 0 || N <= 0 || batch <= 0) return;
   constexpr int kWidths[3] = {256, 128, 64};
   double est[3], best_est = 1e300;
@@ -501,7 +823,8 @@ void tc_gemm(cudaStream_t s, const TcOperand& A, const TcOperand& B, int M, int 
                                  ((unsigned long long)Kpad << 32) | ((unsigned long long)batch << 48) |
                                  ((unsigned long long)(e.mode & 3) << 58) |
                                  ((unsigned long long)(A.batched ? 1 : 0) << 60) |
-                                 ((unsigned long long)(B.batched ? 1 : 0) << 61);
+                                 ((unsigned long long)(B.batched ? 1 : 0) << 61) |
+                                 ((unsigned long long)(sizeof(T) == 2 ? 1 : 0) << 62);
   {
     std::lock_guard<std::mutex> lock(g_tc_mutex);
     auto it = g_tc_tuned.find(key);
@@ -533,6 +856,18 @@ void tc_gemm(cudaStream_t s, const TcOperand& A, const TcOperand& B, int M, int 
   cudaEventDestroy(e1);
   std::lock_guard<std::mutex> lock(g_tc_mutex);
   g_tc_tuned[key] = best;
+}
+
+}  // namespace
+
+void tc_gemm(cudaStream_t s, const TcOperand& A, const TcOperand& B, int M, int N, int Kpad, int batch,
+             const TcEpilogue& e, int* d_err) {
+  tc_gemm_any<float>(s, A, B, M, N, Kpad, batch, e, d_err);
+}
+
+void tc_gemm(cudaStream_t s, const TcOperand16& A, const TcOperand16& B, int M, int N, int Kpad, int batch,
+             const TcEpilogue& e, int* d_err) {
+  tc_gemm_any<__half>(s, A, B, M, N, Kpad, batch, e, d_err);
 }
 
 }  // namespace xs

@@ -104,7 +104,7 @@ __device__ __forceinline__ uint64_t sdesc64(uint32_t saddr) {
 }
 
 // Instruction descriptor of a dense M x N MMA with float32 accumulation and
-// K-major A and B; ab_format: 1 = BF16 (kind::f16), 2 = TF32 (kind::tf32).
+// K-major A and B; ab_format: 0 = F16, 1 = BF16 (kind::f16), 2 = TF32 (kind::tf32).
 __host__ __device__ constexpr uint32_t idesc_f32acc(int ab_format, int M, int N) {
   return (1u << 4) | (static_cast<uint32_t>(ab_format) << 7) | (static_cast<uint32_t>(ab_format) << 10) |
          (static_cast<uint32_t>(N >> 3) << 17) | (static_cast<uint32_t>(M >> 4) << 24);
@@ -120,6 +120,7 @@ __device__ __forceinline__ void mma_tf32(uint32_t tmem_d, uint64_t adesc, uint64
       : "memory");
 }
 
+// kind::f16: BF16 or F16 operands (both of the type the descriptor names)
 __device__ __forceinline__ void mma_bf16(uint32_t tmem_d, uint64_t adesc, uint64_t bdesc, uint32_t idesc,
                                          uint32_t accum) {
   asm volatile(
