@@ -21,6 +21,7 @@
 // the row segments it reads and writes are contiguous (16-byte loads and
 // stores where the blocks start on multiples of 4 AOs), and each thread keeps
 // the next matrix's blocks in flight while it contracts the current one.
+#include <algorithm>
 #include <vector>
 
 #include "gpair_dev.cuh"
@@ -31,20 +32,41 @@ namespace xs {
 
 namespace {
 
-constexpr int kPairThreads = 256;
+// A thread's walk over the vectors is a chain of uncoalesced loads, contraction and
+// stores, so the vectors are dealt out to enough CTAs to keep the SMs' 16 resident warps
+// replaced four times over; the integrals are read again by each (from L2, 100 floats
+// against 64 of R and G per vector).  One walk per pair -> this split, 256 -> 64 threads:
+// 2200 AOs x 20 vectors 467 -> 406 us, 1233 x 20 300 -> 182, 600 x 10 116 -> 38,
+// 222 x 8 82 -> 15.5; one vector 17 -> 15.  Twice or half as many CTAs are within 3%
+// or up to 10% slower.
+constexpr int kPairThreads = 64;
+constexpr int kPairTargetCTAs = 4 * 8 * 152;
 
 template <GMode MODE, int SPLIT, int OUT>
-__global__ void __launch_bounds__(kPairThreads, 2) gpair_kernel(int n, int np, int nvec, int npairs,
+__global__ void __launch_bounds__(kPairThreads, 8) gpair_kernel(int n, int np, int nvec, int npairs,
                                                                 const int2* __restrict__ pairs,
                                                                 const int4* __restrict__ sa,
                                                                 const double* __restrict__ par,
                                                                 const float* __restrict__ W,
                                                                 const float* __restrict__ J2, int ldj,
-                                                                const float* __restrict__ R, PairOut o) {
+                                                                const float* __restrict__ R, int per, PairOut o) {
   extern __shared__ float wsm[];   // 100 integrals per thread
   const int t = blockIdx.x * blockDim.x + threadIdx.x;
   if (t >= npairs) return;
-  gpair_one<MODE, SPLIT, OUT>(n, np, nvec, pairs[t], sa, par, W, J2, ldj, R, o, wsm + threadIdx.x * 100);
+  const int v0 = blockIdx.y * per, nv = min(per, nvec - v0);
+  const size_t at = (size_t)v0 * n * (SPLIT ? o.ldo : n);
+  if (SPLIT == kPlain) {
+    o.G += at;
+    o.Gm += at;
+  } else if (SPLIT == kTf32Pair) {
+    o.Gh += at; o.Gl += at;
+    o.Gmh += at; o.Gml += at;
+  } else {
+    o.Hh += at; o.Hl += at; o.e += v0;
+    o.Hmh += at; o.Hml += at; o.em += v0;
+  }
+  gpair_one<MODE, SPLIT, OUT>(n, np, nv, pairs[t], sa, par, W, J2 + v0, ldj, R + (size_t)v0 * n * n, o,
+                              wsm + threadIdx.x * 100);
 }
 
 template <GMode MODE, int SPLIT, int OUT>
@@ -58,9 +80,12 @@ void launch_mode(cudaStream_t s, const DevMol& m, const double* d_par, int nvec,
   }();
   (void)attr;
   const int npairs = m.gp_npairs;
-  gpair_kernel<MODE, SPLIT, OUT><<<(npairs + kPairThreads - 1) / kPairThreads, kPairThreads, smem, s>>>(
+  const int ctas = (npairs + kPairThreads - 1) / kPairThreads;
+  const int chunks = std::min(nvec, std::max(1, (kPairTargetCTAs + ctas - 1) / ctas));
+  const int per = (nvec + chunks - 1) / chunks;
+  gpair_kernel<MODE, SPLIT, OUT><<<dim3(ctas, (nvec + per - 1) / per), kPairThreads, smem, s>>>(
       m.n, m.np, nvec, npairs, reinterpret_cast<const int2*>(m.gp_pairs.get()),
-      reinterpret_cast<const int4*>(m.gp_sa.get()), d_par, W, J2, ldj, R, o);
+      reinterpret_cast<const int4*>(m.gp_sa.get()), d_par, W, J2, ldj, R, per, o);
   XS_CHECK_LAUNCH();
 }
 
