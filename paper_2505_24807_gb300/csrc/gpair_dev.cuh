@@ -94,7 +94,8 @@ __device__ __forceinline__ int phi(int p) { return p < 4 ? p : (p < 7 ? p - 3 : 
 // Exchange blocks of one off-diagonal pair and one matrix.  ws holds the
 // pair's integrals (row stride ldw); each unique integral is read once and
 // applied to every (mu nu), (lam sig) index order it stands for.
-template <bool HI, bool HJ>
+// ONE: Kij only.
+template <bool HI, bool HJ, bool ONE>
 __device__ __forceinline__ void exchange(const float* ws, int ldw, const float (&Rij)[4][4], const float (&Rji)[4][4],
                                          float (&Kij)[4][4], float (&Kji)[4][4]) {
 #pragma unroll
@@ -120,7 +121,7 @@ __device__ __forceinline__ void exchange(const float* ws, int ldw, const float (
           if (cb == 1 && l0 == s0) continue;
           const int lam = cb ? s0 : l0, sg = cb ? l0 : s0;
           Kij[mu][lam] = fmaf(w, Rij[nu][sg], Kij[mu][lam]);
-          Kji[lam][mu] = fmaf(w, Rji[sg][nu], Kji[lam][mu]);
+          if (!ONE) Kji[lam][mu] = fmaf(w, Rji[sg][nu], Kji[lam][mu]);
         }
       }
     }
@@ -201,6 +202,10 @@ __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, co
                                              const PairOut& o, const float* ws, int ldw) {
   constexpr bool kRpa = MODE == G_RPA || MODE == G_RPA_T;
   constexpr bool kPlus = !kRpa || (OUT & kOutPlus), kMinus = kRpa && (OUT & kOutMinus);
+  // G+ alone is -K(R + R^T) and symmetric, G- alone -K(R - R^T) and antisymmetric: one
+  // contraction of the sum or difference in place of two
+  // (A+B, 20 vectors: 2200 AOs 480 -> 408 us, 1233 222 -> 182)
+  constexpr bool kOne = kRpa && kPlus != kMinus;
   const int nI = sa_nao(I), nJ = sa_nao(J);
   const int ldo = SPLIT ? o.ldo : n;
   // 16-byte row segments: the block starts on a multiple of 4 AOs, is 4 wide
@@ -237,7 +242,13 @@ __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, co
     float nij[4][4], nji[4][4];
     if (v + 1 < nvec) fetch(v + 1, nij, nji);
     float Kij[4][4], Kji[4][4];
-    exchange<HI, HJ>(ws, ldw, cij, cji, Kij, Kji);
+    if (kOne) {
+#pragma unroll
+      for (int i = 0; i < 4; ++i)
+#pragma unroll
+        for (int j = 0; j < 4; ++j) cij[i][j] = kPlus ? cij[i][j] + cji[j][i] : cij[i][j] - cji[j][i];
+    }
+    exchange<HI, HJ, kOne>(ws, ldw, cij, cji, Kij, Kji);
     const size_t vb = (size_t)v * no;
     float p1 = 1.0f, p2 = 1.0f, q1 = 1.0f, q2 = 1.0f;
     if (SPLIT == kHalfPair) {
@@ -250,8 +261,8 @@ __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, co
       float g[4], q[4];
 #pragma unroll
       for (int lam = 0; lam < 4; ++lam) {
-        g[lam] = kRpa ? -(Kij[mu][lam] + Kji[lam][mu]) : -Kij[mu][lam];
-        q[lam] = -(Kij[mu][lam] - Kji[lam][mu]);
+        g[lam] = kRpa && !kOne ? -(Kij[mu][lam] + Kji[lam][mu]) : -Kij[mu][lam];
+        q[lam] = kOne ? -Kij[mu][lam] : -(Kij[mu][lam] - Kji[lam][mu]);
       }
       if (SPLIT == kHalfPair) {
         if (kPlus) put_row_half(o.Hh + vb + out_ij, o.Hl + vb + out_ij, ldo, mu, nJ, vout_ij, g, p1, p2);
@@ -268,8 +279,8 @@ __device__ __forceinline__ void offdiag_pair(int n, int nvec, int4 I, int4 J, co
       float g[4], q[4];
 #pragma unroll
       for (int mu = 0; mu < 4; ++mu) {
-        g[mu] = kRpa ? -(Kij[mu][lam] + Kji[lam][mu]) : -Kji[lam][mu];
-        q[mu] = Kij[mu][lam] - Kji[lam][mu];
+        g[mu] = kOne ? -Kij[mu][lam] : (kRpa ? -(Kij[mu][lam] + Kji[lam][mu]) : -Kji[lam][mu]);
+        q[mu] = kOne ? Kij[mu][lam] : Kij[mu][lam] - Kji[lam][mu];
       }
       if (SPLIT == kHalfPair) {
         if (kPlus) put_row_half(o.Hh + vb + out_ji, o.Hl + vb + out_ji, ldo, lam, nI, vout_ji, g, p1, p2);
