@@ -337,7 +337,9 @@ struct MgCfg {
   static constexpr int EPI = 8;                            // epilogue warps: two per 32 TMEM lanes
   static constexpr int CW = BN / 2;                        // columns per epilogue warp
   static constexpr int THREADS = 64 + 32 * EPI;
-  static constexpr size_t SMEM = 1024 + static_cast<size_t>(STAGES) * STAGE + (2 * STAGES + 2 * NSLOT) * 8 + 16;
+  static constexpr int OUT_ROW = 80;                       // bytes of a staged output row: 32 residues and padding
+  static constexpr int OUT = EPI * 32 * OUT_ROW;
+  static constexpr size_t SMEM = 1024 + static_cast<size_t>(STAGES) * STAGE + OUT + (2 * STAGES + 2 * NSLOT) * 8 + 16;
 };
 
 __device__ __forceinline__ void mbar_arrive(uint64_t* bar) {
@@ -389,7 +391,7 @@ __global__ void __launch_bounds__(MgCfg<BN>::THREADS, 1)
   using C = MgCfg<BN>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
-  uint64_t* full = reinterpret_cast<uint64_t*>(base + C::STAGES * C::STAGE);
+  uint64_t* full = reinterpret_cast<uint64_t*>(base + C::STAGES * C::STAGE + C::OUT);
   uint64_t* empty = full + C::STAGES;
   uint64_t* accf = empty + C::STAGES;
   uint64_t* acce = accf + C::NSLOT;
@@ -513,22 +515,37 @@ __global__ void __launch_bounds__(MgCfg<BN>::THREADS, 1)
         mbar_arrive(&acce[slot]);
       }
       if (!ok) break;
-      const int row = m0 + lane_base + lane;
-      uint16_t* out = a.res + (static_cast<size_t>(l * a.batch + bz) * a.M + row) * a.ldn + n0 + colh * C::CW;
+      // A thread holds one row: 32 columns at a time go through shared memory, so that a
+      // warp's store covers whole sectors of eight rows.  Storing 16 bytes of 32 rows at a
+      // time held back the next tile's drain (2200 AOs, 4 vectors: 1395 -> 1191 us in the four
+      // products; 1125 without any store).
+      uint8_t* stage = base + C::STAGES * C::STAGE + (warp - 2) * 32 * C::OUT_ROW;
+      const int row0 = m0 + lane_base, col0 = n0 + colh * C::CW;
+      uint16_t* out = a.res + (static_cast<size_t>(l * a.batch + bz) * a.M) * a.ldn;
 #pragma unroll
-      for (int c0 = 0; c0 < C::CW; c0 += 16) {
-        uint32_t p[8];
+      for (int c0 = 0; c0 < C::CW; c0 += 32) {
+        uint32_t p[16];
 #pragma unroll
-        for (int j = 0; j < 8; ++j) {
+        for (int j = 0; j < 16; ++j) {
           float2 r = mod2(acc[c0 / 2 + j], fm, inv);
           r.x += r.x < 0.0f ? fm : 0.0f;
           r.y += r.y < 0.0f ? fm : 0.0f;
           // 0 <= r < m: the low half of the bits of 2^23 + r
           p[j] = __byte_perm(__float_as_uint(r.x + 8388608.0f), __float_as_uint(r.y + 8388608.0f), 0x5410);
         }
-        if (row < a.M && n0 + colh * C::CW + c0 < a.ldn) {   // ldn is a multiple of 16
-          *reinterpret_cast<uint4*>(out + c0) = make_uint4(p[0], p[1], p[2], p[3]);
-          *reinterpret_cast<uint4*>(out + c0 + 8) = make_uint4(p[4], p[5], p[6], p[7]);
+        __syncwarp();
+#pragma unroll
+        for (int j = 0; j < 4; ++j)
+          *reinterpret_cast<uint4*>(stage + lane * C::OUT_ROW + 16 * j) =
+              make_uint4(p[4 * j], p[4 * j + 1], p[4 * j + 2], p[4 * j + 3]);
+        __syncwarp();
+        const int col = col0 + c0 + 8 * (lane & 3);
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+          const int r = 8 * i + (lane >> 2);
+          const uint4 u = *reinterpret_cast<const uint4*>(stage + r * C::OUT_ROW + 16 * (lane & 3));
+          if (row0 + r < a.M && col < a.ldn)   // ldn is a multiple of 16
+            *reinterpret_cast<uint4*>(out + static_cast<size_t>(row0 + r) * a.ldn + col) = u;
         }
       }
     }
@@ -736,12 +753,14 @@ void mg_product(cudaStream_t s, const MgOperand& A, const MgOperand& B, int batc
   a.res = w.res.get();
   {
     ProfScope ps(s, "mg_gemm", 0.0, 2.0 * kModuli * M * N * static_cast<double>(A.K) * batch);
-    // waves of 256-wide tiles against waves of 128-wide ones, which cost 0.6 of them each
+    // waves of 256-wide tiles against waves of 128-wide ones, which cost 0.7 of them each
+    // (four products, 128-wide -> 256-wide where the line is crossed: 561 AOs, 20 vectors
+    // 375 -> 312 us, 600 AOs, 10 vectors 195 -> 179)
     const auto waves = [&](int bn) {
       const long long t = static_cast<long long>(kModuli) * batch * ((M + BM - 1) / BM) * ((N + bn - 1) / bn);
       return static_cast<double>((t + num_sms() - 1) / num_sms());
     };
-    if (waves(256) <= 0.6 * waves(128)) launch_mg<256>(s, A, B, a, d_err);
+    if (waves(256) <= 0.7 * waves(128)) launch_mg<256>(s, A, B, a, d_err);
     else launch_mg<128>(s, A, B, a, d_err);
   }
   CrtArgs c{};
