@@ -64,10 +64,7 @@ FP32_SIMT_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 # dram__bytes_write.sum, mean over the captured launches of one solve of the
 # workload), from the ncu summaries named in "source"; a kernel absent here
 # (or changed since its capture) reports traffic null.
-TRAFFIC = {
-    ("tc_gemm_tf32x3", "large"): dict(bytes_per_launch=7.228e8, source="profiles/tc_gemm_tf32x3_large.md"),
-    ("gbuild_assemble_f32", "large"): dict(bytes_per_launch=1.2246e9, source="profiles/tc_gemm_tf32x3_large.md"),
-}
+TRAFFIC = {}
 
 
 def traffic_of(name, workload):
@@ -77,11 +74,11 @@ def traffic_of(name, workload):
 
 def kernel_roofline(name, t, pk, workload=None):
     """Achieved rate of one profiled kernel family against its bound: digit
-    products, digit splits and the G build stream HBM (algorithmic bytes);
-    tensor-core GEMMs against the TF32 peak; SIMT kernels against the float64
-    or float32 pipe."""
+    products, splits into digits, residues or pairs and the G build stream HBM
+    (algorithmic bytes); tensor-core GEMMs against the peak of their operand type;
+    SIMT kernels against the float64 or float32 pipe."""
     per_launch_s = t["ms"] / 1e3 / t["launches"]
-    if name.startswith(("oz_", "gbuild")) and t["bytes"] > 0:
+    if name.startswith(("oz_", "gbuild", "mg_split", "mg_crt", "add_gaps", "split16", "absmax")) and t["bytes"] > 0:
         ach = t["bytes"] / t["launches"] / per_launch_s / 1e9
         traffic, tsrc = traffic_of(name, workload)
         return dict(kernel=name, bound="hbm", achieved=ach, peak=pk["hbm_gbs"], unit="GB/s",
@@ -89,7 +86,9 @@ def kernel_roofline(name, t, pk, workload=None):
                     peak_source=pk["source"] + " hbm_gbs",
                     bytes_per_launch=t["bytes"] / t["launches"], ms_per_launch=per_launch_s * 1e3)
     ach = t["flops"] / t["launches"] / per_launch_s / 1e12
-    if name.startswith("tc_"):
+    if name.startswith(("tc_gemm_f16", "mg_gemm")):
+        peak, src, bound = pk["bf16_sustained"], pk["source"] + " bf16 sustained (f16 runs at its rate)", "tensor"
+    elif name.startswith("tc_"):
         peak, src, bound = pk["bf16_sustained"] / 2.0, pk["source"] + " bf16 sustained x 1/2 (tf32)", "tensor"
     elif "f64" in name:
         peak, src, bound = FP64_SIMT_TFLOPS, "float64 SIMT, nominal 1.25 TFLOP/s", "alu"
