@@ -1,6 +1,6 @@
 // Mixed-precision A*X path of libxs (see tc.h).
 //
-// Per batch of k trial vectors (all tensor-core operands K-major TF32 pairs):
+// Per batch of k trial vectors (all tensor-core operands K-major TF32 pairs; float16 pairs in products_half):
 //   1. X_k (o x v)                    -> TF32 pair, v padded to 32
 //   2. U_k^T (n x o) = C_vir X_k^T    (tc_gemm, epilogue writes a TF32 pair)
 //   3. R_k (n x n)   = C_occ U_k      (tc_gemm, float32 out)

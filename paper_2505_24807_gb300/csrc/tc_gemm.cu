@@ -1,23 +1,25 @@
 // Split-precision tensor-core GEMM of libxs (sm_103a, tcgen05 + TMA).
 //
-// D = A B^T with A (M x K) and B (N x K) both K-major float32 matrices, each
-// given as a TF32 pair (hi, lo) with x ~= hi + lo (hi rounded to TF32, lo the
-// TF32 remainder).  The product is formed as hi*hi + hi*lo + lo*hi on the
-// 5th-generation tensor cores (kind::tf32) -- the "split-precision (hi + lo)
-// products" that carry the dense C X C^T transforms of the A*X product.
+// D = A B^T with A (M x K) and B (N x K) both K-major matrices, each given as a
+// pair (hi, lo) with x ~= hi + lo: TF32 pairs, or float16 pairs of x 2^-e with one
+// exponent per matrix (tc_gemm.h), whose MMAs run at twice the rate on the same two
+// 11-bit significands.  The product is formed as hi*hi + hi*lo + lo*hi on the
+// 5th-generation tensor cores (kind::tf32, kind::f16) -- the "split-precision (hi +
+// lo) products" that carry the dense C X C^T transforms of the A*X product.  Four
+// products of 20 vectors at 2200 AOs: 2697 us with TF32 pairs, 1176 with float16 pairs.
 //
-// The tensor cores add each 8-term MMA step into their float32 accumulator
-// with truncation, a bias of about half an ulp of the running sum per step
+// The tensor cores add each MMA step (8 TF32 or 16 float16 terms) into their float32
+// accumulator with truncation, a bias of about half an ulp of the running sum per step
 // that grows with K.  So the accumulator is promoted every kChunkBlocks K
-// blocks (128 terms): the MMA warp accumulates each chunk of K into its own
+// blocks (128 or 256 terms, 16 steps): the MMA warp accumulates each chunk of K into its own
 // TMEM slot, and the epilogue warps add the finished chunk sums into
 // round-to-nearest float32 registers.  The truncation bias then scales with
-// 128 instead of K (17x less at K = 2200; 32-term chunks cut it 4x further
-// but cost 8% of the GEMM's rate in the epilogue round trips).
+// the chunk instead of K (TF32: 17x less at K = 2200; 32-term chunks cut it 4x
+// further but cost 8% of the GEMM's rate in the epilogue round trips).
 //
 // Persistent CTAs (one per SM) walk the 128 x BN output tiles (cta_group::1,
 // M = 128):
-//   warp 0      TMA producer: four 64-byte-swizzled boxes per K block of 16
+//   warp 0      TMA producer: four 64-byte-swizzled boxes per K block of 64 bytes
 //   warp 1      TMEM allocation and the single-thread MMA issue into a ring
 //               of NSLOT chunk accumulators
 //   warps 2..   epilogue (4, or 8 for 256-wide tiles: two warps per group of

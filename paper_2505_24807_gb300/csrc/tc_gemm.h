@@ -1,4 +1,4 @@
-// Split-precision (TF32 hi + lo) tensor-core GEMM of libxs (tc_gemm.cu).
+// Split-precision (TF32 or float16 hi + lo) tensor-core GEMM of libxs (tc_gemm.cu).
 #pragma once
 
 #include <cuda_fp16.h>
