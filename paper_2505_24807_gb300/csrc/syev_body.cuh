@@ -16,6 +16,7 @@ namespace {
 constexpr int kSmemMax = 224;   // largest S whose working set fits in shared memory
 constexpr int kSeg = 8;         // row segments of the tridiagonalisation's matrix-vector product
 constexpr int kMaxRR = 4;       // clusters up to this size get a Rayleigh-Ritz rotation
+constexpr int kScaleFree = 12;  // matrices with entries up to 2^+-12 are not scaled
 
 // packed lower triangle: element (i, j), j <= i
 __host__ __device__ __forceinline__ int tri(int i, int j) { return i * (i + 1) / 2 + j; }   // i <= 1024
@@ -326,9 +327,33 @@ __device__ void syevk_body(int S, int k, const double* __restrict__ Ain, int lda
   const int tid = threadIdx.x, nt = blockDim.x;
   const int warp = tid >> 5, lane = tid & 31, nwarp = nt >> 5;
 
+  // Entries whose largest lies outside 2^+-kScaleFree (products in eV and eV^2 do not)
+  // are scaled by a power of two, undone on the eigenvalues: the float32 stages below
+  // square and invert numbers of |T|'s size, and two unnormalised float32 solves grow
+  // a vector to 1e16 / |T|^2, past float32 from |T| of 1e-11 down.
+  __shared__ unsigned int tops[32];
+  unsigned int top = 0;
   for (int i = warp; i < S; i += nwarp)
-    for (int j = lane; j <= i; j += 32) a[tri(i, j)] = Ain[(long long)i * lda + j];
+    for (int j = lane; j <= i; j += 32) {
+      const double x = Ain[(long long)i * lda + j];
+      a[tri(i, j)] = x;
+      top = max(top, abs_hi(x));
+    }
+  top = __reduce_max_sync(0xffffffffu, top);
+  if (lane == 0) tops[warp] = top;
   __syncthreads();
+  for (int w = 0; w < nwarp; ++w) top = max(top, tops[w]);
+  const bool zero = top == 0;              // zero, or below 2^-1042
+  int scale = 0;
+  {
+    const int ex = static_cast<int>(top >> 20) - 1023;
+    if (!zero && ex < 1024 && (ex < -kScaleFree || ex > kScaleFree)) scale = max(ex, -1000);
+  }
+  if (scale != 0) {
+    for (int i = warp; i < S; i += nwarp)
+      for (int j = lane; j <= i; j += 32) a[tri(i, j)] = scalbn(a[tri(i, j)], -scale);
+    __syncthreads();
+  }
 
   // 1. Tridiagonalisation by Householder reflectors H = I - beta u u^T on the
   // packed lower triangle.  The products of a step of m remaining rows take m^2
@@ -494,7 +519,7 @@ __device__ void syevk_body(int S, int k, const double* __restrict__ Ain, int lda
     if (lane == 0) {
       scal[3] = lo;
       scal[4] = hi;
-      scal[5] = fmax(fmax(fabs(lo), fabs(hi)), 1e-300);
+      scal[5] = zero ? 1.0 : fmax(fmax(fabs(lo), fabs(hi)), 1e-300);   // any scale serves a zero matrix
       scal[6] = fmax(1e-30 * fmax(emax2, 1.0), 1e-30 * scal[5]);
     }
   }
@@ -785,7 +810,7 @@ __device__ void syevk_body(int S, int k, const double* __restrict__ Ain, int lda
     __syncthreads();
   }
   for (int q = tid; q < S * k; q += nt) Z[(long long)(q / k) * ldz + q % k] = Zw[q];
-  for (int t = tid; t < k; t += nt) wout[t] = lam[t];
+  for (int t = tid; t < k; t += nt) wout[t] = scale ? scalbn(lam[t], scale) : lam[t];
   if (tid == 0 && info) *info = 0;
 }
 
