@@ -1468,15 +1468,6 @@ void ensure_product_operands(Ctx& c, DevMol& m) {
   }
 }
 
-template <int ROLE>
-void set_smem_attr(const void* fn, int bytes) {
-  static const bool once = [&] {
-    XS_CUDA(cudaFuncSetAttribute(fn, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes));
-    return true;
-  }();
-  (void)once;
-}
-
 // one Davidson iteration of the whole batch (the captured sequence)
 template <typename T, int MODE>
 int enqueue_iteration(cudaStream_t s, const BMol* mols, int* st, const BCfg& cfg, const double* par, int* nact,
@@ -1539,31 +1530,30 @@ int enqueue_iteration(cudaStream_t s, const BMol* mols, int* st, const BCfg& cfg
   return launches;
 }
 
+template <int ROLE>
+void allow_combine() {
+  static std::atomic<unsigned long long> done{0};
+  allow_smem(done, bcombine_kernel<ROLE>, 3 * kBatchMaxSub * 32 * 8);
+}
+template <GMode MODE>
+void allow_pair() {
+  static std::atomic<unsigned long long> done{0};
+  allow_smem(done, bgpair_kernel<MODE>, sizeof(float) * 100 * 256);
+}
+
 void set_attributes() {
-  constexpr int kCombSmem = 3 * kBatchMaxSub * 32 * 8;
-  static const bool eig_attr = [] {
-    XS_CUDA(cudaFuncSetAttribute(reinterpret_cast<const void*>(beig_kernel),
-                                 cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(sizeof(double) * kEigSmemDoubles)));
-    return true;
-  }();
-  (void)eig_attr;
-  static const bool pair_attr = [] {
-    for (const void* f : {reinterpret_cast<const void*>(bgpair_kernel<G_CIS>),
-                          reinterpret_cast<const void*>(bgpair_kernel<G_RPA>),
-                          reinterpret_cast<const void*>(bgpair_kernel<G_CIS_T>),
-                          reinterpret_cast<const void*>(bgpair_kernel<G_RPA_T>)})
-      XS_CUDA(cudaFuncSetAttribute(f, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   static_cast<int>(sizeof(float) * 100 * 256)));
-    return true;
-  }();
-  (void)pair_attr;
-  set_smem_attr<CB_RITZ_CIS>(reinterpret_cast<const void*>(bcombine_kernel<CB_RITZ_CIS>), kCombSmem);
-  set_smem_attr<CB_RITZ_RPA_R>(reinterpret_cast<const void*>(bcombine_kernel<CB_RITZ_RPA_R>), kCombSmem);
-  set_smem_attr<CB_RITZ_RPA_X>(reinterpret_cast<const void*>(bcombine_kernel<CB_RITZ_RPA_X>), kCombSmem);
-  set_smem_attr<CB_GS>(reinterpret_cast<const void*>(bcombine_kernel<CB_GS>), kCombSmem);
-  set_smem_attr<CB_APPEND>(reinterpret_cast<const void*>(bcombine_kernel<CB_APPEND>), kCombSmem);
-  set_smem_attr<CB_COLL>(reinterpret_cast<const void*>(bcombine_kernel<CB_COLL>), kCombSmem);
+  static std::atomic<unsigned long long> eig{0};
+  allow_smem(eig, beig_kernel, sizeof(double) * kEigSmemDoubles);
+  allow_pair<G_CIS>();
+  allow_pair<G_RPA>();
+  allow_pair<G_CIS_T>();
+  allow_pair<G_RPA_T>();
+  allow_combine<CB_RITZ_CIS>();
+  allow_combine<CB_RITZ_RPA_R>();
+  allow_combine<CB_RITZ_RPA_X>();
+  allow_combine<CB_GS>();
+  allow_combine<CB_APPEND>();
+  allow_combine<CB_COLL>();
 }
 
 struct GraphGuard {

@@ -5,6 +5,7 @@
 #include <cuda_fp16.h>
 #include <cuda_runtime.h>
 
+#include <atomic>
 #include <cstdio>
 #include <memory>
 #include <stdexcept>
@@ -44,6 +45,20 @@ struct Error : std::runtime_error {
       throw ::xs::Error(e_ == cudaErrorMemoryAllocation ? XS_ENOMEM : XS_ECUDA,            \
                         std::string(#call) + ": " + cudaGetErrorString(e_));                \
   } while (0)
+
+// Allows a kernel `bytes` of dynamic shared memory on the current device.  The
+// attribute holds for one device only, so `done` (a static of the launch site) has
+// a bit per device; setting it twice does no harm.
+template <typename K>
+void allow_smem(std::atomic<unsigned long long>& done, K* kernel, size_t bytes) {
+  int dev = 0;
+  XS_CUDA(cudaGetDevice(&dev));
+  const unsigned long long bit = dev < 64 ? 1ull << dev : 0;   // past 64 devices: set on every launch
+  if (done.load(std::memory_order_acquire) & bit) return;
+  XS_CUDA(cudaFuncSetAttribute(reinterpret_cast<const void*>(kernel), cudaFuncAttributeMaxDynamicSharedMemorySize,
+                               static_cast<int>(bytes)));
+  done.fetch_or(bit, std::memory_order_release);
+}
 
 #define XS_CHECK_LAUNCH()                                   \
   do {                                                      \

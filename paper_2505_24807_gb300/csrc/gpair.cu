@@ -73,12 +73,8 @@ template <GMode MODE, int SPLIT, int OUT>
 void launch_mode(cudaStream_t s, const DevMol& m, const double* d_par, int nvec, const float* W, const float* J2,
                  int ldj, const float* R, const PairOut& o) {
   const size_t smem = sizeof(float) * 100 * kPairThreads;
-  static const bool attr = [] {
-    XS_CUDA(cudaFuncSetAttribute(gpair_kernel<MODE, SPLIT, OUT>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(sizeof(float) * 100 * kPairThreads)));
-    return true;
-  }();
-  (void)attr;
+  static std::atomic<unsigned long long> allowed{0};
+  allow_smem(allowed, gpair_kernel<MODE, SPLIT, OUT>, smem);
   const int npairs = m.gp_npairs;
   const int ctas = (npairs + kPairThreads - 1) / kPairThreads;
   const int chunks = std::min(nvec, std::max(1, (kPairTargetCTAs + ctas - 1) / ctas));

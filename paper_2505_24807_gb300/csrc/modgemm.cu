@@ -678,12 +678,8 @@ int num_sms() {
 template <int BN>
 void launch_mg(cudaStream_t s, const MgOperand& A, const MgOperand& B, MgArgs a, int* err) {
   using C = MgCfg<BN>;
-  static const bool attr = [] {
-    XS_CUDA(cudaFuncSetAttribute(mg_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(C::SMEM)));
-    return true;
-  }();
-  (void)attr;
+  static std::atomic<unsigned long long> smem{0};
+  allow_smem(smem, mg_kernel<BN>, C::SMEM);
   const int Kp = mg_kp(A.K);
   const CUtensorMap ta = make_map(A.planes, Kp, A.rows, static_cast<long long>(kModuli) * A.batch, BM);
   const CUtensorMap tb = make_map(B.planes, Kp, B.rows, static_cast<long long>(kModuli) * B.batch, BN);
@@ -703,12 +699,8 @@ void split_side(cudaStream_t s, const MgOperand& op, MgPlanes& p) {
   const size_t plane = static_cast<size_t>(nrow) * Kp;
   if (op.ks == 1) {
     const size_t smem = sizeof(double) * Kp;
-    static const bool attr = [] {
-      XS_CUDA(cudaFuncSetAttribute(mg_split_rows<SIDE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   static_cast<int>(sizeof(double) * kMgMaxK)));
-      return true;
-    }();
-    (void)attr;
+    static std::atomic<unsigned long long> allowed{0};
+    allow_smem(allowed, mg_split_rows<SIDE>, sizeof(double) * kMgMaxK);
     mg_split_rows<SIDE><<<static_cast<unsigned>(nrow), kRowThreads, smem, s>>>(
         op.rows, op.K, Kp, op.src, op.rs, op.bs, p.planes.get(), plane, p.exps.get());
     XS_CHECK_LAUNCH();

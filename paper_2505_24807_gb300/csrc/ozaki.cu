@@ -557,12 +557,8 @@ template <int BN>
 void launch_oz(cudaStream_t s, const CUtensorMap& a0, const CUtensorMap& a1, const CUtensorMap& a2,
                const CUtensorMap& b, const OzArgs& args, int* err) {
   using C = OzCfg<BN>;
-  static const bool attr = [] {   // once per process (thread-safe initialisation)
-    XS_CUDA(cudaFuncSetAttribute(oz_kernel<BN>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(C::SMEM)));
-    return true;
-  }();
-  (void)attr;
+  static std::atomic<unsigned long long> smem{0};
+  allow_smem(smem, oz_kernel<BN>, C::SMEM);
   const int grid = std::min(args.ntiles, num_sms());   // persistent: one CTA per SM
   oz_kernel<BN><<<grid, 192, C::SMEM, s>>>(a0, a1, a2, b, args, err);
   XS_CHECK_LAUNCH();

@@ -53,6 +53,8 @@ __global__ void __launch_bounds__(1024) jacobi_kernel(int n, double* A, int lda,
 // rotations in the same order as the global-memory form.  The input A is left
 // unchanged.
 constexpr int kJacobiSmemMax = 64;
+constexpr size_t kJacobiSmemBytes = sizeof(double) * (2 * (size_t)kJacobiSmemMax * (kJacobiSmemMax + 1) +
+                                                      2 * kJacobiSmemMax) + sizeof(int) * kJacobiSmemMax;
 
 // the eigen-decomposition in shared memory (V, w in global memory)
 __device__ void jacobi_smem_body(int n, const double* __restrict__ A, int lda, double* __restrict__ V, int ldv,
@@ -208,14 +210,8 @@ void jacobi_eig(cudaStream_t s, int n, double* A, int lda, double* V, int ldv, d
   if (n <= kJacobiSmemMax) {
     // A, V (n x (n + 1)), scratch 2m doubles (c, s, and the pair indices), n ranks
     const size_t smem = sizeof(double) * (2 * (size_t)n * (n + 1) + 2 * m) + sizeof(int) * n;
-    static const bool attr = [] {   // once per process (thread-safe initialisation)
-      const size_t most = sizeof(double) * (2 * (size_t)kJacobiSmemMax * (kJacobiSmemMax + 1) + 2 * kJacobiSmemMax) +
-                          sizeof(int) * kJacobiSmemMax;
-      XS_CUDA(cudaFuncSetAttribute(jacobi_smem_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   static_cast<int>(most)));
-      return true;
-    }();
-    (void)attr;
+    static std::atomic<unsigned long long> allowed{0};
+    allow_smem(allowed, jacobi_smem_kernel, kJacobiSmemBytes);
     jacobi_smem_kernel<<<1, 256, smem, s>>>(n, A, lda, V, ldv, w, info, 60);
     XS_CHECK_LAUNCH();
     return;
@@ -238,13 +234,8 @@ void orthonormaliser(cudaStream_t s, int n, double* G, int ldg, double* V, int l
   ProfScope ps(s, "orth_f64", 0.0, 0.0);
   const int m = n + (n & 1);
   const size_t smem = sizeof(double) * (2 * (size_t)n * (n + 1) + 2 * m) + sizeof(int) * n;
-  static const bool attr = [] {   // once per process (thread-safe initialisation)
-    const size_t most = sizeof(double) * (2 * (size_t)kJacobiSmemMax * (kJacobiSmemMax + 1) + 2 * kJacobiSmemMax) +
-                        sizeof(int) * kJacobiSmemMax;
-    XS_CUDA(cudaFuncSetAttribute(orth_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(most)));
-    return true;
-  }();
-  (void)attr;
+  static std::atomic<unsigned long long> allowed{0};
+  allow_smem(allowed, orth_kernel, kJacobiSmemBytes);
   orth_kernel<<<1, 256, smem, s>>>(n, G, ldg, V, ldv, w, thresh, Bm, ldb, nkeep, info, 60);
   XS_CHECK_LAUNCH();
 }

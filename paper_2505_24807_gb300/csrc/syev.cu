@@ -71,12 +71,8 @@ void syevk(cudaStream_t s, int S, int k, const double* A, int lda, double* w, do
   if (S <= kSmemMax) {
     const bool zsm = syevk_z_fits(S, k);
     const size_t smem = sizeof(double) * (wd + (zsm ? syevk_z_doubles(S, k) : 0));
-    static const bool attr = [&] {   // once per process (thread-safe initialisation)
-      XS_CUDA(cudaFuncSetAttribute(syevk_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   static_cast<int>(sizeof(double) * kEigSmemDoubles)));
-      return true;
-    }();
-    (void)attr;
+    static std::atomic<unsigned long long> allowed{0};
+    allow_smem(allowed, syevk_kernel<true>, sizeof(double) * kEigSmemDoubles);
     syevk_kernel<true><<<1, 512, smem, s>>>(S, k, A, lda, w, Z, ldz, scratch.get(), info, zsm);
   } else {
     syevk_kernel<false><<<1, 1024, 0, s>>>(S, k, A, lda, w, Z, ldz, scratch.get(), info, false);
@@ -89,12 +85,8 @@ void cholesky(cudaStream_t s, int S, double* A, int lda, int* flag) {
   ProfScope ps(s, "cholesky_f64", 0.0, S * (double)S * S / 3.0);
   if (S <= kCholSmemMax) {
     const size_t smem = sizeof(double) * (size_t)S * (S + 1) / 2;
-    static const bool attr = [] {   // once per process (thread-safe initialisation)
-      XS_CUDA(cudaFuncSetAttribute(cholesky_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   static_cast<int>(sizeof(double) * kCholSmemMax * (kCholSmemMax + 1) / 2)));
-      return true;
-    }();
-    (void)attr;
+    static std::atomic<unsigned long long> allowed{0};
+    allow_smem(allowed, cholesky_kernel<true>, sizeof(double) * kCholSmemMax * (kCholSmemMax + 1) / 2);
     cholesky_kernel<true><<<1, 512, smem, s>>>(S, A, lda, flag);
   } else {
     cholesky_kernel<false><<<1, 1024, 0, s>>>(S, A, lda, flag);

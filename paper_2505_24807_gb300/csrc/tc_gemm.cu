@@ -747,12 +747,8 @@ void launch_tc(cudaStream_t s, const TcPair<T>& A, const TcPair<T>& B, int M, in
   const auto al16 = [](const void* p) { return reinterpret_cast<uintptr_t>(p) % 16 == 0; };
   ep.vec = e.ld % 4 == 0 && e.bstride % 4 == 0 && al16(e.D);
   const size_t smem = smem_bytes<BNv>();
-  static const bool attr_set = [smem] {   // once per process (thread-safe initialisation)
-    XS_CUDA(cudaFuncSetAttribute(tc_gemm_kernel<BNv, T, MODE>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 static_cast<int>(smem)));
-    return true;
-  }();
-  (void)attr_set;
+  static std::atomic<unsigned long long> allowed{0};
+  allow_smem(allowed, tc_gemm_kernel<BNv, T, MODE>, smem);
   const int ntm = (M + BM - 1) / BM, ntn = (N + BNv - 1) / BNv;
   const int ntiles = ntm * ntn * batch;
   const int nsm = sm_count();
