@@ -7,6 +7,7 @@
 
 #include <atomic>
 #include <cstdio>
+#include <map>
 #include <memory>
 #include <stdexcept>
 #include <string>
@@ -90,6 +91,18 @@ struct DevBuf {
   void ensure(size_t count) { if (count > n) alloc(count); }
   void release() { if (p) cudaFree(p); p = nullptr; n = 0; }
   T* get() const { return p; }
+};
+
+// Scratch that a launch site keeps (a static thread_local there): a buffer per device
+// that the thread has used.
+template <typename T>
+struct ThreadScratch {
+  std::map<int, DevBuf<T>> buf;
+  DevBuf<T>& here() {
+    int dev = 0;
+    XS_CUDA(cudaGetDevice(&dev));
+    return buf[dev];
+  }
 };
 
 // Device copy of one molecule's ground state and integrals.

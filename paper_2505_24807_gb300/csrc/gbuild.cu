@@ -359,8 +359,8 @@ void gbuild<float>(cudaStream_t s, const DevMol& m, const double* d_par, GMode m
     pack_diag_kernel<float><<<grid, block, 0, s>>>(m.L.natoms, n, np, nvec, m.atom_ao_off.get(), m.atom_nao.get(),
                                                    m.atom_prod_off.get(), R, rT);
     XS_CHECK_LAUNCH();
-    static thread_local DevBuf<float> j2_ws;
-    coulomb_j2(s, np, nvec, W, rT, J2, j2_ws);
+    static thread_local ThreadScratch<float> j2_ws;
+    coulomb_j2(s, np, nvec, W, rT, J2, j2_ws.here());
   }
   // algorithmic traffic: read R, write G (and G-), read the pair integrals once
   const double outs = (G ? 1.0 : 0.0) + (Gm ? 1.0 : 0.0);
@@ -396,8 +396,8 @@ void gbuild_split(cudaStream_t s, const DevMol& m, const double* d_par, GMode mo
     pack_diag_kernel<float><<<grid, block, 0, s>>>(m.L.natoms, n, np, nvec, m.atom_ao_off.get(),
                                                           m.atom_nao.get(), m.atom_prod_off.get(), R, rT);
     XS_CHECK_LAUNCH();
-    static thread_local DevBuf<float> j2_ws;
-    coulomb_j2(s, np, nvec, W, rT, J2, j2_ws);
+    static thread_local ThreadScratch<float> j2_ws;
+    coulomb_j2(s, np, nvec, W, rT, J2, j2_ws.here());
   }
   if (ldo > n) {
     const long long cnt = (long long)nvec * n * (ldo - n);

@@ -262,8 +262,8 @@ void gbuild_half(cudaStream_t s, const DevMol& m, const double* d_par, GMode mod
     pack_diag_kernel<float><<<(m.L.natoms + 31) / 32, dim3(8, 32), 0, s>>>(
         m.L.natoms, n, np, nvec, m.atom_ao_off.get(), m.atom_nao.get(), m.atom_prod_off.get(), R, r);
     XS_CHECK_LAUNCH();
-    static thread_local DevBuf<float> j2_ws;
-    coulomb_j2(s, np, nvec, m.Wf.get(), r, J2, j2_ws);
+    static thread_local ThreadScratch<float> j2_ws;
+    coulomb_j2(s, np, nvec, m.Wf.get(), r, J2, j2_ws.here());
   }
   g_exponents_kernel<<<nvec, 256, 0, s>>>(np, nvec, coulomb ? J2 : nullptr, nvec, rmax, wmax, d_par, o.e, o.em);
   XS_CHECK_LAUNCH();

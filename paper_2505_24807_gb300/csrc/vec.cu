@@ -242,7 +242,8 @@ void residual_norms(cudaStream_t s, int nvec, long long len, const double* A, co
   // thread spend their time there (10 rows of 90000: 17 us with 256 CTAs a row)
   const int blocks = static_cast<int>(
       std::max<long long>(1, std::min<long long>((8LL * 152 + nvec - 1) / nvec, (len + 2047) / 2048)));
-  static thread_local DevBuf<double> part;
+  static thread_local ThreadScratch<double> scratch;
+  DevBuf<double>& part = scratch.here();
   part.ensure((size_t)nvec * blocks);
   ProfScope ps(s, "resid_norms", 8.0 * nvec * len * (B ? 2.0 : 1.0) + (R ? 8.0 * nvec * len : 0.0), 0.0);
   resid_kernel<<<dim3(blocks, nvec), 256, 0, s>>>(len, A, B, omega, part.get(), R);

@@ -1,6 +1,6 @@
 """Calls on two devices of one process, one after the other: a kernel's shared-memory
 limit holds for the device that was current when it was set, so each device needs
-its own."""
+its own, and scratch that outlives a call lies on the device that the call ran on."""
 from tests import fake_cuda
 
 SCRIPT = """
@@ -30,7 +30,9 @@ def every_path(device):
                     assert e.status != xs.XS_ECUDA, e
     xs.xs_destroy(h)
 every_path(0)
+assert fake.fake_used(0) > 0 and fake.fake_used(1) == 0
 every_path(1)
+assert fake.fake_used(1) == fake.fake_used(0)
 print("both devices")
 """
 
