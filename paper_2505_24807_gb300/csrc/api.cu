@@ -37,11 +37,7 @@ int guarded(xs_ctx* ctx, F&& f) {
     XS_CUDA(cudaSetDevice(ctx->c.device));
     return f(ctx->c);
   } catch (const Error& e) {
-    if (e.status == XS_ENOMEM) {   // give back what is only kept for speed
-      ctx->c.io.release();
-      ctx->c.oz_work.reset();
-      ctx->c.mg_work.reset();
-    }
+    if (e.status == XS_ENOMEM) ctx->c.release_kept();
     ctx->c.err = e.what();
     return e.status;
   } catch (const std::bad_alloc&) {
@@ -234,8 +230,7 @@ int xs_ground_state(xs_ctx* ctx, int n_mol, const int* natoms, const int* Z, con
     if (!(scf_tol > 0.0)) scf_tol = 1e-10;
     if (max_iter <= 0) max_iter = 300;
     cudaStream_t s = c.stream;
-    c.io.release();
-    c.oz_work.reset();
+    c.release_kept();
     c.mols.clear();
     c.mols.resize(n_mol);
     int off = 0, maxit = 0;
@@ -382,7 +377,7 @@ int xs_excited(xs_ctx* ctx, const xs_ex_opts* opts, double* omega, double* osc, 
     std::vector<int> rcs(nmol, XS_OK);
     if (o.batched < 0 || o.batched > 2) throw Error(XS_EINVAL, "batched must be 0, 1 or 2");
     const int form = o.batched;
-    if (form != 0) c.io.release();   // batched solvers size their arenas by the free memory
+    if (form != 0) c.release_kept();   // the batch's arenas, or the workers' subspaces, share the free memory
     if (form == 1) {
       long long replays = 0;
       xs::davidson_batched(c, o, stats, rcs, &replays);

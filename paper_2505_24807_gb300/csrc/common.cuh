@@ -141,8 +141,7 @@ struct DevMol {
 // between calls: a cudaMalloc / cudaFree pair costs 20 to 800 us by size, and
 // the cudaFree waits for the device (a 120 x 20 subspace projection over 373100
 // amplitudes took 1.9 ms for 0.6 ms of kernels).  Held memory is bounded: an
-// entry calls trim() at its end, and ground states and Davidson solves that run
-// short of memory release it.
+// entry calls trim() at its end, and Ctx::release_kept gives it back.
 struct CallScratch {
   static constexpr int kSlots = 5;
   static constexpr size_t kKeep = size_t(2) << 30;   // bytes kept between calls
@@ -185,6 +184,16 @@ struct Ctx {
   std::vector<std::unique_ptr<Ctx>> workers;
   // learned guess / preconditioner network (shared by the workers)
   std::shared_ptr<Mlp> mlp;
+
+  // Gives back the scratch that is kept between calls for speed alone and rebuilt on
+  // use (staged arrays, digits, residues), the workers' too: where molecules change,
+  // before solvers that share the device's memory out, and when memory runs short.
+  void release_kept() {
+    io.release();
+    oz_work.reset();
+    mg_work.reset();
+    for (auto& w : workers) w->release_kept();
+  }
 };
 
 inline dim3 grid1(long long n, int block) { return dim3(static_cast<unsigned>((n + block - 1) / block)); }

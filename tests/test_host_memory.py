@@ -1,0 +1,49 @@
+"""Device memory that contexts keep between calls, counted on the CPU against a
+stand-in for the CUDA runtime: given back where it is said to be."""
+import pytest
+
+from tests import fake_cuda
+
+SETUP = """
+Z, xyz = molgen.make_chain(3, 40, 62)          # 222 AOs: residue products in float64
+mols = [(Z, xyz), (Z, xyz)]
+rng = np.random.default_rng(0)
+"""
+
+GIVEN_BACK = """
+def every_scratch(h):
+    global n, o
+    n, o, _ = xs.xs_get_sizes(h, 0)
+    xs.xs_apply(h, 0, xs.XS_KIND_APB, rng.standard_normal((20, o * (n - o))))
+    xs.xs_subspace_gram(h, rng.standard_normal((40, 20000)), rng.standard_normal((4, 20000)))
+    xs.xs_subspace_combine(h, rng.standard_normal((2, 12, 20000)), rng.standard_normal((2, 12, 4)))
+def solve(h):
+    try:
+        xs.xs_excited(h, nroots=3, tol=1e-6, batched=FORM)
+    except xs.XSError:
+        pass                                   # nothing converges here
+h = context()
+xs.xs_ground_state(h, mols)
+every_scratch(h)
+if FORM is not None:
+    solve(h)                                   # what the solver itself keeps
+every_scratch(h)
+kept = fake.fake_used(0)
+if FORM is None:
+    xs.xs_ground_state(h, mols)
+else:
+    solve(h)
+# residues of 20 vectors: 13 bfloat16 planes of W (n x 128), G and the result (n x 256 and n x 224)
+residues = 13 * 2 * 20 * 222 * (128 + 256 + 224)
+# arrays staged for 20 vectors, 44 vectors of digits
+staged = 2 * 8 * 20 * o * (n - o) + 8 * 44 * 20000 + 16 * 44 * 20000
+assert kept - fake.fake_used(0) > residues + staged // 2, (kept - fake.fake_used(0), residues, staged)
+print("given back")
+"""
+
+
+@pytest.mark.parametrize("form", [None, 1, 2])
+def test_scratch_given_back(tmp_path, form):
+    """Ground states (None), the lock-step batch and concurrent molecules give back
+    the scratch of products and subspace entries."""
+    assert "given back" in fake_cuda.run(tmp_path, SETUP + f"FORM = {form}\n" + GIVEN_BACK)
