@@ -370,10 +370,11 @@ int davidson(Ctx& c, DevMol& m, const xs_ex_opts& opt, SolveStats& st) {
     const double per_vec = 8.0 * nstore * ov + (use_oz ? 16.0 * (double)oz_lp(ov) + 16.0 * nstore * ov : 0.0);
     double budget = opt.memory_limit;
     if (!(budget > 0.0)) {
-      size_t free_b = 0, total_b = 0;
-      XS_CUDA(cudaMemGetInfo(&free_b, &total_b));
-      // scratch of other entries counts as free: given back when the cap needs it
-      for (auto& b : c.io.buf) free_b += b.n;
+      auto free_bytes = []() {
+        size_t free_b = 0, total_b = 0;
+        XS_CUDA(cudaMemGetInfo(&free_b, &total_b));
+        return (double)free_b;
+      };
       double held = 0.0;   // this context's subspace buffers are reused
       if (c.dav_cache) {
         const Work& w0 = *static_cast<const Work*>(c.dav_cache.get());
@@ -382,17 +383,24 @@ int davidson(Ctx& c, DevMol& m, const xs_ex_opts& opt, SolveStats& st) {
       // reserve: Ritz vectors, residuals, new directions and their digit
       // scratch (a few 2k-row blocks of amplitudes), product scratch, headroom
       const double reserve = 8.0 * ov * (8.0 * kk + 8.0) + 32.0 * ov * (2.0 * kk + 2.0) + 4.0 * 1073741824.0;
-      budget = (double)free_b + held - reserve;
+      // float64 products run without their residue scratch when it does not fit, but fifty times slower at 2200 AOs
+      const int widest = std::max(nguess, maxnew);
+      auto residues = [&]() { return opt.precision == XS_FP64 ? (double)residue_bytes(c, m, widest) : 0.0; };
+      double extra = residues();
+      budget = free_bytes() + held - reserve;
+      if (std::floor((budget - extra) / per_vec) < Smax) {   // what other calls left behind makes room
+        c.release_kept();
+        extra = residues();
+        budget = free_bytes() + held - reserve;
+      }
+      if (std::floor((budget - extra) / per_vec) >= Smin) budget -= extra;
     }
     const double cap = std::floor(budget / per_vec);
     if (cap < Smin)
       throw Error(XS_ENOMEM, "subspace needs " + std::to_string(static_cast<long long>(Smin * per_vec)) +
                                  " bytes for its first " + std::to_string(Smin) + " vectors; budget " +
                                  std::to_string(static_cast<long long>(budget)));
-    if (cap < Smax) {
-      Smax = static_cast<int>(cap);
-      c.io.release();
-    }
+    if (cap < Smax) Smax = static_cast<int>(cap);
   }
   st.smax = Smax;
   // Mixed-precision products carry rounding noise of ~1e-6 relative, so their

@@ -80,6 +80,23 @@ bool mg_applies(const DevMol& m, int nvec) {
   return m.n >= 160 || 4.0 * nvec * (n * o * v + n * n * v) >= 8e7;
 }
 
+// vectors per pass of the residue products: kMgBytes of planes
+int mg_chunk(const DevMol& m, int nvec) {
+  const double per = 2.0 * kModuli * m.n * (2.0 * mg_kp(m.n) + mg_kp(m.v));
+  return std::max(1, std::min(std::min(nvec, product_batch(m)), static_cast<int>(kMgBytes / per)));
+}
+
+// scratch of a pass (mg_prepare) and operands of the orbitals
+size_t mg_scratch_bytes(const DevMol& m, int chunk) {
+  return sizeof(mg_t) * (mg_plane_count(m.n, m.v, chunk) +
+                         std::max(mg_plane_count(m.n, m.n, chunk), mg_plane_count(m.v, m.o, chunk)) +
+                         (size_t)kModuli * chunk * m.n * mg_ldn(m.n)) + sizeof(int) * 2 * (size_t)chunk * m.n;
+}
+size_t mg_orbital_bytes(const DevMol& m) {
+  return sizeof(mg_t) * (mg_plane_count(m.n, m.o, 1) + mg_plane_count(m.n, m.v, 1) + mg_plane_count(m.v, m.n, 1) +
+                         mg_plane_count(m.o, m.n, 1)) + sizeof(int) * 3 * (size_t)m.n;
+}
+
 // operands and scratch for the residue products of `chunk` vectors, or null
 // where they do not fit the device (the float64-pipe path serves those)
 MgOrbitals* mg_prepare(Ctx& c, DevMol& m, int chunk) {
@@ -168,6 +185,17 @@ int product_batch(const DevMol& m) {
   return nb;
 }
 
+size_t residue_bytes(const Ctx& c, const DevMol& m, int nvec) {
+  if (!mg_applies(m, nvec)) return 0;
+  size_t held = 0;
+  if (c.mg_work) {
+    const MgWork& w = *static_cast<const MgWork*>(c.mg_work.get());
+    held = sizeof(mg_t) * (w.a.planes.n + w.b.planes.n + w.res.n) + sizeof(int) * (w.a.exps.n + w.b.exps.n);
+  }
+  const size_t need = mg_scratch_bytes(m, mg_chunk(m, nvec));
+  return (need > held ? need - held : 0) + (m.mg_orb ? 0 : mg_orbital_bytes(m));
+}
+
 void products_fp64(Ctx& c, DevMol& m, int method, int nvec, const double* X, double* Y1, double* Y2, bool triplet) {
   cudaStream_t s = c.stream;
   const int n = m.n, o = m.o, v = m.v;
@@ -176,8 +204,7 @@ void products_fp64(Ctx& c, DevMol& m, int method, int nvec, const double* X, dou
   int chunk = nvec < nb ? nvec : nb;
   MgOrbitals* q = nullptr;
   if (mg_applies(m, nvec)) {
-    const double per = 2.0 * kModuli * n * (2.0 * mg_kp(n) + mg_kp(v));
-    const int mc = std::max(1, std::min(chunk, static_cast<int>(kMgBytes / per)));
+    const int mc = mg_chunk(m, nvec);
     q = mg_prepare(c, m, mc);
     if (q) chunk = mc;
   }

@@ -17,6 +17,8 @@ constexpr int kPrecF32 = 2;
 // digit split of the Davidson subspace needs it).
 void products(Ctx& c, DevMol& m, int method, int precision, int nvec, const double* X, double* Y1, double* Y2,
               bool triplet = false, unsigned int* mx1 = nullptr, unsigned int* mx2 = nullptr);
+// Device memory that float64 products of nvec vectors would still allocate to run as residue products (0: they do not)
+size_t residue_bytes(const Ctx& c, const DevMol& m, int nvec);
 void products_fp64(Ctx& c, DevMol& m, int method, int nvec, const double* X, double* Y1, double* Y2,
                    bool triplet = false);
 // G_CIS(R) of nvec AO matrices (float64 device arrays)

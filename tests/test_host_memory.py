@@ -47,3 +47,44 @@ def test_scratch_given_back(tmp_path, form):
     """Ground states (None), the lock-step batch and concurrent molecules give back
     the scratch of products and subspace entries."""
     assert "given back" in fake_cuda.run(tmp_path, SETUP + f"FORM = {form}\n" + GIVEN_BACK)
+
+
+BUDGET = """
+h = context()
+xs.xs_ground_state(h, mols[:1])
+n, o, _ = xs.xs_get_sizes(h, 0)
+GB = 1 << 30
+def solve():
+    fake.fake_reset_peak(0)
+    try:
+        xs.xs_excited(h, nroots=6, tol=1e-6, max_subspace=400, precision=PRECISION)
+    except xs.XSError as e:
+        assert e.status != xs.XS_ENOMEM, e     # nothing converges here
+    return fake.fake_peak(0)
+fresh = fake.fake_used(0)
+solve()                                        # 400 vectors and their products
+most = fake.fake_peak(0) - fresh
+xs.xs_destroy(h)
+h = context()
+xs.xs_ground_state(h, mols[:1])
+if KEPT == "staged":                           # staged arrays and digits of another call
+    xs.xs_subspace_gram(h, rng.standard_normal((60, 100000)), rng.standard_normal((4, 100000)))
+else:                                          # residues
+    xs.xs_apply(h, 0, xs.XS_KIND_A, rng.standard_normal((60, o * (n - o))))
+kept = fake.fake_used(0) - fresh
+assert kept > 100 << 20, kept
+# room for the subspace (X and its products) and the reserve of 4 GB, but only without what is kept
+fake.fake_set_capacity(0, fake.fake_used(0) + 16 * 400 * o * (n - o) + 4 * GB - kept // 2)
+solve()
+assert fake.fake_used(0) < fresh + most + kept // 2, (fake.fake_used(0) - fresh - most, kept)
+print("given back")
+"""
+
+
+@pytest.mark.parametrize("kept", ["staged", "residues"])
+@pytest.mark.parametrize("precision", [0, 1])
+def test_solve_short_of_memory(tmp_path, kept, precision):
+    """A solve short of memory gives back what other calls left behind instead of
+    spending the memory that it reserves for its own scratch."""
+    script = SETUP + f"KEPT, PRECISION = {kept!r}, {precision}\n" + BUDGET
+    assert "given back" in fake_cuda.run(tmp_path, script)
