@@ -25,28 +25,56 @@ using xs::Error;
 
 namespace {
 
+// Runs an entry's body and turns its exceptions into statuses.  What is kept between
+// calls for speed must not cost a call its memory: a body that ran out of memory is
+// run again (may_retry: from its start, to the same result), first after the kept
+// scratch has been given back, then without the float64 products' residues.
+template <typename F, typename R>
+int guarded(xs_ctx* ctx, F&& f, R&& may_retry) {
+  if (!ctx) return XS_EINVAL;
+  Ctx& c = ctx->c;
+  c.err.clear();
+  struct Bind {
+    Ctx& c;
+    explicit Bind(Ctx& ctx) : c(ctx) { xs::g_prof = &c.prof; }
+    ~Bind() {
+      xs::g_prof = nullptr;
+      c.set_residues(true);
+    }
+  } bind(c);
+  int tried = 0;   // 1: kept scratch given back, 2: no residues either
+  for (;;) {
+    try {
+      XS_CUDA(cudaSetDevice(c.device));
+      return f(c);
+    } catch (const Error& e) {
+      if (e.status == XS_ENOMEM) {
+        cudaGetLastError();
+        const bool held = c.release_kept();
+        if (tried == 0 && held && may_retry()) {
+          tried = 1;
+          continue;
+        }
+        if (tried < 2 && (c.set_residues(false) || held) && may_retry()) {
+          tried = 2;
+          continue;
+        }
+      }
+      c.err = e.what();
+      return e.status;
+    } catch (const std::bad_alloc&) {
+      c.err = "host allocation failed";
+      return XS_ENOMEM;
+    } catch (const std::exception& e) {
+      c.err = e.what();
+      return XS_ECUDA;
+    }
+  }
+}
+
 template <typename F>
 int guarded(xs_ctx* ctx, F&& f) {
-  if (!ctx) return XS_EINVAL;
-  ctx->c.err.clear();
-  struct Bind {
-    Bind(xs::Profiler* p) { xs::g_prof = p; }
-    ~Bind() { xs::g_prof = nullptr; }
-  } bind(&ctx->c.prof);
-  try {
-    XS_CUDA(cudaSetDevice(ctx->c.device));
-    return f(ctx->c);
-  } catch (const Error& e) {
-    if (e.status == XS_ENOMEM) ctx->c.release_kept();
-    ctx->c.err = e.what();
-    return e.status;
-  } catch (const std::bad_alloc&) {
-    ctx->c.err = "host allocation failed";
-    return XS_ENOMEM;
-  } catch (const std::exception& e) {
-    ctx->c.err = e.what();
-    return XS_ECUDA;
-  }
+  return guarded(ctx, std::forward<F>(f), [] { return true; });
 }
 
 DevMol& molecule(Ctx& c, int mol) {
@@ -662,6 +690,8 @@ int xs_mlp_grad(xs_ctx* ctx, int rows, const float* features, const float* targe
 
 int xs_mlp_train(xs_ctx* ctx, int rows, const float* features, const float* targets, int epochs, int batch,
                  float lr, float* loss) {
+  const long long step0 = ctx && ctx->c.mlp ? ctx->c.mlp->step : 0;
+  auto untrained = [&] { return !ctx->c.mlp || ctx->c.mlp->step == step0; };   // else a second run would train twice
   return guarded(ctx, [&](Ctx& c) {
     if (!c.mlp || !c.mlp->ready) throw Error(XS_ESTATE, "initialise or load the network first");
     if (rows <= 0 || epochs <= 0 || batch <= 0 || !features || !targets) throw Error(XS_EINVAL, "bad request");
@@ -684,7 +714,7 @@ int xs_mlp_train(xs_ctx* ctx, int rows, const float* features, const float* targ
       if (loss) loss[e] = static_cast<float>(sum / nb);
     }
     return XS_OK;
-  });
+  }, untrained);
 }
 
 int xs_profile(xs_ctx* ctx, int enable) {

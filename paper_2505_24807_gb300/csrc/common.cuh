@@ -188,11 +188,32 @@ struct Ctx {
   // Gives back the scratch that is kept between calls for speed alone and rebuilt on
   // use (staged arrays, digits, residues), the workers' too: where molecules change,
   // before solvers that share the device's memory out, and when memory runs short.
-  void release_kept() {
+  // True if anything was held.
+  bool release_kept() {
+    bool held = oz_work || mg_work;
+    for (auto& b : io.buf) held = held || b.n > 0;
     io.release();
     oz_work.reset();
     mg_work.reset();
-    for (auto& w : workers) w->release_kept();
+    for (auto& w : workers) held = w->release_kept() || held;
+    return held;
+  }
+  // Whether float64 products may use residue products (products.cu); off: the
+  // molecules' residue operands are given back too, true if there were any.
+  bool residues = true;
+  bool set_residues(bool on) {
+    residues = on;
+    for (auto& w : workers) w->residues = on;
+    return !on && drop_operands(nullptr);
+  }
+  bool drop_operands(const DevMol* except) {
+    bool held = false;
+    for (auto& m : mols)
+      if (&m != except && m.mg_orb) {
+        m.mg_orb.reset();
+        held = true;
+      }
+    return held;
   }
 };
 

@@ -98,11 +98,12 @@ size_t mg_orbital_bytes(const DevMol& m) {
 }
 
 // operands and scratch for the residue products of `chunk` vectors, or null
-// where they do not fit the device (the float64-pipe path serves those)
+// where they do not fit the device beside those of the other molecules, which are
+// dropped first (the float64-pipe path serves those)
 MgOrbitals* mg_prepare(Ctx& c, DevMol& m, int chunk) {
   const int n = m.n, o = m.o, v = m.v;
   cudaStream_t s = c.stream;
-  try {
+  for (;;) try {
     if (!c.mg_work) c.mg_work = std::make_shared<MgWork>();
     MgWork& w = *static_cast<MgWork*>(c.mg_work.get());
     w.a.planes.ensure(mg_plane_count(n, v, chunk));
@@ -134,7 +135,7 @@ MgOrbitals* mg_prepare(Ctx& c, DevMol& m, int chunk) {
     if (e.status != XS_ENOMEM) throw;
     cudaGetLastError();
     c.mg_work.reset();
-    return nullptr;
+    if (!c.drop_operands(&m)) return nullptr;
   }
 }
 
@@ -186,7 +187,7 @@ int product_batch(const DevMol& m) {
 }
 
 size_t residue_bytes(const Ctx& c, const DevMol& m, int nvec) {
-  if (!mg_applies(m, nvec)) return 0;
+  if (!c.residues || !mg_applies(m, nvec)) return 0;
   size_t held = 0;
   if (c.mg_work) {
     const MgWork& w = *static_cast<const MgWork*>(c.mg_work.get());
@@ -203,7 +204,7 @@ void products_fp64(Ctx& c, DevMol& m, int method, int nvec, const double* X, dou
   const int nb = product_batch(m);
   int chunk = nvec < nb ? nvec : nb;
   MgOrbitals* q = nullptr;
-  if (mg_applies(m, nvec)) {
+  if (c.residues && mg_applies(m, nvec)) {
     const int mc = mg_chunk(m, nvec);
     q = mg_prepare(c, m, mc);
     if (q) chunk = mc;

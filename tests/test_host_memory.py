@@ -88,3 +88,58 @@ def test_solve_short_of_memory(tmp_path, kept, precision):
     spending the memory that it reserves for its own scratch."""
     script = SETUP + f"KEPT, PRECISION = {kept!r}, {precision}\n" + BUDGET
     assert "given back" in fake_cuda.run(tmp_path, script)
+
+
+RETRY = """
+h = context()
+xs.xs_mlp_init(h, 1)
+xs.xs_ground_state(h, mols)
+n, o, _ = xs.xs_get_sizes(h, 0)
+X, R = rng.standard_normal((20, o * (n - o))), rng.standard_normal((30, n, n))
+F, T = np.zeros((4000, 11), np.float32), np.zeros((4000, 2), np.float32)
+calls = [lambda: xs.xs_get_orbitals(h, 0),
+         lambda: xs.xs_subspace_eig(h, np.eye(300), 10),
+         lambda: xs.xs_apply(h, 0, xs.XS_KIND_APB, X, precision=xs.XS_MIXED),
+         lambda: xs.xs_apply(h, 1, xs.XS_KIND_G, R),
+         lambda: xs.xs_mlp_train(h, F, T, 1, 4000, 1e-3),
+         lambda: xs.xs_ground_state(h, mols)]
+for call in calls:
+    # staged arrays, digits and the residues of both molecules, which fill the device
+    xs.xs_subspace_gram(h, rng.standard_normal((60, 100000)), rng.standard_normal((4, 100000)))
+    for mol in (0, 1):
+        xs.xs_apply(h, mol, xs.XS_KIND_A, rng.standard_normal((60, o * (n - o))))
+    fake.fake_set_capacity(0, fake.fake_used(0) + (64 << 10))
+    call()
+    fake.fake_set_capacity(0, 1 << 40)
+print("ran")
+"""
+
+
+def test_kept_scratch_costs_no_call_its_memory(tmp_path):
+    """Calls run, the first time, also where the scratch that earlier calls left
+    behind fills the device."""
+    assert "ran" in fake_cuda.run(tmp_path, SETUP + RETRY)
+
+
+FALLBACK = """
+planes = work = None
+for share in (0.25, 0.5, 0.9):
+    h = context()
+    xs.xs_ground_state(h, mols)
+    n, o, _ = xs.xs_get_sizes(h, 0)
+    X = rng.standard_normal((20, o * (n - o)))
+    planes = 13 * 2 * (20 * n * (128 + 256 + 224) + 4 * n * 128)
+    work = 8 * 20 * (2 * n * n + n * (n - o)) + 8 * 2 * X.size   # R, G, transform scratch, staged vectors
+    assert planes > work + (8 << 20)                             # the work arrays fit by themselves
+    fake.fake_set_capacity(0, fake.fake_used(0) + planes + int(share * work))
+    xs.xs_apply(h, 0, xs.XS_KIND_A, X)
+    fake.fake_set_capacity(0, 1 << 40)
+    xs.xs_destroy(h)
+print("ran")
+"""
+
+
+def test_products_fall_back_to_the_float64_pipe(tmp_path):
+    """A float64 product whose work arrays do not fit beside the residue planes runs
+    without the planes, as it did before there were any."""
+    assert "ran" in fake_cuda.run(tmp_path, SETUP + FALLBACK)
