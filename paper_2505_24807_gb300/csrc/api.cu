@@ -25,6 +25,14 @@ using xs::Error;
 
 namespace {
 
+// After a failure in mid-call: kernels and copies already launched may use the caller's
+// arrays, and the body did not come to its trim()
+void abandon(Ctx& c) {
+  cudaStreamSynchronize(c.stream);
+  cudaGetLastError();
+  c.io.trim();
+}
+
 // Runs an entry's body and turns its exceptions into statuses.  What is kept between
 // calls for speed must not cost a call its memory: a body that ran out of memory is
 // run again (may_retry: from its start, to the same result), first after the kept
@@ -60,12 +68,15 @@ int guarded(xs_ctx* ctx, F&& f, R&& may_retry) {
           continue;
         }
       }
+      if (e.status != XS_EINVAL && e.status != XS_ESTATE) abandon(c);
       c.err = e.what();
       return e.status;
     } catch (const std::bad_alloc&) {
+      abandon(c);
       c.err = "host allocation failed";
       return XS_ENOMEM;
     } catch (const std::exception& e) {
+      abandon(c);
       c.err = e.what();
       return XS_ECUDA;
     }

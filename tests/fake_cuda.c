@@ -21,7 +21,7 @@ static int nblocks;
 static size_t capacity[2] = {(size_t)1 << 40, (size_t)1 << 40}, used[2], peak[2];
 static struct { const void* f; size_t n[2]; } attrs[MAX_ATTR];
 static int nattrs;
-static long long launches, syncs;
+static long long pending;   /* launches since the device was last waited for */
 static __thread int cur;
 static __thread cudaError_t last;
 static __thread struct { dim3 g, b; size_t smem; void* s; } conf;
@@ -31,8 +31,13 @@ void fake_set_capacity(int dev, size_t bytes) { capacity[dev] = bytes; }
 size_t fake_used(int dev) { return used[dev]; }
 size_t fake_peak(int dev) { return peak[dev]; }
 void fake_reset_peak(int dev) { peak[dev] = used[dev]; }
-long long fake_launches(void) { return launches; }
-long long fake_syncs(void) { return syncs; }
+long long fake_pending(void) { return pending; }
+/* sets every word of the device blocks of n bytes */
+void fake_fill(size_t n, int word) {
+  for (int i = 0; i < nblocks; ++i)
+    if (blocks[i].n == n)
+      for (size_t k = 0; k < n / 4; ++k) ((int*)blocks[i].p)[k] = word;
+}
 
 static cudaError_t fail(cudaError_t e) { return last = e; }
 
@@ -57,6 +62,7 @@ cudaError_t cudaFree(void* p) {
   if (!p) return cudaSuccess;
   pthread_mutex_lock(&mu);
   cudaError_t e = cudaErrorInvalidValue;
+  pending = 0;
   for (int i = nblocks - 1; i >= 0; --i)
     if (blocks[i].p == p) {
       munmap(p, blocks[i].n);
@@ -135,7 +141,7 @@ static cudaError_t launch(const void* f, size_t smem) {
   pthread_mutex_lock(&mu);
   for (int i = 0; i < nattrs; ++i)
     if (attrs[i].f == f && attrs[i].n[cur] > allowed) allowed = attrs[i].n[cur];
-  ++launches;
+  ++pending;
   pthread_mutex_unlock(&mu);
   return smem > allowed ? fail(cudaErrorInvalidValue) : cudaSuccess;
 }
@@ -161,7 +167,7 @@ void __cudaRegisterVar(void** h, char* v, char* d, const char* n, int e, size_t 
 
 cudaError_t cudaStreamCreateWithFlags(cudaStream_t* s, unsigned f) { (void)f; static char h; *s = (cudaStream_t)&h; return cudaSuccess; }
 cudaError_t cudaStreamDestroy(cudaStream_t s) { (void)s; return cudaSuccess; }
-cudaError_t cudaStreamSynchronize(cudaStream_t s) { (void)s; ++syncs; return cudaSuccess; }
+cudaError_t cudaStreamSynchronize(cudaStream_t s) { (void)s; pending = 0; return cudaSuccess; }
 cudaError_t cudaStreamIsCapturing(cudaStream_t s, enum cudaStreamCaptureStatus* c) { (void)s; *c = cudaStreamCaptureStatusNone; return cudaSuccess; }
 cudaError_t cudaStreamBeginCapture(cudaStream_t s, enum cudaStreamCaptureMode m) { (void)s; (void)m; return cudaSuccess; }
 cudaError_t cudaStreamEndCapture(cudaStream_t s, cudaGraph_t* g) { (void)s; static char h; *g = (cudaGraph_t)&h; return cudaSuccess; }
@@ -172,7 +178,7 @@ cudaError_t cudaGraphDestroy(cudaGraph_t g) { (void)g; return cudaSuccess; }
 cudaError_t cudaEventCreate(cudaEvent_t* e) { static char h; *e = (cudaEvent_t)&h; return cudaSuccess; }
 cudaError_t cudaEventDestroy(cudaEvent_t e) { (void)e; return cudaSuccess; }
 cudaError_t cudaEventRecord(cudaEvent_t e, cudaStream_t s) { (void)e; (void)s; return cudaSuccess; }
-cudaError_t cudaEventSynchronize(cudaEvent_t e) { (void)e; return cudaSuccess; }
+cudaError_t cudaEventSynchronize(cudaEvent_t e) { (void)e; pending = 0; return cudaSuccess; }
 cudaError_t cudaEventElapsedTime(float* ms, cudaEvent_t a, cudaEvent_t b) { (void)a; (void)b; *ms = 1.0f; return cudaSuccess; }
 
 int cusolverDnCreate(void** h) { static char x; *h = &x; return 0; }

@@ -14,7 +14,15 @@ from paper_2505_24807_gb300 import xs
 fake = ctypes.CDLL(None)
 fake.fake_used.restype = fake.fake_peak.restype = ctypes.c_size_t
 fake.fake_set_capacity.argtypes = [ctypes.c_int, ctypes.c_size_t]
-fake.fake_launches.restype = fake.fake_syncs.restype = ctypes.c_longlong
+fake.fake_pending.restype = ctypes.c_longlong
+fake.fake_fill.argtypes = [ctypes.c_size_t, ctypes.c_int]
+class device_array:                            # float64, zero
+    def __init__(self, *shape):
+        self.shape, p = shape, ctypes.c_void_p()
+        assert fake.cudaMalloc(ctypes.byref(p), ctypes.c_size_t(8 * int(np.prod(shape)))) == 0
+        self.p = p.value
+    def data_ptr(self):
+        return self.p
 PARAMS = molgen.params_table(molgen.make_params(0))
 def context(device=0):
     h = xs.xs_create(device)

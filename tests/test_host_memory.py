@@ -143,3 +143,44 @@ def test_products_fall_back_to_the_float64_pipe(tmp_path):
     """A float64 product whose work arrays do not fit beside the residue planes runs
     without the planes, as it did before there were any."""
     assert "ran" in fake_cuda.run(tmp_path, SETUP + FALLBACK)
+
+
+FAILED = """
+Zs, xyzs = molgen.make_chain(3, 12, 14)
+h = context()
+xs.xs_ground_state(h, [(Zs, xyzs)])
+n, o, _ = xs.xs_get_sizes(h, 0)
+X, Y = device_array(20, o * (n - o)), device_array(20, o * (n - o))
+lib = xs.load()
+base, failed = fake.fake_used(0), 0
+for room in range(0, 64 << 20, 32 << 10):
+    fake.fake_set_capacity(0, fake.fake_used(0) + room)
+    rc = lib.xs_apply(h, 0, xs.XS_KIND_A, 20, xs._ptr(X), xs._ptr(Y), PRECISION)
+    assert fake.fake_pending() == 0, room
+    if rc == xs.XS_OK:
+        break
+    assert rc == xs.XS_ENOMEM
+    failed += 1
+    xs.xs_destroy(h)
+    fake.fake_set_capacity(0, 1 << 40)
+    h = context()
+    xs.xs_ground_state(h, [(Zs, xyzs)])
+assert failed and rc == xs.XS_OK
+fake.fake_set_capacity(0, 1 << 40)
+# a call that ends in a device error keeps no more than one that succeeds
+L = 2000000
+A, B, C = device_array(70, L), device_array(1, L), device_array(70, 1)
+xs._check(h, lib.xs_subspace_gram(h, 1, 1, 64, xs._ptr(A), xs._ptr(B), xs._ptr(C), 1))
+base = fake.fake_used(0)
+fake.fake_fill(4, 10)                          # the error word: a non-finite value was met
+assert lib.xs_subspace_gram(h, 70, 1, L, xs._ptr(A), xs._ptr(B), xs._ptr(C), 1) == xs.XS_ECUDA
+assert fake.fake_used(0) - base < 1 << 30, (fake.fake_used(0) - base) / (1 << 30)
+print("done")
+"""
+
+
+@pytest.mark.parametrize("precision", [0, 1])
+def test_failed_calls_leave_nothing_behind(tmp_path, precision):
+    """A call that fails half-way returns after its kernels have ended (they read and
+    write the caller's device arrays) and keeps no scratch above the limit."""
+    assert "done" in fake_cuda.run(tmp_path, SETUP + f"PRECISION = {precision}\n" + FAILED)
