@@ -32,7 +32,17 @@
  *     crosses this boundary.
  *   - The caller owns every host array it passes; the library copies what it
  *     needs and owns all device memory it allocates.  Pointers documented as
- *     "host or device" may point to either (unified addressing decides).
+ *     "host or device" may point to either (unified addressing decides);
+ *     xs_apply, xs_subspace_gram and xs_subspace_combine use 16-byte aligned
+ *     device arrays where they are.
+ *   - xs_apply and the xs_subspace calls leave their output arrays as they were
+ *     when they fail (also for a non-finite input), except device arrays used in
+ *     place after XS_ETIMEOUT or a CUDA failure, which may be partly written.
+ *   - A context keeps scratch between calls: staged arrays and digits (at most
+ *     2 GB), residues of float64 products (at most 1.5 GB, more only where a
+ *     single vector needs more) and, per molecule, copies of its orbitals for
+ *     the tensor cores.  xs_ground_state and xs_destroy give it back, and so does
+ *     a call that runs short of memory before it reports XS_ENOMEM.
  *   - One context per host thread; calls on one context are not re-entrant.
  */
 #ifndef XS_H

@@ -862,6 +862,7 @@ int xs_subspace_combine(xs_ctx* ctx, int nb, int S, int nout, long long L, const
         xs::oz_slice(s, S, L, Xb, L, e + b * S, nullptr, 0, 0, nn + (size_t)b * L * ldk, ldk, 0);
         blk[b] = xs::OzBlock{nn + (size_t)b * L * ldk, ldk, e + b * S, dc + (size_t)b * S * nout, nout};
       }
+      xs::oz_check_coefficients(s, nb, blk, S, nout, c.tc_err.get());
       xs::oz_combine(s, nb, blk, S, nout, L, 1.0, 0.0, dY.dev, L, w, c.tc_err.get());
       xs::check_device_error(c);
     } else {

@@ -274,6 +274,8 @@ __global__ void __launch_bounds__(192, 1)
     // epilogue: TMEM lanes 32 (warp % 4) .. + 31
     const int q = warp & 3;
     const int r = 32 * q + lane;
+    // a non-finite value met by an earlier kernel: the caller's output stays as it was
+    const bool skip = a.mode == 1 && *static_cast<volatile int*>(err) != 0;
     int i = 0;
     for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x, ++i) {
       int m0, kb0, nk, kc;
@@ -301,7 +303,7 @@ __global__ void __launch_bounds__(192, 1)
         }
       } else {
         const long long l = static_cast<long long>(m0) + r;
-        for (int k = 0; k < a.ncols; ++k) {
+        for (int k = 0; k < a.ncols && !skip; ++k) {
           float v[8];
           tmem_ld8(trow + k * 8, v);
           unsigned int ym = 0;
@@ -462,7 +464,8 @@ struct CoefArgs {
 // Digit matrix of the combination coefficients, one CTA per output k:
 // column (k, t) of the product (row k * 8 + t here, K-major over the
 // concatenated blocks) holds at K index (b, m, i) the digit t - i of
-// c'[b][m] = coef_b[m][k] 2^(e_b[m]), split with the common exponent f[k].
+// c'[b][m] = coef_b[m][k] 2^(e_b[m]), split with the common exponent f[k].  Without
+// bmat only the error word is raised.
 __global__ void oz_coef_kernel(int nb, int S, int Kp, int k0, CoefArgs ca, double alpha, oz_t* __restrict__ bmat,
                                double* __restrict__ scale, int* err) {
   const int k = blockIdx.x;
@@ -483,6 +486,7 @@ __global__ void oz_coef_kernel(int nb, int S, int Kp, int k0, CoefArgs ca, doubl
   const unsigned long long M = smax;
   const int ex = static_cast<int>((M >> 52) & 0x7FF);
   if (threadIdx.x == 0 && ex == 0x7FF) atomicCAS(err, 0, 11);
+  if (!bmat) return;
   const int f = (M == 0) ? 0 : ex - 1021;
   if (threadIdx.x == 0) {
     // output weights of the anti-diagonal sums split as in horner8
@@ -653,6 +657,18 @@ void oz_gram(cudaStream_t s, int M, int N, long long L, const oz_t* Atn, long lo
                                                                 C + n0, ldc);
     XS_CHECK_LAUNCH();
   }
+}
+
+void oz_check_coefficients(cudaStream_t s, int nb, const OzBlock* blk, int S, int nout, int* err) {
+  if (nout <= kMaxCols) return;   // one launch of oz_coef_kernel precedes every output
+  CoefArgs ca{};
+  for (int b = 0; b < nb; ++b) {
+    ca.coef[b] = blk[b].coef;
+    ca.ldc[b] = blk[b].ldc;
+    ca.e[b] = blk[b].e;
+  }
+  oz_coef_kernel<<<nout, 256, 0, s>>>(nb, S, 0, 0, ca, 1.0, nullptr, nullptr, err);
+  XS_CHECK_LAUNCH();
 }
 
 void oz_combine(cudaStream_t s, int nb, const OzBlock* blk, int S, int nout, long long L, double alpha, double beta,

@@ -79,6 +79,10 @@ struct OzBlock {
 // epilogue (input of oz_exponents_from_max).
 void oz_combine(cudaStream_t s, int nb, const OzBlock* blk, int S, int nout, long long L, double alpha, double beta,
                 double* Y, long long ldy, OzWork& w, int* err, unsigned int* rowmax = nullptr);
+// With the error word already raised oz_combine leaves Y alone.  It raises the word
+// itself for a non-finite coefficient, but goes through many outputs in groups: this
+// raises it ahead of the first.
+void oz_check_coefficients(cudaStream_t s, int nb, const OzBlock* blk, int S, int nout, int* err);
 
 // Column capacity of the nn layout for up to S rows (whole 64-column blocks).
 inline int oz_ldk(int S) { return ((S * kOzDigits + 63) / 64) * 64; }
