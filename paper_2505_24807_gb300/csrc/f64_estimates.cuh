@@ -38,17 +38,22 @@ __device__ __forceinline__ float rsqrt_estimate(float x) {
   return r;
 }
 
-// reciprocal to ~1e-14 relative: a float32 estimate refined by one Newton
-// step (inverse iteration needs directions, not correctly rounded quotients)
+// The corrections are binomial series (Householder's iterations of the first and second
+// order) in the residual e of a float32 estimate r, |e| <= 2^-19:
+//   1 / x = r / (1 - e),           e = 1 - x r:     r (1 + e + e^2 + ...)
+//   1 / sqrt(x) = r (1 - e)^-1/2,  e = 1 - x r^2:   r (1 + e / 2 + 3 e^2 / 8 + ...)
+//   sqrt(x) = x r (1 - e)^-1/2
+
+// reciprocal to 2^-45 relative (seen), the first order (inverse iteration needs
+// directions, not correctly rounded quotients)
 __device__ __forceinline__ double rcp_fast(double x) {
   if (!float_range(x)) return 1.0 / x;
   const double r = widen_bits(rcp_estimate(narrow_bits(x)));
   return r * fma(-x, r, 2.0);
 }
 
-// square root, its reciprocal and the reciprocal to rounding (x > 0 for the
-// roots): float32 estimates with one third-order correction each, whose
-// remainder is 2^-66 relative
+// square root, its reciprocal and the reciprocal (x > 0 for the roots), the second
+// order: the terms left out are e^3 (below 2^-57), 2 ulp with the roundings (1 seen)
 __device__ __forceinline__ double sqrt_fast(double x) {
   if (!float_range(x)) return sqrt(x);
   const double r = widen_bits(rsqrt_estimate(narrow_bits(x)));
