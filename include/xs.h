@@ -69,8 +69,18 @@ extern "C" {
 #define XS_CIS 0
 #define XS_TDHF 1
 
-#define XS_FP64 0   /* every step in float64 */
-#define XS_MIXED 1  /* split-precision tensor-core transforms, float32 G build, float64 subspace */
+/* XS_FP64: every step in float64.  The transforms of molecules of 160 to 8192 AOs (96 for
+ * large batches) are products of 57-bit integers on the tensor cores, accurate to
+ * about 2^-57.8 of the norms of the two rows that meet in an output, which a
+ * float64 sum of as many terms is not; but an output in which only entries far
+ * below those norms meet (amplitudes over many decades) is accurate to the norms
+ * and not to its own size.
+ * XS_MIXED: split-precision tensor-core transforms, float32 G build, float64
+ * subspace.  From 512 AOs up the transforms' operands are float16 pairs with one
+ * exponent per vector and stage: 22 bits down to 2^-17 of the largest entry (or of
+ * the bound of it that sets the exponent), to 2^-40 of it below. */
+#define XS_FP64 0
+#define XS_MIXED 1
 
 #define XS_KIND_A 0    /* A X          (CIS)  */
 #define XS_KIND_APB 1  /* (A + B) X    (TDHF) */

@@ -12,12 +12,16 @@
 // of two of them sum exactly in a float32 accumulator (2^8 2^16 = 2^24).  13
 // bfloat16 products replace one on the float64 pipe (1.2 TFLOP/s measured).
 //
-// The error is 2^-57.8 |a| |b| per element (two roundings of 57-bit integers
-// with unit norms), against about 2^-54 |a| |b| of a K-term float64
-// accumulation; the result is rounded once to float64.  Products A X of the
-// response matrices against a float64 evaluation elsewhere, relative to the part
-// that the transforms form: 2200 AOs 2.33e-15 (float64 pipe 2.91e-15), 579 AOs
-// 1.33e-15 (1.55e-15), 222 AOs 8.3e-16 (1.0e-15).
+// The error is relative to the rows' norms: every entry of a row is rounded to
+// 2^-58 of a power of two at most 2.01 times its norm, so an output is off by at most
+// 2^-57 (|a| sum|b_k| + |b| sum|a_k|) before its one rounding to float64, about 2^-57.8 |a| |b|
+// with entries of random signs, against about 2^-54 |a| |b| of a K-term float64
+// accumulation.  An entry 2^-k of its row's norm keeps 57 - k bits, and an output in
+// which only small entries meet (graded rows, distant fragments) is not accurate to
+// its own size, as a float64 GEMM's would be.  Products A X of the response matrices
+// against a float64 evaluation elsewhere, relative to the part that the transforms
+// form: 2200 AOs 2.33e-15 (float64 pipe 2.91e-15), 579 AOs 1.33e-15 (1.55e-15),
+// 222 AOs 8.3e-16 (1.0e-15).
 #pragma once
 
 #include <cuda_runtime.h>
@@ -29,7 +33,10 @@
 namespace xs {
 
 constexpr int kModuli = 13;
-constexpr int kMgMaxK = 8192;      // largest K: the int32 sums of chunk sums stay below 2^30
+// largest K: mg_split_rows stages a row of K float64 in shared memory, 64 KB of the
+// 227 KB a CTA may have, so that three CTAs share an SM.  (The sums of a product's
+// chunks, 32 of them below 2^8 at this K, would stay exact in float32 to K = 2^23.)
+constexpr int kMgMaxK = 8192;
 using mg_t = uint16_t;             // bfloat16 bit pattern of one residue
 
 // K-major operand of a product: `batch` matrices (1: shared by the batch) of

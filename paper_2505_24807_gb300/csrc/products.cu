@@ -74,6 +74,8 @@ constexpr double kMgBytes = 1.5e9;
 // 116 -> 128, 16 vectors (108 MFLOP) 170 -> 158; 178 AOs, 1 vector 118 -> 122,
 // 4 vectors 131 -> 127; 222 AOs, 1 vector 133 -> 123; 579 AOs, 20 vectors
 // 9932 -> 807 us.
+// Above kMgMaxK AOs a row does not fit the split kernel's share of shared memory and the
+// float64 pipe serves the products, as it did all before.
 bool mg_applies(const DevMol& m, int nvec) {
   const double n = m.n, o = m.o, v = m.v;
   if (m.v > m.o || m.n < 96 || m.n > kMgMaxK) return false;

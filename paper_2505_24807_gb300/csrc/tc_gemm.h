@@ -10,9 +10,10 @@ namespace xs {
 // and base), batch entries bstride apart when batched.  Kpad is a multiple of 32
 // and the padding columns are zero.  T = float: TF32 pairs.  T = __half: float16
 // pairs of x 2^-e, with one exponent e per batch entry (one for the operand when
-// it is not batched) that puts the entry's largest |x| just below 2^15: the same
-// two 11-bit significands as a TF32 pair, and what float16's exponent range cuts
-// off lies 2^-40 below the largest entry.
+// it is not batched) that puts the entry's largest |x|, or a bound of it, just below
+// 2^15.  Down to 2^-17 of that a value has the two 11-bit significands of a TF32 pair;
+// below, the low half meets float16's smallest step, 2^-25 absolute, 2^-40 of the
+// largest: smaller values keep fewer bits than a TF32 pair's 22 and end there.
 template <typename T>
 struct TcPair {
   const T* hi;
