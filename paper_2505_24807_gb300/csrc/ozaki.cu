@@ -160,6 +160,8 @@ __global__ void __launch_bounds__(192, 1)
   using C = OzCfg<BN>;
   extern __shared__ uint8_t smem_raw[];
   __shared__ unsigned int kmax[32];   // mode 1 with rowmax: this CTA's per-output maxima
+  __shared__ int tiles;               // mode 1: none once an earlier kernel has met a non-finite value, so that
+                                      // the caller's output stays as it was
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) & ~uintptr_t(1023));
   uint64_t* full = reinterpret_cast<uint64_t*>(base + C::STAGES * C::STAGE);
   uint64_t* empty = full + C::STAGES;
@@ -183,6 +185,7 @@ __global__ void __launch_bounds__(192, 1)
   };
 
   if (threadIdx.x == 0) {
+    const int raised = a.mode == 1 ? *static_cast<volatile int*>(err) : 0;
     for (int s = 0; s < C::STAGES; ++s) {
       mbar_init(&full[s], 1);
       mbar_init(&empty[s], 1);
@@ -191,6 +194,7 @@ __global__ void __launch_bounds__(192, 1)
       mbar_init(&accf[b], 1);
       mbar_init(&acce[b], 128);
     }
+    tiles = raised ? 0 : a.ntiles;
     asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
   }
   if (warp == 1) tmem_alloc(tmem_slot, C::NBUF * C::TCOLS);
@@ -199,12 +203,13 @@ __global__ void __launch_bounds__(192, 1)
   __syncthreads();
   fence_after_sync();
   const uint32_t tmem = *tmem_slot;
+  const int ntiles = tiles;
 
   if (warp == 0 && lane == 0) {
     // TMA producer
     long long g = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x) {
+    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
       int m0, kb0, nk, kc;
       tile_of(t, m0, kb0, nk, kc);
       for (int it = 0; it < nk; ++it, ++g) {
@@ -243,7 +248,7 @@ __global__ void __launch_bounds__(192, 1)
     long long g = 0;
     int i = 0;
     bool ok = true;
-    for (int t = blockIdx.x; t < a.ntiles && ok; t += gridDim.x, ++i) {
+    for (int t = blockIdx.x; t < ntiles && ok; t += gridDim.x, ++i) {
       int m0, kb0, nk, kc;
       tile_of(t, m0, kb0, nk, kc);
       const int buf = i % C::NBUF, use = i / C::NBUF;
@@ -274,10 +279,8 @@ __global__ void __launch_bounds__(192, 1)
     // epilogue: TMEM lanes 32 (warp % 4) .. + 31
     const int q = warp & 3;
     const int r = 32 * q + lane;
-    // a non-finite value met by an earlier kernel: the caller's output stays as it was
-    const bool skip = a.mode == 1 && *static_cast<volatile int*>(err) != 0;
     int i = 0;
-    for (int t = blockIdx.x; t < a.ntiles; t += gridDim.x, ++i) {
+    for (int t = blockIdx.x; t < ntiles; t += gridDim.x, ++i) {
       int m0, kb0, nk, kc;
       tile_of(t, m0, kb0, nk, kc);
       const int buf = i % C::NBUF;
@@ -303,7 +306,7 @@ __global__ void __launch_bounds__(192, 1)
         }
       } else {
         const long long l = static_cast<long long>(m0) + r;
-        for (int k = 0; k < a.ncols && !skip; ++k) {
+        for (int k = 0; k < a.ncols; ++k) {
           float v[8];
           tmem_ld8(trow + k * 8, v);
           unsigned int ym = 0;
