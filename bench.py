@@ -64,7 +64,9 @@ FP32_SIMT_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 # dram__bytes_write.sum, mean over the captured launches of one solve of the
 # workload), from the ncu summaries named in "source"; a kernel absent here
 # (or changed since its capture) reports traffic null.
-TRAFFIC = {}
+TRAFFIC = {(name, "large"): dict(bytes_per_launch=b, source="profiles/dram_large_tdhf.md")
+           for name, b in dict(oz_combine=2.812e9, oz_gram=1.549e9, oz_slice=5.19e8, tc_gemm_f16x3=2.783e8,
+                               gbuild_assemble_f32=8.91e8).items()}
 
 
 def traffic_of(name, workload):

@@ -315,10 +315,10 @@ int xs_subspace_combine(xs_ctx* ctx, int nb, int S, int nout, long long L, const
  * the k lowest eigenpairs of the symmetric S x S float64 matrix A (row-major,
  * 1 <= k <= S <= 1024), eigenvalues ascending in w (k entries), eigenvectors
  * in the columns of Z (S x k, row-major: Z[i * k + t]).  Householder
- * tridiagonalisation, float32 Sturm multisection, float64 inverse iteration
- * (clusters of close eigenvalues orthogonalised as they are found), one CTA.
- * Host or device pointers owned by the caller; synchronous.  XS_EINVAL for bad
- * sizes. */
+ * tridiagonalisation, float32 Sturm multisection, inverse iteration (float32
+ * solves finished by float64 ones; clusters of close eigenvalues in float64,
+ * orthogonalised as they are found), one CTA.  Host or device pointers owned by
+ * the caller; synchronous.  XS_EINVAL for bad sizes. */
 int xs_subspace_eig(xs_ctx* ctx, int S, int k, const double* A, double* w, double* Z);
 
 /* Parameter derivatives of a CIS or TDHF excitation energy (paper, Section

@@ -18,10 +18,11 @@
 // with entries of random signs, against about 2^-54 |a| |b| of a K-term float64
 // accumulation.  An entry 2^-k of its row's norm keeps 57 - k bits, and an output in
 // which only small entries meet (graded rows, distant fragments) is not accurate to
-// its own size, as a float64 GEMM's would be.  Products A X of the response matrices
-// against a float64 evaluation elsewhere, relative to the part that the transforms
-// form: 2200 AOs 2.33e-15 (float64 pipe 2.91e-15), 579 AOs 1.33e-15 (1.55e-15),
-// 222 AOs 8.3e-16 (1.0e-15).
+// its own size, as a float64 GEMM's would be.  Products A X and (A + B) X of 4 response
+// vectors against a float64 evaluation elsewhere, root mean square of the difference
+// over that of the part that the transforms form: 2200 AOs 2.3e-15 and 2.6e-15 (float64
+// pipe 2.9e-15 and 3.2e-15), 579 AOs 1.3e-15 and 1.6e-15 (1.6e-15, 1.8e-15), 222 AOs
+// 8.3e-16 and 9.7e-16 (9.9e-16, 1.1e-15).
 #pragma once
 
 #include <cuda_runtime.h>

@@ -3,7 +3,8 @@ the public API, sized for profiling one or a few launches (Nsight Compute
 captures of the full workload would hold ~12 GB on the device):
 
   python -m paper_2505_24807_gb300.kernel_cases oz      # digit-product kernel: combination, then Gram
-  python -m paper_2505_24807_gb300.kernel_cases tc      # TF32 transforms: one TDHF product, large molecule
+  python -m paper_2505_24807_gb300.kernel_cases tc      # float16-pair transforms: one TDHF product, large molecule
+  python -m paper_2505_24807_gb300.kernel_cases fp64    # residue products: one float64 TDHF product, large molecule
   python -m paper_2505_24807_gb300.kernel_cases gbuild  # G build: one TDHF product, medium molecule
   python -m paper_2505_24807_gb300.kernel_cases slice   # digit split of 3 x 20 vectors of 600k amplitudes
   python -m paper_2505_24807_gb300.kernel_cases batch   # one lock-step batched CIS solve, 256 molecules of 20-200 atoms
@@ -39,14 +40,14 @@ def case_oz():
     return float(np.abs(Y).max()), float(np.abs(C).max())
 
 
-def _product_case(gen, nvec):
+def _product_case(gen, nvec, precision=xs.XS_MIXED):
     ctx = xs.xs_create(0)
     xs.xs_set_params(ctx, molgen.params_table(molgen.make_params(0)))
     Z, xyz = gen(0)
     xs.xs_ground_state(ctx, [(Z, xyz)])
     n, o, _ = xs.xs_get_sizes(ctx, 0)
     X = np.random.default_rng(1).standard_normal((nvec, o * (n - o)))
-    Y = xs.xs_apply(ctx, 0, xs.XS_KIND_APB, X, precision=xs.XS_MIXED)
+    Y = xs.xs_apply(ctx, 0, xs.XS_KIND_APB, X, precision=precision)
     return (float(np.abs(Y).max()),)
 
 
@@ -70,6 +71,7 @@ def case_batch():
 CASES = {
     "oz": case_oz,
     "tc": lambda: _product_case(molgen.config_large, 10),
+    "fp64": lambda: _product_case(molgen.config_large, 4, xs.XS_FP64),
     "gbuild": lambda: _product_case(molgen.config_medium, 8),
     "slice": case_slice,
     "batch": case_batch,
