@@ -1698,7 +1698,7 @@ void solve_group(Ctx& c, BatchWork& bw, const xs_ex_opts& opt, int first, int co
     d.dip = triplet ? nullptr : m.dip.get();
     d.CT = sizeof(T) == 4 ? static_cast<const void*>(m.CTf.get()) : static_cast<const void*>(m.CT.get());
     d.W = sizeof(T) == 4 ? static_cast<const void*>(m.Wf.get()) : static_cast<const void*>(m.W.get());
-    m.nroots = d.kk;
+    m.nroots = 0;   // until the batch is through
     m.method = opt.method;
     m.spin = opt.spin;
     m.U.alloc((size_t)d.kk * ov);
@@ -1825,6 +1825,7 @@ void solve_group(Ctx& c, BatchWork& bw, const xs_ex_opts& opt, int first, int co
     ss.learned = learned;
     ss.fallback = sq[F_NOSHIFT] != 0;
     const double* r = res.data() + (size_t)q * ldo;
+    m.nroots = d.kk;
     m.omega.assign(r, r + d.kk);
     m.resid.assign(r + d.kk, r + 2 * d.kk);
     m.osc.assign(r + 2 * d.kk, r + 3 * d.kk);

@@ -312,16 +312,17 @@ void mo_dipoles(Ctx& c, DevMol& m) {
   cudaStream_t s = c.stream;
   const int n = m.n, o = m.o, v = m.v;
   const long long ov = (long long)o * v;
-  m.dip.alloc((size_t)3 * ov);
+  DevBuf<double> dip((size_t)3 * ov);   // the molecule gets it when it is complete
   c.ws4.ensure((size_t)v * n);
   for (int x = 0; x < 3; ++x) {
     dipole_rc_kernel<<<grid1((long long)v * n, 256), 256, 0, s>>>(n, o, v, x, m.ao_atom.get(), m.ao_local.get(),
                                                                 m.atom_elem.get(), m.xyz.get(), c.d_par.get(),
                                                                 m.CT.get(), c.ws4.get());
     XS_CHECK_LAUNCH();
-    gemm<double>(s, false, true, o, v, n, 1.0, m.CT.get(), n, 0, c.ws4.get(), n, 0, 0.0, m.dip.get() + (size_t)x * ov, v,
+    gemm<double>(s, false, true, o, v, n, 1.0, m.CT.get(), n, 0, c.ws4.get(), n, 0, 0.0, dip.get() + (size_t)x * ov, v,
                  0, 1);
   }
+  m.dip = std::move(dip);
 }
 
 void oscillator_strengths(Ctx& c, DevMol& m, int kk, const double* U, const double* omega_dev, double* f_dev) {
@@ -871,7 +872,7 @@ int davidson(Ctx& c, DevMol& m, const xs_ex_opts& opt, SolveStats& st) {
   if (status != XS_OK) return status;
 
   // keep the roots: U = X+Y (CIS: X), W = X-Y (CIS: X)
-  m.nroots = kk;
+  m.nroots = 0;   // until all of them are there
   m.method = opt.method;
   m.spin = opt.spin;
   m.U.alloc((size_t)kk * ov);
@@ -887,6 +888,7 @@ int davidson(Ctx& c, DevMol& m, const xs_ex_opts& opt, SolveStats& st) {
     oscillator_strengths(c, m, kk, m.U.get(), w.omega.get(), w.fdev.get());
     sync_copy(s, m.osc.data(), w.fdev.get(), sizeof(double) * kk);
   }
+  m.nroots = kk;
   m.iterations = st.iterations;
   st.converged = converged;
   return converged ? XS_OK : XS_ENOCONV;

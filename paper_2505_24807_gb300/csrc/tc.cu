@@ -61,21 +61,25 @@ void products_half(Ctx& c, DevMol& m, int method, int nvec, const double* X, dou
     absmax_f64(s, (long long)m.np * m.np, m.W.get(), 0, 1, m.w_max.get());
   }
   if (!m.CTh_hi.get()) {
-    // orbital operands, cached until the orbitals change (as in products_mixed), one exponent
+    // orbital operands, cached until the orbitals change (as in products_mixed), one exponent;
+    // the molecule gets them when they are complete
+    const size_t orb = s_vir + s_occ + s_virT + s_occT;
     DevBuf<unsigned int> amax(1);
+    DevBuf<int> ce(1);
+    DevBuf<__half> ch(orb), cl(orb);
     XS_CUDA(cudaMemsetAsync(amax.get(), 0, sizeof(unsigned int), s));
-    m.CTh_e.alloc(1);
-    m.CTh_hi.alloc(s_vir + s_occ + s_virT + s_occT);
-    m.CTh_lo.alloc(s_vir + s_occ + s_virT + s_occT);
     const double* CT = m.CT.get();
     absmax_f64(s, nn, CT, 0, 1, amax.get());
-    __half* h = m.CTh_hi.get();
-    __half* l = m.CTh_lo.get();
-    int* e = m.CTh_e.get();
+    __half* h = ch.get();
+    __half* l = cl.get();
+    int* e = ce.get();
     split16(s, n, v, vp, CT + (size_t)o * n, n, 0, 0, 1, true, amax.get(), e, h, l);
     split16(s, n, o, op, CT, n, 0, 0, 1, true, amax.get(), e, h + s_vir, l + s_vir);
     split16(s, v, n, np_, CT + (size_t)o * n, n, 0, 0, 1, false, amax.get(), e, h + s_vir + s_occ, l + s_vir + s_occ);
     split16(s, o, n, np_, CT, n, 0, 0, 1, false, amax.get(), e, h + s_vir + s_occ + s_virT, l + s_vir + s_occ + s_virT);
+    m.CTh_e = std::move(ce);
+    m.CTh_lo = std::move(cl);
+    m.CTh_hi = std::move(ch);
   }
   const __half* ch = m.CTh_hi.get();
   const __half* cl = m.CTh_lo.get();
@@ -181,10 +185,9 @@ void products_mixed(Ctx& c, DevMol& m, int method, int nvec, const double* X, do
   //   CTvir (v x np) = CT[o + a][mu], CTocc (o x np) = CT[i][mu]
   const size_t orb = (size_t)n * vp + (size_t)n * op + (size_t)v * np_ + (size_t)o * np_;
   if (!m.CTf_hi.get()) {
-    m.CTf_hi.alloc(orb);
-    m.CTf_lo.alloc(orb);
-    float* h = m.CTf_hi.get();
-    float* l = m.CTf_lo.get();
+    DevBuf<float> hi(orb), lo(orb);   // the molecule gets them when they are complete
+    float* h = hi.get();
+    float* l = lo.get();
     const double* CT = m.CT.get();
     split_pad<double>(s, n, v, vp, CT + (size_t)o * n, n, 0, 0, 1, true, h, l);
     h += (size_t)n * vp; l += (size_t)n * vp;
@@ -193,6 +196,8 @@ void products_mixed(Ctx& c, DevMol& m, int method, int nvec, const double* X, do
     split_pad<double>(s, v, n, np_, CT + (size_t)o * n, n, 0, 0, 1, false, h, l);
     h += (size_t)v * np_; l += (size_t)v * np_;
     split_pad<double>(s, o, n, np_, CT, n, 0, 0, 1, false, h, l);
+    m.CTf_lo = std::move(lo);
+    m.CTf_hi = std::move(hi);
   }
   const float* Cvir_h = m.CTf_hi.get();
   const float* Cvir_l = m.CTf_lo.get();

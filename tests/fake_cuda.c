@@ -22,6 +22,9 @@ static size_t capacity[2] = {(size_t)1 << 40, (size_t)1 << 40}, used[2], peak[2]
 static struct { const void* f; size_t n[2]; } attrs[MAX_ATTR];
 static int nattrs;
 static long long pending;   /* launches since the device was last waited for */
+static long long fail_after = -1, fail_times;
+static struct { const void* f; const char* name; long long n; } kernels[MAX_ATTR];
+static int nkernels;
 static __thread int cur;
 static __thread cudaError_t last;
 static __thread struct { dim3 g, b; size_t smem; void* s; } conf;
@@ -32,6 +35,15 @@ size_t fake_used(int dev) { return used[dev]; }
 size_t fake_peak(int dev) { return peak[dev]; }
 void fake_reset_peak(int dev) { peak[dev] = used[dev]; }
 long long fake_pending(void) { return pending; }
+/* after `after` more allocations the next `times` fail */
+void fake_fail(long long after, long long times) { fail_after = after; fail_times = times; }
+/* launches of the kernels whose names contain `part` */
+long long fake_launched(const char* part) {
+  long long n = 0;
+  for (int i = 0; i < nkernels; ++i)
+    if (strstr(kernels[i].name, part)) n += kernels[i].n;
+  return n;
+}
 /* sets every word of the device blocks of n bytes */
 void fake_fill(size_t n, int word) {
   for (int i = 0; i < nblocks; ++i)
@@ -44,7 +56,10 @@ static cudaError_t fail(cudaError_t e) { return last = e; }
 cudaError_t cudaMalloc(void** p, size_t n) {
   pthread_mutex_lock(&mu);
   cudaError_t e = cudaSuccess;
-  if (nblocks == MAX_BLOCKS || used[cur] + n > capacity[cur]) e = cudaErrorMemoryAllocation;
+  int planned = 0;
+  if (fail_after == 0 && fail_times > 0) { planned = 1; --fail_times; }
+  else if (fail_after > 0) --fail_after;
+  if (planned || nblocks == MAX_BLOCKS || used[cur] + n > capacity[cur]) e = cudaErrorMemoryAllocation;
   else {
     char* q = mmap(NULL, n, PROT_READ | PROT_WRITE, MAP_PRIVATE | MAP_ANONYMOUS | MAP_NORESERVE, -1, 0);
     if (q == MAP_FAILED) e = cudaErrorMemoryAllocation;
@@ -102,7 +117,13 @@ static CUresult address_range(CUdeviceptr* base, size_t* n, CUdeviceptr p) {
   pthread_mutex_unlock(&mu);
   return i < 0 ? CUDA_ERROR_INVALID_VALUE : CUDA_SUCCESS;
 }
-static CUresult encode_tiled(CUtensorMap* m) { (void)m; return CUDA_SUCCESS; }
+static CUresult encode_tiled(CUtensorMap* m, CUtensorMapDataType t, cuuint32_t rank, void* p) {
+  (void)m; (void)t; (void)rank;
+  pthread_mutex_lock(&mu);
+  const int i = find(p);
+  pthread_mutex_unlock(&mu);
+  return i < 0 || blocks[i].dev != cur ? CUDA_ERROR_INVALID_VALUE : CUDA_SUCCESS;
+}
 cudaError_t cudaGetDriverEntryPointByVersion(const char* s, void** f, unsigned v, unsigned long long fl, enum cudaDriverEntryPointQueryResult* q) {
   (void)v; (void)fl;
   *f = !strcmp(s, "cuMemGetAddressRange") ? (void*)address_range : !strcmp(s, "cuTensorMapEncodeTiled") ? (void*)encode_tiled : NULL;
@@ -142,6 +163,8 @@ static cudaError_t launch(const void* f, size_t smem) {
   for (int i = 0; i < nattrs; ++i)
     if (attrs[i].f == f && attrs[i].n[cur] > allowed) allowed = attrs[i].n[cur];
   ++pending;
+  for (int i = 0; i < nkernels; ++i)
+    if (kernels[i].f == f) ++kernels[i].n;
   pthread_mutex_unlock(&mu);
   return smem > allowed ? fail(cudaErrorInvalidValue) : cudaSuccess;
 }
@@ -159,7 +182,8 @@ void** __cudaRegisterFatBinary(void* f) { (void)f; static void* h; return &h; }
 void __cudaRegisterFatBinaryEnd(void** h) { (void)h; }
 void __cudaUnregisterFatBinary(void** h) { (void)h; }
 void __cudaRegisterFunction(void** h, const char* f, char* d, const char* n, int t, void* a, void* b, void* c, void* e, int* w) {
-  (void)h; (void)f; (void)d; (void)n; (void)t; (void)a; (void)b; (void)c; (void)e; (void)w;
+  (void)h; (void)d; (void)t; (void)a; (void)b; (void)c; (void)e; (void)w;
+  if (nkernels < MAX_ATTR) { kernels[nkernels].f = f; kernels[nkernels].name = n; ++nkernels; }
 }
 void __cudaRegisterVar(void** h, char* v, char* d, const char* n, int e, size_t s, int c, int g) {
   (void)h; (void)v; (void)d; (void)n; (void)e; (void)s; (void)c; (void)g;

@@ -16,6 +16,8 @@ fake.fake_used.restype = fake.fake_peak.restype = ctypes.c_size_t
 fake.fake_set_capacity.argtypes = [ctypes.c_int, ctypes.c_size_t]
 fake.fake_pending.restype = ctypes.c_longlong
 fake.fake_fill.argtypes = [ctypes.c_size_t, ctypes.c_int]
+fake.fake_fail.argtypes = [ctypes.c_longlong, ctypes.c_longlong]
+fake.fake_launched.restype = ctypes.c_longlong
 class device_array:                            # float64, zero
     def __init__(self, *shape):
         self.shape, p = shape, ctypes.c_void_p()
