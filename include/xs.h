@@ -38,11 +38,13 @@
  *   - xs_apply and the xs_subspace calls leave their output arrays as they were
  *     when they fail (also for a non-finite input), except device arrays used in
  *     place after XS_ETIMEOUT or a CUDA failure, which may be partly written.
- *   - A context keeps scratch between calls: staged arrays and digits (at most
- *     2 GB), residues of float64 products (at most 1.5 GB, more only where a
- *     single vector needs more) and, per molecule, copies of its orbitals for
- *     the tensor cores.  xs_ground_state and xs_destroy give it back, and so does
- *     a call that runs short of memory before it reports XS_ENOMEM.
+ *   - Beside its solvers' workspaces a context keeps scratch between calls for
+ *     speed alone: staged arrays and digits (at most 2 GB), residues of float64
+ *     products (at most 1.5 GB, more only where a single vector needs more) and,
+ *     per molecule, copies of its orbitals for the tensor cores.  xs_ground_state
+ *     and xs_destroy give it back, and a call that runs out of memory gives back
+ *     the scratch and the residue copies and runs again before it reports
+ *     XS_ENOMEM.
  *   - One context per host thread; calls on one context are not re-entrant.
  */
 #ifndef XS_H
