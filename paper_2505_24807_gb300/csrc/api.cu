@@ -59,11 +59,11 @@ int guarded(xs_ctx* ctx, F&& f, R&& may_retry) {
       if (e.status == XS_ENOMEM) {
         cudaGetLastError();
         const bool held = c.release_kept();
-        if (tried == 0 && held && may_retry()) {
+        if (tried == 0 && held && e.again && may_retry()) {
           tried = 1;
           continue;
         }
-        if (tried < 2 && (c.set_residues(false) || held) && may_retry()) {
+        if (tried < 2 && e.again && (c.set_residues(false) || held) && may_retry()) {
           tried = 2;
           continue;
         }
@@ -431,6 +431,7 @@ int xs_excited(xs_ctx* ctx, const xs_ex_opts* opts, double* omega, double* osc, 
       XS_CUDA(cudaStreamSynchronize(c.stream));
       std::atomic<int> next{0};
       std::vector<std::string> errs(nmol);
+      std::vector<char> again(nmol, 1);
       std::vector<std::thread> th;
       for (int t = 0; t < nw; ++t) {
         th.emplace_back([&, t]() {
@@ -442,6 +443,7 @@ int xs_excited(xs_ctx* ctx, const xs_ex_opts* opts, double* omega, double* osc, 
             } catch (const Error& e) {
               rcs[i] = e.status;
               errs[i] = e.what();
+              again[i] = e.again;
             } catch (const std::exception& e) {
               rcs[i] = XS_ECUDA;
               errs[i] = e.what();
@@ -452,7 +454,7 @@ int xs_excited(xs_ctx* ctx, const xs_ex_opts* opts, double* omega, double* osc, 
       }
       for (auto& x : th) x.join();
       for (int i = 0; i < nmol; ++i)
-        if (!errs[i].empty()) throw Error(rcs[i], "molecule " + std::to_string(i) + ": " + errs[i]);
+        if (!errs[i].empty()) throw Error(rcs[i], "molecule " + std::to_string(i) + ": " + errs[i], again[i]);
     } else {
       for (int i = 0; i < nmol; ++i) {
         molecule(c, i);

@@ -36,7 +36,9 @@ namespace xs {
 // layer catches them, stores the message and returns the status.
 struct Error : std::runtime_error {
   int status;
-  Error(int s, const std::string& m) : std::runtime_error(m), status(s) {}
+  bool again;   // XS_ENOMEM: more free memory could help
+  Error(int s, const std::string& m, bool more_memory_helps = true)
+      : std::runtime_error(m), status(s), again(more_memory_helps) {}
 };
 
 #define XS_CUDA(call)                                                                       \

@@ -400,7 +400,8 @@ int davidson(Ctx& c, DevMol& m, const xs_ex_opts& opt, SolveStats& st) {
     if (cap < Smin)
       throw Error(XS_ENOMEM, "subspace needs " + std::to_string(static_cast<long long>(Smin * per_vec)) +
                                  " bytes for its first " + std::to_string(Smin) + " vectors; budget " +
-                                 std::to_string(static_cast<long long>(budget)));
+                                 std::to_string(static_cast<long long>(budget)),
+                  !(opt.memory_limit > 0.0));
     if (cap < Smax) Smax = static_cast<int>(cap);
   }
   st.smax = Smax;

@@ -184,3 +184,31 @@ def test_failed_calls_leave_nothing_behind(tmp_path, precision):
     """A call that fails half-way returns after its kernels have ended (they read and
     write the caller's device arrays) and keeps no scratch above the limit."""
     assert "done" in fake_cuda.run(tmp_path, SETUP + f"PRECISION = {precision}\n" + FAILED)
+
+
+LIMIT = """
+h = context()
+Zs, xyzs = molgen.make_chain(3, 12, 14)
+xs.xs_ground_state(h, [(Zs, xyzs), (Z, xyz)])
+n, o, _ = xs.xs_get_sizes(h, 1)
+def launches():
+    before = fake.fake_launched(b"")
+    try:
+        xs.xs_excited(h, nroots=3, tol=1e-6, max_iter=2, n_mol=2, batched=FORM, memory_limit=16.0 * o * (n - o) * 8)
+        assert False
+    except xs.XSError as e:                    # the second molecule's least subspace is beyond the limit
+        assert e.status == xs.XS_ENOMEM and "subspace needs" in str(e), e
+    return fake.fake_launched(b"") - before
+launches()
+once = launches()
+xs.xs_apply(h, 1, xs.XS_KIND_A, rng.standard_normal((20, o * (n - o))))   # scratch to give back
+assert launches() == once, once
+print("once")
+"""
+
+
+@pytest.mark.parametrize("form", [0, 2])
+def test_memory_limit_is_not_tried_again(tmp_path, form):
+    """A subspace beyond the caller's own limit is refused once: free memory would not
+    help, and the molecules before it are not solved again."""
+    assert "once" in fake_cuda.run(tmp_path, SETUP + f"FORM = {form}\n" + LIMIT)
