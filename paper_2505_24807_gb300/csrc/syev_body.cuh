@@ -94,7 +94,9 @@ __device__ double rayleigh(int n, const double* d, const double* e, const double
 // LU into lu (5 n doubles: 1/pivot, the two super-diagonals of U, the
 // multiplier, the row-swap flag; field f of row i at lu[(f n + i) ldy]) when
 // factor is set, else reusing it; then normalise y unless raw.  Pivots below
-// tiny are raised to tiny.
+// tiny are raised to tiny, and a row is not exchanged for a coupling below it: where
+// the couplings fall off by many decades, exchanges for smaller and smaller ones would
+// grow the vector past every range.
 __device__ void inverse_step(int n, const double* d, const double* e, double shift, double tiny, bool factor,
                              double* lu, double* y, int ldy, bool raw = false) {
   const int fs = n * ldy;
@@ -115,7 +117,7 @@ __device__ void inverse_step(int n, const double* d, const double* e, double shi
       pd = more ? d[i + 2] : 0.0;
       py = more ? y[(i + 2) * ldy] : 0.0;
       double n2 = pe;
-      const bool swp = mag_bits(n0) > mag_bits(c0);
+      const bool swp = mag_bits(n0) > mag_bits(c0) && mag_bits(n0) > mag_bits(tiny);
       const double t0 = c0, t1 = c1, t2 = c2, tr = cur;
       c0 = swp ? n0 : t0; c1 = swp ? n1 : t1; c2 = swp ? n2 : t2; cur = swp ? nr : tr;
       n0 = swp ? t0 : n0; n1 = swp ? t1 : n1; n2 = swp ? t2 : n2; nr = swp ? tr : nr;
@@ -174,7 +176,10 @@ __device__ void inverse_step(int n, const double* d, const double* e, double shi
 
 // Two float32 inverse-iteration solves of (T - shift I) from the start vector in
 // y, one factorisation (fields as in inverse_step); pivots below tiny are raised
-// to it, which also bounds the growth of the unnormalised result.
+// to it.  A solve grows the vector by 1 / |lambda - shift|, which has no lower
+// bound in a graded T (a root coupled to the others by 1e-13 of |T| and a shift that
+// rounds to its diagonal entry: 1e20 and more), so a grown vector is scaled back
+// between the solves; what overflows all the same the caller finds in its norm.
 __device__ void inverse_step_f(int n, const float* d, const float* e, float shift, float tiny, float* lu, float* y,
                                int ldy) {
   const int fs = n * ldy;
@@ -189,7 +194,7 @@ __device__ void inverse_step_f(int n, const float* d, const float* e, float shif
       float c0 = d[0] - shift, c1 = n > 1 ? e[0] : 0.0f, c2 = 0.0f;
       for (int i = 0; i + 1 < n; ++i) {
         float n0 = e[i], n1 = d[i + 1] - shift, n2 = i + 2 < n ? e[i + 1] : 0.0f, nr = y[(i + 1) * ldy];
-        const bool swp = fabsf(n0) > fabsf(c0);
+        const bool swp = fabsf(n0) > fabsf(c0) && fabsf(n0) > tiny;
         const float t0 = c0, t1 = c1, t2 = c2, tr = cur;
         c0 = swp ? n0 : t0; c1 = swp ? n1 : t1; c2 = swp ? n2 : t2; cur = swp ? nr : tr;
         n0 = swp ? t0 : n0; n1 = swp ? t1 : n1; n2 = swp ? t2 : n2; nr = swp ? tr : nr;
@@ -220,13 +225,18 @@ __device__ void inverse_step_f(int n, const float* d, const float* e, float shif
       }
       y[(n - 1) * ldy] = cur;
     }
-    float y1 = 0.0f, y2 = 0.0f;
+    float y1 = 0.0f, y2 = 0.0f, top = 0.0f;
     for (int i = n - 1; i >= 0; --i) {
       const int at = i * ldy;
       const float yi = fmaf(-u1[at], y1, fmaf(-u2[at], y2, y[at])) * rc[at];
       y[at] = yi;
+      top = fmaxf(top, fabsf(yi));
       y2 = y1;
       y1 = yi;
+    }
+    if (pass == 0 && top > 1e12f) {
+      const float down = 1.0f / top;
+      for (int i = 0; i < n; ++i) y[i * ldy] *= down;
     }
   }
 }
@@ -568,7 +578,7 @@ __device__ void syevk_body(int S, int k, const double* __restrict__ Ain, int lda
   //    degenerate pair converge to nearly the same vector, and orthogonalising
   //    them afterwards would magnify their error outside the cluster by the
   //    inverse of the angle between them.
-  const double tiny = 1e-30 * tnorm;
+  const double tiny = 0x1p-56 * tnorm;   // below the rounding of T
   auto orth_against = [&](double* y, int c0, int u) {   // y -= sum_{c0 <= v < u} (z_v . y) z_v, then normalise
     for (int v = c0; v < u; ++v) {
       const double* z = Zw + v;
@@ -602,6 +612,12 @@ __device__ void syevk_body(int S, int k, const double* __restrict__ Ain, int lda
       }
       nn = warp_sum_int(nn);
       rq = warp_sum_int(rq);
+      // a vector that overflowed or vanished: its eigenvalue keeps its shift and is
+      // solved again below, in float64 and normalised after every solve
+      if (!(mag_bits(nn) > 0 && mag_bits(nn) < mag_bits(1e300) && mag_bits(rq) < mag_bits(1e300))) {
+        if (lane == 0) cl[t] = -1 - t;
+        continue;
+      }
       const double inv = rsqrt_full(nn);
       for (int i = lane; i < S; i += 32) y[(long long)i * k] *= inv;
       if (lane == 0) lam[t] = rq * rcp_full(nn);
@@ -634,9 +650,9 @@ __device__ void syevk_body(int S, int k, const double* __restrict__ Ain, int lda
   }
   __syncthreads();
   normalise();
-  // clusters, a thread each
+  // clusters, a thread each, and the vectors given up above
   for (int c0 = tid; c0 < k; c0 += nt) {
-    if (cl[c0] != c0 || isolated(c0)) continue;
+    if (cl[c0] != -1 - c0 && (cl[c0] != c0 || isolated(c0))) continue;
     int c1 = c0 + 1;
     while (c1 < k && cl[c1] == c0) ++c1;
     for (int t = c0; t < c1; ++t) {
