@@ -17,10 +17,12 @@
 //      eigenvector): two float32 solves with the float32 shift, then two
 //      float64 solves shifted by the Rayleigh quotient; the Rayleigh quotient
 //      of the result is the float64 eigenvalue (its error is quadratic in the
-//      vector's).  Shifts closer than 2e-6 |T| form clusters: spread apart,
-//      solved three times in float64 with their own shift, re-orthogonalised
-//      (Gram-Schmidt) and, up to four members, rotated by a Rayleigh-Ritz step
-//      inside the cluster;
+//      vector's).  Eigenvalues closer than 2e-6 |T| form clusters, which take in
+//      what lies within 1e-4 |T| of them: start vectors of their own, two float64
+//      solves with the float32 shift, two shifted by the Rayleigh quotient and one
+//      more with the float32 shift, each followed by Gram-Schmidt against the members
+//      already found and, up to eight members, a Rayleigh-Ritz rotation inside the
+//      cluster;
 //   4. back-transformation z = H_0 H_1 ... H_{S-3} y in blocks of eight
 //      reflectors (compact WY form).
 // Figures are at syevk_body.

@@ -15,7 +15,7 @@ namespace {
 
 constexpr int kSmemMax = 224;   // largest S whose working set fits in shared memory
 constexpr int kSeg = 8;         // row segments of the tridiagonalisation's matrix-vector product
-constexpr int kMaxRR = 4;       // clusters up to this size get a Rayleigh-Ritz rotation
+constexpr int kMaxRR = 8;       // clusters up to this size get a Rayleigh-Ritz rotation
 constexpr int kScaleFree = 12;  // matrices with entries up to 2^+-12 are not scaled
 
 // packed lower triangle: element (i, j), j <= i
@@ -556,17 +556,16 @@ __device__ void syevk_body(int S, int k, const double* __restrict__ Ain, int lda
     if (lane == 0) lam[t] = 0.5 * (static_cast<double>(a0) + static_cast<double>(b0));
   }
   __syncthreads();
-  // clusters: shifts closer than sep are spread apart by sep
-  const double sep = 2e-6 * tnorm;
+  // clusters: eigenvalues closer than the float32 values can tell; a cluster of several
+  // takes in what lies within 1e-4 |T| of it, whose float32 solves would let in too much
+  // of the cluster (at 1e-5 |T|: residuals of 4e-13 |T|)
   if (tid == 0) {
     cl[0] = 0;
+    for (int t = 1; t < k; ++t) cl[t] = lam[t] - lam[t - 1] < 2e-6 * tnorm ? cl[t - 1] : t;
     for (int t = 1; t < k; ++t) {
-      if (lam[t] - lam[t - 1] < sep) {
-        lam[t] = lam[t - 1] + sep;
-        cl[t] = cl[t - 1];
-      } else {
-        cl[t] = t;
-      }
+      if (cl[t] != t || !(lam[t] - lam[t - 1] < 1e-4 * tnorm)) continue;
+      if (cl[t - 1] == t - 1 && (t + 1 == k || cl[t + 1] != t)) continue;   // one beside one
+      for (int u = t; u < k && (u == t || cl[u] == t); ++u) cl[u] = cl[t - 1];
     }
   }
   __syncthreads();
@@ -658,17 +657,31 @@ __device__ void syevk_body(int S, int k, const double* __restrict__ Ain, int lda
     for (int t = c0; t < c1; ++t) {
       double* y = Zw + t;
       double* lut = lu + t;
-      for (int i = 0; i < S; ++i) y[(long long)i * k] = 1.0 + 0.01 * ((i * 7 + t * 3) % 11);
+      // start vectors of their own (a scrambled index): members started alike differ by
+      // little once the earlier ones are taken out, and what is left of other
+      // eigenvectors weighs the more
+      for (int i = 0; i < S; ++i) {
+        unsigned r = static_cast<unsigned>(i) * 2654435761u + static_cast<unsigned>(t + 1) * 2246822519u;
+        r = (r ^ (r >> 15)) * 3266489917u;
+        r ^= r >> 13;
+        y[(long long)i * k] = static_cast<double>(static_cast<int>(r)) * 0x1p-31;
+      }
       inverse_step(S, d, e, lam[t], tiny, true, lut, y, k);
       orth_against(y, c0, t);
       inverse_step(S, d, e, lam[t], tiny, false, lut, y, k);
       orth_against(y, c0, t);
-      // one more solve shifted by the Rayleigh quotient: the spread shift of
-      // a cluster member sits up to (members) x sep from the cluster, which
-      // leaves neighbouring eigenvectors in y at (sep / gap)^2; shifted by the
-      // Rayleigh quotient they fall by a further (spread inside / gap)
-      const double rq = rayleigh(S, d, e, y, k);
-      inverse_step(S, d, e, rq, tiny, true, lut, y, k);
+      // the shift is off by 2e-7 |T|, which leaves neighbouring eigenvectors in y at
+      // its square over the gap's; two solves shifted by the Rayleigh quotient take
+      // that to the third power each
+      for (int pass = 0; pass < 2; ++pass) {
+        const double rq = rayleigh(S, d, e, y, k);
+        inverse_step(S, d, e, rq, tiny, true, lut, y, k);
+        orth_against(y, c0, t);
+      }
+      // that close to a degenerate eigenvalue the members found before grow at rates of
+      // their own, and taking them out magnifies the rounding outside the cluster: the
+      // float32 shift treats them alike
+      inverse_step(S, d, e, lam[t], tiny, true, lut, y, k);
       orth_against(y, c0, t);
     }
     for (int t = c0; t < c1; ++t) lam[t] = rayleigh(S, d, e, Zw + t, k);
